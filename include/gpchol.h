@@ -268,18 +268,23 @@ int gpc_tri_solve_adjoint(int n, int m, const double *Linv, int ldi, const doubl
                           gpc_stream_t stream);
 
 /*
- * General matrix product C = A B (Section 3.1, primitive function) on the FP64
- * tensor path.  A: m x k (lda >= k), B: k x n (ldb >= n), C: m x n (ldc >= n),
+ * General matrix product C = A B (Section 3.1, primitive function) at FP64
+ * accuracy.  A: m x k (lda >= k), B: k x n (ldb >= n), C: m x n (ldc >= n),
  * all row-major device arrays; C must not overlap A or B.  ws/ws_bytes: NULL/0,
- * or at least gpc_gemm_workspace_size() bytes, which lets a product whose
- * output is too small to fill the GPU split its k range over CTAs (the
- * paper's large-k special case; partial products summed in a fixed order).
+ * or at least 40 MiB (gpc_gemm_workspace_size() gives a size for any product,
+ * gpc_gemm_scratch_size() the one of a given product, 0 where none is used).
+ * With a workspace a large product runs on BF16 slices of its operands on the
+ * tensor cores, to at least the accuracy of the FP64 chain (output blocks for
+ * which that cannot be shown are computed in FP64), and a product whose output
+ * is too small to fill the GPU splits its k range over CTAs (the paper's
+ * large-k special case; partial products summed in a fixed order).
  * k == 0 writes C = 0; m == 0 or n == 0 does nothing.  Errors:
  * GPC_ERR_INVALID_ARG for negative sizes, null pointers, short leading
  * dimensions, overlaps or a short non-null workspace (nothing enqueued);
  * GPC_ERR_CUDA on a launch error.
  */
 int gpc_gemm_workspace_size(size_t *bytes);
+int gpc_gemm_scratch_size(int m, int n, int k, size_t *bytes);
 int gpc_gemm(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
              void *ws, size_t ws_bytes, gpc_stream_t stream);
 

@@ -65,6 +65,7 @@ _SIGNATURES = {
     "gpc_trsv_noalloc": ([_c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp], _c_int),
     "gpc_tri_inverse": ([_c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp], _c_int),
     "gpc_gemm_workspace_size": ([ctypes.POINTER(_c_size)], _c_int),
+    "gpc_gemm_scratch_size": ([_c_int, _c_int, _c_int, ctypes.POINTER(_c_size)], _c_int),
     "gpc_gemm": ([_c_int, _c_int, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_size, _c_vp],
                  _c_int),
     "gpc_gemm_adjoint": ([_c_int, _c_int, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int,
@@ -454,13 +455,25 @@ def _rows(t: torch.Tensor, name: str) -> tuple[int, int, int]:
     return r, c, (int(t.stride(0)) if r > 0 and c > 0 else max(c, 1))
 
 
+def _gemm_scratch(device, *shapes) -> torch.Tensor | None:
+    """Slice scratch for products of the given (m, n, k), or None where none of them uses any."""
+    need = 0
+    b = ctypes.c_size_t()
+    for m, n, k in shapes:
+        _check(capi.gpc_gemm_scratch_size(m, n, k, ctypes.byref(b)), "gpc_gemm_scratch_size")
+        need = max(need, b.value)
+    return torch.empty(need, dtype=torch.uint8, device=device) if need else None
+
+
 def gemm(A: torch.Tensor, B: torch.Tensor, out: torch.Tensor | None = None,
          ws: torch.Tensor | None = None) -> torch.Tensor:
-    """C = A B on the FP64 tensor path (ws: optional split-k scratch)."""
+    """C = A B at FP64 accuracy (ws: optional scratch, gemm_workspace; large products allocate their own)."""
     m, k, lda = _rows(A, "A")
     k2, n, ldb = _rows(B, "B")
     if k2 != k:
         raise ValueError("inner dimensions differ")
+    if ws is None:
+        ws = _gemm_scratch(A.device, (m, n, k))
     C = out if out is not None else torch.empty(m, n, dtype=torch.float64, device=A.device)
     _, _, ldc = _rows(C, "C")
     _check(capi.gpc_gemm(m, n, k, _ptr(A), lda, _ptr(B), ldb, _ptr(C), ldc, _ptr(ws),
@@ -476,6 +489,8 @@ def gemm_adjoint(A: torch.Tensor, B: torch.Tensor, Cbar: torch.Tensor,
     _, _, ldcb = _rows(Cbar, "Cbar")
     if tuple(Cbar.shape) != (m, n) or B.shape[0] != k:
         raise ValueError("shape mismatch")
+    if ws is None:
+        ws = _gemm_scratch(A.device, (m, k, n), (k, n, m))
     Abar = torch.empty(m, k, dtype=torch.float64, device=A.device)
     Bbar = torch.empty(k, n, dtype=torch.float64, device=A.device)
     _check(capi.gpc_gemm_adjoint(m, n, k, _ptr(A), lda, _ptr(B), ldb, _ptr(Cbar), ldcb, _ptr(Abar), max(k, 1),

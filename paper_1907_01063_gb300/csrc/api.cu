@@ -36,6 +36,7 @@ struct ApiWs {
 
 constexpr int kRefineMaxIters = 10;
 constexpr double kRefineTol = 1e-14;
+constexpr size_t kGemmWorkspace = size_t(256) << 20;  // gpc_gemm_workspace_size; 40 MB (split-K tiles) is accepted
 
 size_t core_bytes(int n, int precision) {
   size_t c = std::max(chol_workspace_bytes(n, precision), adjoint_workspace_bytes(n, precision));
@@ -253,7 +254,16 @@ int gpc_trsv(int n, const double *L, int ldl, double *x, int trans, void *ws, si
 
 int gpc_gemm_workspace_size(size_t *bytes) {
   if (!bytes) return GPC_ERR_INVALID_ARG;
-  *bytes = gemm_f64_scratch_bytes();
+  *bytes = kGemmWorkspace;
+  return GPC_OK;
+}
+
+int gpc_gemm_scratch_size(int m, int n, int k, size_t *bytes) {
+  if (!bytes || m < 0 || n < 0 || k < 0) return GPC_ERR_INVALID_ARG;
+  Gemm g;
+  g.M = m; g.N = n; g.K = k;
+  *bytes = f64x_worth(g) ? std::max(f64x_scratch_bytes(m, n, k, 1), gemm_f64_scratch_bytes())
+                         : (gemm_f64_splits(g) ? gemm_f64_scratch_bytes() : 0);
   return GPC_OK;
 }
 
@@ -273,7 +283,7 @@ int gpc_gemm(int m, int n, int k, const double *A, int lda, const double *B, int
   g.A = A; g.lda = lda;
   g.B = B; g.ldb = ldb;
   g.C = C; g.ldc = ldc;
-  return status_of(gemm_f64(g, (double *)ws, stream));
+  return status_of(gemm_f64x(g, ws, ws ? ws_bytes : 0, stream));
 }
 
 int gpc_gemm_adjoint(int m, int n, int k, const double *A, int lda, const double *B, int ldb,
@@ -296,7 +306,7 @@ int gpc_gemm_adjoint(int m, int n, int k, const double *A, int lda, const double
     a.A = Cbar; a.lda = ldcb;
     a.transB = true; a.B = B; a.ldb = ldb;
     a.C = Abar; a.ldc = ldab;
-    cudaError_t e = gemm_f64(a, (double *)ws, stream);
+    cudaError_t e = gemm_f64x(a, ws, ws ? ws_bytes : 0, stream);
     if (e != cudaSuccess) return status_of(e);
   }
   if (k > 0 && n > 0) {
@@ -305,7 +315,7 @@ int gpc_gemm_adjoint(int m, int n, int k, const double *A, int lda, const double
     b.transA = true; b.A = A; b.lda = lda;
     b.B = Cbar; b.ldb = ldcb;
     b.C = Bbar; b.ldc = ldbb;
-    cudaError_t e = gemm_f64(b, (double *)ws, stream);
+    cudaError_t e = gemm_f64x(b, ws, ws ? ws_bytes : 0, stream);
     if (e != cudaSuccess) return status_of(e);
   }
   return GPC_OK;

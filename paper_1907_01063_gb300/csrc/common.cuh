@@ -212,9 +212,19 @@ struct Gemm {
   // (never split over K).
   int batch = 1;
   long long sA = 0, sB = 0, sC = 0;
+  // flags != null: only the 32 x 32 output blocks whose flag is zero are
+  // computed (flag of block (r, c) of product b at flags[b flag_stride + r
+  // flag_ld + c]); ksh_m and ksh_n are added to the row and column indices
+  // that kskip compares with k (a panel of a larger product).
+  const unsigned char *flags = nullptr;
+  int flag_ld = 0;
+  long long flag_stride = 0;
+  int ksh_m = 0, ksh_n = 0;
 };
 // Bytes of split-K scratch any gemm_f64 call may use (a fixed cap).
 size_t gemm_f64_scratch_bytes();
+// Whether a product would use split-K scratch.
+bool gemm_f64_splits(const Gemm &g);
 cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t s);
 
 // ---------------------------------------------------------------- diagonal blocks
@@ -338,6 +348,33 @@ cudaError_t lml_lbar(int n, const double *L, long long ldl, const double *alpha,
                      const double *z, double gbar, double *Lbar, long long ldlb, cudaStream_t s, bool df = false);
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+// ---------------------------------------------------------------- FP64-accurate split products (f64x.cu)
+struct SliceBuf;
+constexpr int kF64xSlices = 7;                     // BF16 slices per operand of the factorisation's products
+constexpr size_t kF64xScratchCap = size_t(1) << 30;  // a general product's slices per pass
+// A checked product (8 slices) of K terms loses at most K 2^-62.5 relative to
+// its operands' row scales; the FP64 chain's bound is K 2^-53 S with S = sum
+// |a'||b'| in the same units, so S >= 2^-9.5 suffices.  S is formed from the
+// leading digits, which exceed an entry by at most a factor of two each: 2^-7.
+constexpr float kF64xTheta = 0.0078125f;
+size_t f64x_slice_bytes(int rows, int kchunks);
+// The slices of split_operand, kF64xSlices of them, of the entries scaled by
+// 2^(kexp_sign kexp[k] - rexp[r]) (either may be null).  saturate: scaled
+// entries above 2^30 become 2^30, otherwise (and for NaN) NaN.
+cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,
+                       const int *rexp, const int *kexp, int kexp_sign, bool saturate, cudaStream_t s,
+                       int chunk_offset = 0, int row_offset = 0);
+// C (FP64) -= 2^(ra_i + rb_j) A B^T; the other arguments as for ozaki_gemm.
+cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
+                      int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
+                      double *partial, int *err, cudaStream_t s, int max_ctas = 0, int kdepth = 0, int max_items = 0);
+// gemm_f64 through checked split products where the size pays for the split
+// and ws (f64x_scratch_bytes, or less: more passes) allows; otherwise gemm_f64,
+// with ws as its split-K scratch.
+size_t f64x_scratch_bytes(int M, int N, int K, int batch);
+bool f64x_worth(const Gemm &g);
+cudaError_t gemm_f64x(const Gemm &g, void *ws, size_t ws_bytes, cudaStream_t s);
 
 // ---------------------------------------------------------------- mixed precision (ozaki.cu)
 // BF16 slice planes of an operand, K-major: plane p, row r, K index k at

@@ -38,6 +38,9 @@ struct Params {
   int uplo, tiles_n, kchunk, kskip;
   long long sA, sB, sC;  // per-product offsets of a batch (grid.y)
   double *partial;  // non-null when grid.z > 1
+  const unsigned char *flags;  // Gemm::flags
+  int flag_ld, ksh_m, ksh_n;
+  long long flag_stride;
 };
 
 __device__ __forceinline__ void tri_index(int x, int &ti, int &tj) {
@@ -151,9 +154,19 @@ __global__ void __launch_bounds__(THREADS) gemm_f64_kernel(Params p) {
     tn = blockIdx.x - tm * p.tiles_n;
   }
   const int m0 = tm * T, n0 = tn * T;
-  // a skipped leading K range is a multiple of T, so kbeg stays on a K step
-  const int kfirst = p.kskip == KSKIP_ROWS ? m0 : (p.kskip == KSKIP_COLS ? n0 : 0);
-  const int klast = p.kskip == KSKIP_ROWS_END ? m0 + T : (p.kskip == KSKIP_COLS_END ? n0 + T : p.K);
+  const unsigned char *fl = nullptr;
+  if constexpr (T == 64) {
+    if (p.flags) {  // 2 x 2 blocks of 32, one per warp
+      fl = p.flags + (size_t)blockIdx.y * p.flag_stride + (size_t)(m0 / 32) * p.flag_ld + n0 / 32;
+      // blocks past the output's edge are not flagged
+      const bool r1 = m0 + 32 < p.M, c1 = n0 + 32 < p.N;
+      if (fl[0] && (!c1 || fl[1]) && (!r1 || fl[p.flag_ld]) && (!r1 || !c1 || fl[p.flag_ld + 1])) return;
+    }
+  }
+  // a skipped leading K range is a multiple of 64, so kbeg stays on a K step
+  const int kfirst = p.kskip == KSKIP_ROWS ? m0 + p.ksh_m : (p.kskip == KSKIP_COLS ? n0 + p.ksh_n : 0);
+  const int klast =
+      p.kskip == KSKIP_ROWS_END ? m0 + T + p.ksh_m : (p.kskip == KSKIP_COLS_END ? n0 + T + p.ksh_n : p.K);
   const int kbeg = max((int)blockIdx.z * p.kchunk, kfirst);
   const int kend = min(min(p.K, klast), (int)blockIdx.z * p.kchunk + p.kchunk);
 
@@ -217,6 +230,7 @@ __global__ void __launch_bounds__(THREADS) gemm_f64_kernel(Params p) {
     }
   }
 
+  if (fl && fl[wm * p.flag_ld + wn]) return;
   // Epilogue: fragment (mi, ni) element r sits at row g (+8 for r >= 2),
   // column 2*tg + (r & 1) of the 16 x 8 tile.
   const bool split = p.partial != nullptr;
@@ -250,6 +264,7 @@ __global__ void splitk_reduce_kernel(Params p, int splits) {
   if (idx >= total) return;
   const int row = (int)(idx / p.N), col = (int)(idx - (long long)row * p.N);
   if (p.uplo != UPLO_FULL && col > row) return;
+  if (p.flags && p.flags[(size_t)(row / 32) * p.flag_ld + col / 32]) return;
   double s = 0.0;
   for (int z = 0; z < splits; ++z) s += p.partial[(size_t)z * total + idx];
   double *dst = p.C + (long long)row * p.ldc + col;
@@ -282,6 +297,11 @@ cudaError_t small_tile_carveout() {
 }
 }  // namespace
 
+bool gemm_f64_splits(const Gemm &g) {
+  const long long tiles = (long long)((g.M + 63) / 64) * ((g.N + 63) / 64);
+  return g.M > 0 && g.N > 0 && g.batch == 1 && tiles < 3LL * sm_count() && g.K >= 2 * std::max(tuning().splitk_min, BK);
+}
+
 cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   if (g.uplo != UPLO_FULL && g.M != g.N) return cudaErrorInvalidValue;
@@ -303,6 +323,11 @@ cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t s) {
   p.sA = g.sA;
   p.sB = g.sB;
   p.sC = g.sC;
+  p.flags = g.flags;
+  p.flag_ld = g.flag_ld;
+  p.flag_stride = g.flag_stride;
+  p.ksh_m = g.ksh_m;
+  p.ksh_n = g.ksh_n;
   // 64-wide tiles; a single product that 64-wide tiles and split K cannot
   // spread over every SM takes 32-wide tiles and K steps down to 16 (the
   // symbolic steps of the adjoint, 128 x 128 x 128: 16 CTAs with 64-wide
@@ -320,7 +345,7 @@ cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t s) {
   };
   const int kmin64 = std::max(tuning().splitk_min, BK);
   const int small_max = tuning().f64_small_tile;
-  const bool small = g.batch == 1 && scratch != nullptr && g.M <= small_max && g.N <= small_max &&
+  const bool small = g.batch == 1 && scratch != nullptr && g.flags == nullptr && g.M <= small_max && g.N <= small_max &&
                      tile_count(64) * max_splits(kmin64) < sm_count();
   const int T = small ? 32 : 64;
   p.tiles_n = (g.N + T - 1) / T;
