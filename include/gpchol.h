@@ -268,6 +268,22 @@ int gpc_tri_solve_adjoint(int n, int m, const double *Linv, int ldi, const doubl
                           gpc_stream_t stream);
 
 /*
+ * The three calls above with scratch: ws of gpc_tri_workspace_size(n, m) bytes
+ * (m = 0 for the inverse alone; 0 bytes: none is used) lets their larger
+ * products run on BF16 slices on the tensor cores at FP64 accuracy, as in
+ * gpc_gemm.  A smaller or null ws takes more passes or the FP64 kernel.  ws
+ * must not overlap an output; errors as without it.
+ */
+int gpc_tri_workspace_size(int n, int m, size_t *bytes);
+int gpc_tri_inverse_ws(int n, const double *L, int ldl, double *Linv, int ldi, void *ws, size_t ws_bytes,
+                       gpc_stream_t stream);
+int gpc_tri_solve_ws(int n, int m, const double *L, int ldl, const double *B, int ldb, double *Linv, int ldi,
+                     double *C, int ldc, void *ws, size_t ws_bytes, gpc_stream_t stream);
+int gpc_tri_solve_adjoint_ws(int n, int m, const double *Linv, int ldi, const double *C, int ldc,
+                             const double *Cbar, int ldcb, double *Bbar, int ldbb, double *Lbar, int ldlb, void *ws,
+                             size_t ws_bytes, gpc_stream_t stream);
+
+/*
  * General matrix product C = A B (Section 3.1, primitive function) at FP64
  * accuracy.  A: m x k (lda >= k), B: k x n (ldb >= n), C: m x n (ldc >= n),
  * all row-major device arrays; C must not overlap A or B.  ws/ws_bytes: NULL/0,

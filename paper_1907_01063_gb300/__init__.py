@@ -63,7 +63,9 @@ _SIGNATURES = {
                           _c_vp, _c_size, _c_vp], _c_int),
     "gpc_trsv": ([_c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_size, _c_vp], _c_int),
     "gpc_trsv_noalloc": ([_c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp], _c_int),
+    "gpc_tri_workspace_size": ([_c_int, _c_int, ctypes.POINTER(_c_size)], _c_int),
     "gpc_tri_inverse": ([_c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp], _c_int),
+    "gpc_tri_inverse_ws": ([_c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_size, _c_vp], _c_int),
     "gpc_gemm_workspace_size": ([ctypes.POINTER(_c_size)], _c_int),
     "gpc_gemm_scratch_size": ([_c_int, _c_int, _c_int, ctypes.POINTER(_c_size)], _c_int),
     "gpc_gemm": ([_c_int, _c_int, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_size, _c_vp],
@@ -82,6 +84,10 @@ _SIGNATURES = {
                       _c_int),
     "gpc_tri_solve_adjoint": ([_c_int, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int,
                                _c_vp, _c_int, _c_vp], _c_int),
+    "gpc_tri_solve_adjoint_ws": ([_c_int, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int,
+                               _c_vp, _c_int, _c_vp, _c_size, _c_vp], _c_int),
+    "gpc_tri_solve_ws": ([_c_int, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp, _c_int, _c_vp,
+                          _c_size, _c_vp], _c_int),
     "gpc_gp_lml": ([_c_int, _c_vp, _c_int, _c_vp, _c_vp, _c_int, _c_int, _c_vp, _c_vp, _c_vp,
                     _c_vp, _c_size, _c_vp, _c_vp], _c_int),
     "gpc_gp_lml_grad": ([_c_int, _c_vp, _c_int, _c_vp, _c_double, _c_vp, _c_int, _c_int, _c_vp,
@@ -393,13 +399,21 @@ def _rect(t: torch.Tensor, n: int, name: str) -> tuple[int, int]:
     return m, (int(t.stride(0)) if n > 0 and m > 0 else max(m, 1))
 
 
+def _tri_scratch(n: int, m: int, device) -> tuple[torch.Tensor | None, int]:
+    """Slice scratch of the triangular calls and its bytes (None, 0 where none is used)."""
+    b = ctypes.c_size_t()
+    _check(capi.gpc_tri_workspace_size(n, m, ctypes.byref(b)), "gpc_tri_workspace_size")
+    return (torch.empty(b.value, dtype=torch.uint8, device=device) if b.value else None), b.value
+
+
 def tri_inverse(L: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
     """L^{-1} of the lower triangle of L (zero strict upper); out may be L itself."""
     n = L.shape[0]
     ldl = _square(L, "L")
     X = out if out is not None else torch.empty_like(L)
     ldx = _square(X, "Linv")
-    _check(capi.gpc_tri_inverse(n, _ptr(L), ldl, _ptr(X), ldx, _stream()), "gpc_tri_inverse")
+    ws, nbytes = _tri_scratch(n, 0, L.device)
+    _check(capi.gpc_tri_inverse_ws(n, _ptr(L), ldl, _ptr(X), ldx, _ptr(ws), nbytes, _stream()), "gpc_tri_inverse")
     return X
 
 
@@ -413,7 +427,9 @@ def tri_solve(L: torch.Tensor, B: torch.Tensor, Linv: torch.Tensor | None = None
     ldx = _square(X, "Linv")
     C = out if out is not None else torch.empty(n, m, dtype=torch.float64, device=B.device)
     _, ldc = _rect(C, n, "C")
-    _check(capi.gpc_tri_solve(n, m, _ptr(L), ldl, _ptr(B), ldb, _ptr(X), ldx, _ptr(C), ldc, _stream()),
+    ws, nbytes = _tri_scratch(n, m, L.device)
+    _check(capi.gpc_tri_solve_ws(n, m, _ptr(L), ldl, _ptr(B), ldb, _ptr(X), ldx, _ptr(C), ldc, _ptr(ws), nbytes,
+                                 _stream()),
            "gpc_tri_solve")
     return C, X
 
@@ -432,8 +448,9 @@ def tri_solve_adjoint(Linv: torch.Tensor, C: torch.Tensor, Cbar: torch.Tensor,
     _, ldbb = _rect(Bb, n, "Bbar")
     Lb = Lbar if Lbar is not None else torch.empty_like(Linv)
     ldlb = _square(Lb, "Lbar")
-    _check(capi.gpc_tri_solve_adjoint(n, m, _ptr(Linv), ldx, _ptr(C), ldc, _ptr(Cbar), ldcb, _ptr(Bb), ldbb,
-                                      _ptr(Lb), ldlb, _stream()),
+    ws, nbytes = _tri_scratch(n, m, Linv.device)
+    _check(capi.gpc_tri_solve_adjoint_ws(n, m, _ptr(Linv), ldx, _ptr(C), ldc, _ptr(Cbar), ldcb, _ptr(Bb), ldbb,
+                                         _ptr(Lb), ldlb, _ptr(ws), nbytes, _stream()),
            "gpc_tri_solve_adjoint")
     return Bb, Lb
 

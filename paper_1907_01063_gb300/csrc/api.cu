@@ -371,16 +371,28 @@ int gpc_glm_categorical(long long n, int k, int C, const double *X, long long ld
   return status_of(glm_categorical(n, k, C, X, ldx, y, alpha, beta, lp, dalpha, dbeta, ws, stream));
 }
 
-int gpc_tri_inverse(int n, const double *L, int ldl, double *Linv, int ldi, gpc_stream_t stream) {
+int gpc_tri_workspace_size(int n, int m, size_t *bytes) {
+  if (!bytes || n < 0 || m < 0) return GPC_ERR_INVALID_ARG;
+  *bytes = tri_workspace_bytes(n, m);
+  return GPC_OK;
+}
+
+int gpc_tri_inverse_ws(int n, const double *L, int ldl, double *Linv, int ldi, void *ws, size_t ws_bytes,
+                       gpc_stream_t stream) {
   if (n < 0) return GPC_ERR_INVALID_ARG;
   if (n == 0) return GPC_OK;
   if (bad_square(n, L, ldl) || bad_square(n, Linv, ldi) || bad_inverse_pair(n, L, ldl, Linv, ldi))
     return GPC_ERR_INVALID_ARG;
-  return status_of(tri_inverse(n, L, ldl, Linv, ldi, stream));
+  if (ws && overlaps(ws, ws_bytes, Linv, mat_bytes(n, ldi))) return GPC_ERR_INVALID_ARG;
+  return status_of(tri_inverse(n, L, ldl, Linv, ldi, ws, ws ? ws_bytes : 0, stream));
 }
 
-int gpc_tri_solve(int n, int m, const double *L, int ldl, const double *B, int ldb, double *Linv, int ldi,
-                  double *C, int ldc, gpc_stream_t stream) {
+int gpc_tri_inverse(int n, const double *L, int ldl, double *Linv, int ldi, gpc_stream_t stream) {
+  return gpc_tri_inverse_ws(n, L, ldl, Linv, ldi, nullptr, 0, stream);
+}
+
+int gpc_tri_solve_ws(int n, int m, const double *L, int ldl, const double *B, int ldb, double *Linv, int ldi,
+                     double *C, int ldc, void *ws, size_t ws_bytes, gpc_stream_t stream) {
   if (n < 0 || m < 0) return GPC_ERR_INVALID_ARG;
   if (n == 0) return GPC_OK;
   if (bad_square(n, L, ldl) || bad_square(n, Linv, ldi) || bad_inverse_pair(n, L, ldl, Linv, ldi) ||
@@ -392,12 +404,19 @@ int gpc_tri_solve(int n, int m, const double *L, int ldl, const double *B, int l
         overlaps(B, bb, Linv, mat_bytes(n, ldi)))
       return GPC_ERR_INVALID_ARG;
   }
-  return status_of(tri_solve(n, m, L, ldl, B, ldb, Linv, ldi, C, ldc, stream));
+  if (ws && (overlaps(ws, ws_bytes, Linv, mat_bytes(n, ldi)) || overlaps(ws, ws_bytes, C, rect_bytes(n, m, ldc))))
+    return GPC_ERR_INVALID_ARG;
+  return status_of(tri_solve(n, m, L, ldl, B, ldb, Linv, ldi, C, ldc, ws, ws ? ws_bytes : 0, stream));
 }
 
-int gpc_tri_solve_adjoint(int n, int m, const double *Linv, int ldi, const double *C, int ldc,
-                          const double *Cbar, int ldcb, double *Bbar, int ldbb, double *Lbar, int ldlb,
-                          gpc_stream_t stream) {
+int gpc_tri_solve(int n, int m, const double *L, int ldl, const double *B, int ldb, double *Linv, int ldi,
+                  double *C, int ldc, gpc_stream_t stream) {
+  return gpc_tri_solve_ws(n, m, L, ldl, B, ldb, Linv, ldi, C, ldc, nullptr, 0, stream);
+}
+
+int gpc_tri_solve_adjoint_ws(int n, int m, const double *Linv, int ldi, const double *C, int ldc,
+                             const double *Cbar, int ldcb, double *Bbar, int ldbb, double *Lbar, int ldlb, void *ws,
+                             size_t ws_bytes, gpc_stream_t stream) {
   if (n < 0 || m < 0) return GPC_ERR_INVALID_ARG;
   if (n == 0) return GPC_OK;
   if (bad_square(n, Linv, ldi) || bad_square(n, Lbar, ldlb) || bad_rect(n, m, C, ldc) ||
@@ -409,7 +428,15 @@ int gpc_tri_solve_adjoint(int n, int m, const double *Linv, int ldi, const doubl
       overlaps(Lbar, lb, Bbar, bbb) || overlaps(Bbar, bbb, Linv, xb) || overlaps(Bbar, bbb, C, cb) ||
       overlaps(Bbar, bbb, Cbar, cbb))
     return GPC_ERR_INVALID_ARG;
-  return status_of(tri_solve_adjoint(n, m, Linv, ldi, C, ldc, Cbar, ldcb, Bbar, ldbb, Lbar, ldlb, stream));
+  if (ws && (overlaps(ws, ws_bytes, Lbar, lb) || overlaps(ws, ws_bytes, Bbar, bbb))) return GPC_ERR_INVALID_ARG;
+  return status_of(tri_solve_adjoint(n, m, Linv, ldi, C, ldc, Cbar, ldcb, Bbar, ldbb, Lbar, ldlb, ws,
+                                     ws ? ws_bytes : 0, stream));
+}
+
+int gpc_tri_solve_adjoint(int n, int m, const double *Linv, int ldi, const double *C, int ldc,
+                          const double *Cbar, int ldcb, double *Bbar, int ldbb, double *Lbar, int ldlb,
+                          gpc_stream_t stream) {
+  return gpc_tri_solve_adjoint_ws(n, m, Linv, ldi, C, ldc, Cbar, ldcb, Bbar, ldbb, Lbar, ldlb, nullptr, 0, stream);
 }
 
 int gpc_gp_lml(int n, const double *K, int ldk, const double *y, double *L, int ldl,

@@ -229,12 +229,8 @@ cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t s);
 
 // ---------------------------------------------------------------- diagonal blocks
 constexpr int kMaxBlock = 128;
-// Factor the nb x nb lower block at A (in place, upper part of the block set
-// to zero) and write its inverse (lower, ld = nb) to Winv.  On a failing
-// pivot p records {pivot_offset + p, status} in info if info[1] is still 0.
-cudaError_t potrf_trtri_diag(int nb, double *A, long long lda, double *Winv, int *info,
-                             int pivot_offset, cudaStream_t s);
-// Factor only (no inverse) of the nb x nb block at A, in place.
+// Factor of the nb x nb block at A, in place.  On a failing pivot p records
+// {pivot_offset + p, status} in info if info[1] is still 0.
 // df: the block is read in double-float storage (written back as FP64).
 cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_offset, cudaStream_t s,
                        bool df = false);
@@ -242,8 +238,6 @@ cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_of
 // mode 1 X <- X T^{-1}.  df: X is read in double-float storage (written back as FP64).
 cudaError_t trsm_rows(int m, int nb, double *X, long long ldx, const double *T, long long ldt, int mode,
                       cudaStream_t s, bool df = false);
-// Inverse (lower, ld = nb) of the nb x nb lower block D.
-cudaError_t trtri_diag(int nb, const double *D, long long ldd, double *Dinv, cudaStream_t s);
 // Inverses of all diagonal blocks of L in one launch: block 0 = rows [0, first),
 // block ib >= 1 = [first + (ib-1) b, first + ib b); inverse ib at out + ib b^2
 // (leading dimension = block size), or, when ldo != 0, at its diagonal
@@ -282,12 +276,15 @@ cudaError_t glm_categorical(long long n, int k, int C, const double *X, long lon
                             const double *alpha, const double *beta, double *lp, double *dalpha, double *dbeta,
                             void *ws, cudaStream_t s);
 // Triangular inverse, solve and solve adjoint (trinv.cu); X is the inverse.
-cudaError_t tri_inverse(int n, const double *L, long long ldl, double *X, long long ldx, cudaStream_t s);
+// ws (may be null): scratch for split products, tri_workspace_bytes or less.
+size_t tri_workspace_bytes(int n, int m);
+cudaError_t tri_inverse(int n, const double *L, long long ldl, double *X, long long ldx, void *ws, size_t ws_bytes,
+                        cudaStream_t s);
 cudaError_t tri_solve(int n, int m, const double *L, long long ldl, const double *B, long long ldb, double *X,
-                      long long ldx, double *C, long long ldc, cudaStream_t s);
+                      long long ldx, double *C, long long ldc, void *ws, size_t ws_bytes, cudaStream_t s);
 cudaError_t tri_solve_adjoint(int n, int m, const double *X, long long ldx, const double *C, long long ldc,
                               const double *Cbar, long long ldcb, double *Bbar, long long ldbb, double *Lbar,
-                              long long ldlb, cudaStream_t s);
+                              long long ldlb, void *ws, size_t ws_bytes, cudaStream_t s);
 size_t chol_workspace_bytes(int n, int precision);
 size_t adjoint_workspace_bytes(int n, int precision);
 size_t trsv_workspace_bytes(int n);
@@ -356,8 +353,8 @@ constexpr size_t kF64xScratchCap = size_t(1) << 30;  // a general product's slic
 // A checked product (8 slices) of K terms loses at most K 2^-62.5 relative to
 // its operands' row scales; the FP64 chain's bound is K 2^-53 S with S = sum
 // |a'||b'| in the same units, so S >= 2^-9.5 suffices.  S is formed from the
-// leading digits, which exceed an entry by at most a factor of two each: 2^-7.
-constexpr float kF64xTheta = 0.0078125f;
+// leading eight bits of the magnitudes (rounded toward zero: never too large).
+constexpr float kF64xTheta = 0x1.7p-10f;
 size_t f64x_slice_bytes(int rows, int kchunks);
 // The slices of split_operand, kF64xSlices of them, of the entries scaled by
 // 2^(kexp_sign kexp[k] - rexp[r]) (either may be null).  saturate: scaled

@@ -33,8 +33,8 @@
 // term, absolutely, where the FP64 chain's bound is K 2^-53 sum |a'||b'|.  The
 // factorisation and its adjoint only need the bound relative to the scales
 // (2^E_i 2^E_j bounds |K_ij| by the diagonal; see mixed.cu).  A general product
-// is checked: an S = 1 pass forms sum |a'_1||b'_1| from the leading digits for
-// every output, and a 32 x 32 block with an output below the threshold (or with
+// is checked: an S = 1 pass forms sum |a'||b'| from the magnitudes' leading eight bits
+// for every output, and a 32 x 32 block with an output below the threshold (or with
 // an infinity, a NaN or denormal rows) is left to the FP64 kernel, which
 // computes just those blocks in the following launch.
 //
@@ -306,7 +306,7 @@ __device__ __forceinline__ void prefetch_output(const FxParams &p, const Work &k
 }
 
 // ------------------------------------------------------------------ the product
-// S slices; CHECK (S = 1): sums of |a'_1||b'_1| against theta, into flags.
+// S slices; CHECK (S = 1): sums of the magnitudes' products against theta, into flags.
 template <int S, bool NEG, bool CHECK>
 __global__ void __launch_bounds__(FX_THREADS, 1)
 f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, FxParams p) {
@@ -655,7 +655,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 // set to 2^30 when sat is 1 (a row of an indefinite matrix: its pivot fails
 // either way) and to NaN otherwise; NaN stays NaN (codes: both left out, the
 // row is flagged).  Plane p of row r: dst[p plane + (r + row offset) kpad + ..];
-// ABS adds plane S with the magnitudes of the leading digits.  One row per
+// ABS adds plane S with the magnitudes, rounded toward zero to BF16.  One row per
 // warp, 8 rows (8 KiB) per CTA, as in ozaki.cu's split.
 struct FxOperand {
   const double *src;
@@ -742,6 +742,14 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   emax = __reduce_max_sync(0xffffffffu, emax);
   unsigned short *dst =
       o.dst + (long long)blockIdx.z * o.dst_stride + (long long)r * o.kpad + (long long)c * FX_CHUNK + lane * 4;
+  if (ABS) {  // magnitudes, rounded toward zero to BF16
+    uint32_t h[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      h[i] = (mant[i] != 0 && ex[i] >= -126)
+                 ? ((uint32_t)(ex[i] + 127) << 7) | ((uint32_t)(mant[i] >> 45) & 0x7Fu) : 0u;
+    *(uint2 *)(dst + S * o.plane) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+  }
   // X + 128 (1 + 256 + ..) has the balanced digits plus 128 as its lower bytes
   unsigned long long Y[4];
   uint32_t top[4];
@@ -768,8 +776,6 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
       const float d = __fsub_rn(__uint_as_float(0x4B000000u | byte), pp == 0 ? 8388608.0f : 8388736.0f);
       h[i] = __float_as_uint(__fmul_rn(d, __uint_as_float(sb)));
     }
-    if (ABS && pp == 0)
-      *(uint2 *)(dst + S * o.plane) = make_uint2((h[0] >> 16) | (h[1] & 0xFFFF0000u), (h[2] >> 16) | (h[3] & 0xFFFF0000u));
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       h[i] ^= (neg >> i & 1u) << 31;
@@ -1210,7 +1216,7 @@ size_t f64x_scratch_bytes(int M, int N, int K, int batch) {
 // at 1024 x 1024 x 64 (6.7e7; 62 us here).
 bool f64x_worth(const Gemm &g) {
   auto pad = [](int v) { return (double)((v + 63) / 64 * 64); };
-  return g.M >= 8 && g.N >= 8 && g.K >= 32 && g.batch * pad(g.M) * pad(g.N) * g.K >= 3e7;
+  return g.M >= 8 && g.N >= 8 && g.K >= 16 && g.batch * pad(g.M) * pad(g.N) * g.K >= 3e7;
 }
 
 cudaError_t gemm_f64x(const Gemm &g, void *ws, size_t ws_bytes, cudaStream_t s) {

@@ -39,7 +39,7 @@ struct Params {
   long long sA, sB, sC;  // per-product offsets of a batch (grid.y)
   double *partial;  // non-null when grid.z > 1
   const unsigned char *flags;  // Gemm::flags
-  int flag_ld, ksh_m, ksh_n;
+  int flag_ld, flag_any, ksh_m, ksh_n;
   long long flag_stride;
 };
 
@@ -154,14 +154,18 @@ __global__ void __launch_bounds__(THREADS) gemm_f64_kernel(Params p) {
     tn = blockIdx.x - tm * p.tiles_n;
   }
   const int m0 = tm * T, n0 = tn * T;
+  // Flagged products (Gemm::flags): a 64-wide tile whose blocks are all asked for
+  // is computed as one; a single block takes the 32-wide kernel, where it costs
+  // 20 us for 64 K steps against 79 us as part of a tile (one SM's FP64 rate).
+  // With split K (flag_any) the 64-wide kernel takes every tile with a block in it.
   const unsigned char *fl = nullptr;
-  if constexpr (T == 64) {
-    if (p.flags) {  // 2 x 2 blocks of 32, one per warp
-      fl = p.flags + (size_t)blockIdx.y * p.flag_stride + (size_t)(m0 / 32) * p.flag_ld + n0 / 32;
-      // blocks past the output's edge are not flagged
-      const bool r1 = m0 + 32 < p.M, c1 = n0 + 32 < p.N;
-      if (fl[0] && (!c1 || fl[1]) && (!r1 || fl[p.flag_ld]) && (!r1 || !c1 || fl[p.flag_ld + 1])) return;
-    }
+  if (p.flags) {
+    const int t0 = (m0 / 64) * 2, u0 = (n0 / 64) * 2;
+    fl = p.flags + (size_t)blockIdx.y * p.flag_stride + (size_t)t0 * p.flag_ld + u0;
+    const bool r1 = 32 * (t0 + 1) < p.M, c1 = 32 * (u0 + 1) < p.N;  // blocks past the edge are not flagged
+    const bool all = !fl[0] && (!c1 || !fl[1]) && (!r1 || !fl[p.flag_ld]) && (!r1 || !c1 || !fl[p.flag_ld + 1]);
+    const bool none = fl[0] && (!c1 || fl[1]) && (!r1 || fl[p.flag_ld]) && (!r1 || !c1 || fl[p.flag_ld + 1]);
+    if (T == 64 ? (p.flag_any ? none : !all) : (all || fl[(m0 / 32 - t0) * p.flag_ld + n0 / 32 - u0])) return;
   }
   // a skipped leading K range is a multiple of 64, so kbeg stays on a K step
   const int kfirst = p.kskip == KSKIP_ROWS ? m0 + p.ksh_m : (p.kskip == KSKIP_COLS ? n0 + p.ksh_n : 0);
@@ -183,7 +187,10 @@ __global__ void __launch_bounds__(THREADS) gemm_f64_kernel(Params p) {
       for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.0;
 
   double ra[V], rb[V];
+  // a flagged product: a warp whose block is not asked for only helps to load
+  const bool idle = T == 64 && fl && fl[wm * p.flag_ld + wn];
   auto compute = [&](int buf) {
+    if (idle) return;
     double a[MI][8], b[NI][4];
 #pragma unroll
     for (int mi = 0; mi < MI; ++mi) {
@@ -230,7 +237,7 @@ __global__ void __launch_bounds__(THREADS) gemm_f64_kernel(Params p) {
     }
   }
 
-  if (fl && fl[wm * p.flag_ld + wn]) return;
+  if (idle) return;
   // Epilogue: fragment (mi, ni) element r sits at row g (+8 for r >= 2),
   // column 2*tg + (r & 1) of the 16 x 8 tile.
   const bool split = p.partial != nullptr;
@@ -371,6 +378,19 @@ cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t s) {
   const double flops = g.algo_flops > 0.0 ? g.algo_flops : 2.0 * mn * (double)p.K * g.batch;
   const double bytes =
       8.0 * g.batch * ((double)g.M * p.K + (double)p.K * g.N + (g.beta != 0.0 ? 2.0 : 1.0) * mn);
+  p.flag_any = splits > 1;
+  if (g.flags && splits == 1) {  // single blocks: the 32-wide kernel (before the 64-wide one changes nothing it reads)
+    const int tiles_n = p.tiles_n;
+    p.tiles_n = (g.N + 31) / 32;
+    const dim3 bgrid((unsigned)tile_count(32), (unsigned)g.batch, 1);
+    GPC_LAUNCH(GPC_TRACE_GEMM_F64, 0.0, 0.0, s, {
+      if (!g.transA && !g.transB) gemm_f64_kernel<32, false, false><<<bgrid, THREADS, 0, s>>>(p);
+      else if (!g.transA && g.transB) gemm_f64_kernel<32, false, true><<<bgrid, THREADS, 0, s>>>(p);
+      else if (g.transA && !g.transB) gemm_f64_kernel<32, true, false><<<bgrid, THREADS, 0, s>>>(p);
+      else gemm_f64_kernel<32, true, true><<<bgrid, THREADS, 0, s>>>(p);
+    });
+    p.tiles_n = tiles_n;
+  }
   if (small) {
     if (cudaError_t ce = small_tile_carveout(); ce != cudaSuccess) return ce;
     GPC_LAUNCH(GPC_TRACE_GEMM_F64, flops, bytes, s, {

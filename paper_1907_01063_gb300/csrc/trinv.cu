@@ -57,7 +57,7 @@ cudaError_t zero_strict_upper(int n, double *X, long long ldx, cudaStream_t s) {
 // block of pair p has rows [r0 + 2wp, r0 + 2wp + w), the lower one the next h
 // rows.  A3 is read from L, C1 and C2 from X, and C3 is written to X.
 cudaError_t combine_pairs(int w, int h, int count, int r0, const double *L, long long ldl, double *X,
-                          long long ldx, cudaStream_t s) {
+                          long long ldx, void *ws, size_t ws_bytes, cudaStream_t s) {
   const long long stepL = 2LL * w * (ldl + 1), stepX = 2LL * w * (ldx + 1);
   // T^T (w x h) = A3^T C2^T, into the mirror image of C3 in X's upper triangle.
   // op(B) = C2^T is upper triangular: columns below n0 + 64 need k < n0 + 64.
@@ -72,7 +72,7 @@ cudaError_t combine_pairs(int w, int h, int count, int r0, const double *L, long
   t.kskip = KSKIP_COLS_END;
   t.batch = count; t.sA = stepL; t.sB = stepX; t.sC = stepX;
   t.algo_flops = (double)count * w * h * (h + 1.0);
-  TRY(gemm_f64(t, nullptr, s));
+  TRY(gemm_f64x(t, ws, ws_bytes, s));
   // C3 (h x w) = -T C1; op(B) = C1 is lower triangular: columns from n0 need k >= n0.
   Gemm c;
   c.M = h; c.N = w; c.K = w;
@@ -84,28 +84,55 @@ cudaError_t combine_pairs(int w, int h, int count, int r0, const double *L, long
   c.kskip = KSKIP_COLS;
   c.batch = count; c.sA = stepX; c.sB = stepX; c.sC = stepX;
   c.algo_flops = (double)count * h * w * (w + 1.0);
-  return gemm_f64(c, nullptr, s);
+  return gemm_f64x(c, ws, ws_bytes, s);
 }
 
 }  // namespace
 
-cudaError_t tri_inverse(int n, const double *L, long long ldl, double *X, long long ldx, cudaStream_t s) {
+// Slice scratch of the largest product of an inverse of order n and, with m > 0,
+// of the solve and its reverse mode (0: every product is too small for slices).
+size_t tri_workspace_bytes(int n, int m) {
+  size_t need = 0;
+  auto add = [&](int M, int N, int K, int batch) {
+    Gemm g;
+    g.M = M;
+    g.N = N;
+    g.K = K;
+    g.batch = batch;
+    if (f64x_worth(g)) need = std::max(need, f64x_scratch_bytes(M, N, K, batch));
+    else if (gemm_f64_splits(g)) need = std::max(need, gemm_f64_scratch_bytes());
+  };
+  for (long long w = kInvBlock; w < n; w *= 2) {
+    const int full = (int)(n / (2 * w)), rest = (int)(n - full * 2 * w);
+    if (full > 0) add((int)w, (int)w, (int)w, full);
+    if (rest > w) add((int)w, rest - (int)w, (int)w, 1);
+  }
+  if (m > 0) {
+    add(n, m, n, 1);
+    add(n, n, m, 1);
+  }
+  return need ? std::max(need, gemm_f64_scratch_bytes()) : 0;
+}
+
+cudaError_t tri_inverse(int n, const double *L, long long ldl, double *X, long long ldx, void *ws, size_t ws_bytes,
+                        cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int b = kInvBlock;
   TRY(trtri_batched(n, L, ldl, std::min(b, n), b, X, s, ldx));
   for (long long w = b; w < n; w *= 2) {
     const long long full = n / (2 * w);  // pairs whose lower block has all w rows
     const long long rest = n - full * 2 * w;
-    if (full > 0) TRY(combine_pairs((int)w, (int)w, (int)full, 0, L, ldl, X, ldx, s));
-    if (rest > w) TRY(combine_pairs((int)w, (int)(rest - w), 1, (int)(full * 2 * w), L, ldl, X, ldx, s));
+    if (full > 0) TRY(combine_pairs((int)w, (int)w, (int)full, 0, L, ldl, X, ldx, ws, ws_bytes, s));
+    if (rest > w) TRY(combine_pairs((int)w, (int)(rest - w), 1, (int)(full * 2 * w), L, ldl, X, ldx, ws,
+                                    ws_bytes, s));
   }
   return zero_strict_upper(n, X, ldx, s);
 }
 
 cudaError_t tri_solve(int n, int m, const double *L, long long ldl, const double *B, long long ldb, double *X,
-                      long long ldx, double *C, long long ldc, cudaStream_t s) {
+                      long long ldx, double *C, long long ldc, void *ws, size_t ws_bytes, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  TRY(tri_inverse(n, L, ldl, X, ldx, s));
+  TRY(tri_inverse(n, L, ldl, X, ldx, ws, ws_bytes, s));
   if (m <= 0) return cudaSuccess;
   Gemm g;  // C = X B; op(A) = X is lower triangular: rows below m0 + 64 need k < m0 + 64
   g.M = n; g.N = m; g.K = n;
@@ -114,12 +141,12 @@ cudaError_t tri_solve(int n, int m, const double *L, long long ldl, const double
   g.C = C; g.ldc = ldc;
   g.kskip = KSKIP_ROWS_END;
   g.algo_flops = (double)n * n * m;
-  return gemm_f64(g, nullptr, s);
+  return gemm_f64x(g, ws, ws_bytes, s);
 }
 
 cudaError_t tri_solve_adjoint(int n, int m, const double *X, long long ldx, const double *C, long long ldc,
                               const double *Cbar, long long ldcb, double *Bbar, long long ldbb, double *Lbar,
-                              long long ldlb, cudaStream_t s) {
+                              long long ldlb, void *ws, size_t ws_bytes, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (m <= 0)
     return cudaMemset2DAsync(Lbar, (size_t)ldlb * sizeof(double), 0, (size_t)n * sizeof(double), (size_t)n, s);
@@ -130,7 +157,7 @@ cudaError_t tri_solve_adjoint(int n, int m, const double *X, long long ldx, cons
   g.C = Bbar; g.ldc = ldbb;
   g.kskip = KSKIP_ROWS;
   g.algo_flops = (double)n * n * m;
-  TRY(gemm_f64(g, nullptr, s));
+  TRY(gemm_f64x(g, ws, ws_bytes, s));
   Gemm l;  // Lbar = -tril(Bbar C^T), lower output tiles only
   l.M = n; l.N = n; l.K = m;
   l.A = Bbar; l.lda = ldbb;
@@ -138,7 +165,7 @@ cudaError_t tri_solve_adjoint(int n, int m, const double *X, long long ldx, cons
   l.C = Lbar; l.ldc = ldlb;
   l.alpha = -1.0;
   l.uplo = UPLO_LOWER;
-  TRY(gemm_f64(l, nullptr, s));
+  TRY(gemm_f64x(l, ws, ws_bytes, s));
   return zero_strict_upper(n, Lbar, ldlb, s);
 }
 
