@@ -1,11 +1,9 @@
 // Diagonal-block kernels and elementwise helpers of the blocked factorisation.
 //
-// potrf_trtri_diag: the small-block factorisation of Section 3.3 (one thread
-// block factors a b x b diagonal block with the classic sequential algorithm,
-// its inner loops spread over the threads), followed by the block's inverse
-// (the per-block inverses of Section 3.2's divide-and-conquer triangular
-// inverse), which turns the panel solve L21 = A21 L11^{-T} into a product.
-// The block lives in shared memory for the whole kernel.
+// The small-block factorisation of Section 3.3 (potrf_la_kernel,
+// potrf_diag_kernel), the panel solve against a factored block
+// (trsm_quad_kernel, trsm_rows_kernel) and the inverses of all diagonal blocks
+// (trtri_cols_kernel; the per-block inverses of Section 3.2).
 #include "common.cuh"
 
 namespace gpc {
@@ -15,99 +13,155 @@ constexpr int DIAG_THREADS = 256;
 
 __device__ __forceinline__ double &S(double *s, int ld, int i, int j) { return s[i * ld + j]; }
 
-// In-place inverse of the lower nb x nb factor held in shared memory
-// (backward column sweep: with L = [[l, 0], [x, L2]],
-//  L^{-1} = [[1/l, 0], [-L2^{-1} x / l, L2^{-1}]]).
-__device__ void invert_lower_smem(double *s, int ld, int nb) {
-  __shared__ double col[kMaxBlock];
-  for (int j = nb - 1; j >= 0; --j) {
-    const double ljj = S(s, ld, j, j);
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) {
-      double t = 0.0;
-      for (int k = j + 1; k <= i; ++k) t = fma(S(s, ld, i, k), S(s, ld, k, j), t);
-      col[i] = -t / ljj;
+// All diagonal-block inverses of L at once.  Block 0 is rows [0, first),
+// block ib >= 1 is [first + (ib - 1) b, first + ib b).  With ldo == 0 the
+// inverse of block ib goes to out + ib * b * b with leading dimension equal to
+// its size; otherwise to its diagonal position in an n x n matrix out with
+// leading dimension ldo (out may be L itself: the CTAs of a block form a cluster
+// then and meet between their reads and their writes).  (The
+// per-block inverses of Section 3.2, computed as a batch.)
+//
+// FP64 work bounds it: one SM's rate makes a whole 128 block 106 us (nb^3 / 6
+// multiply-adds at 1.6 per cycle), and a batch of a few blocks would leave the
+// other SMs idle.  The columns of an inverse are independent, so a CTA takes 8
+// columns of one block (16 CTAs per 128 block).  trtri16_kernel first inverts
+// every 16 x 16 diagonal sub-block (a warp each, lane = column and row parity)
+// into its final place; trtri_cols_kernel then solves L X = E over 16-row blocks,
+// a warp per block: X_K = Dinv_K R_K by 128 threads (a product of one warp would
+// hold its sub-partition's FP64 pipe 2.5 us), then every later warp subtracts
+// L_IK X_K (one m16n8k16 instruction, its fragment of L loaded one step ahead).
+// Measured (both launches; one CTA per block before): 480 -> 42 us for two 128
+// blocks (n = 256), 500 -> 69 us for 32 (n = 4096).
+constexpr int TI_NB = 16, TI_COLS = 8, TI_WARPS = kMaxBlock / TI_NB;
+
+__device__ __forceinline__ void dmma_16816(double (&c)[4], const double (&a)[8], const double (&b)[4]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f64.f64.f64.f64 {%0,%1,%2,%3}, "
+      "{%4,%5,%6,%7,%8,%9,%10,%11}, {%12,%13,%14,%15}, {%0,%1,%2,%3};\n"
+      : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3])
+      : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(a[4]), "d"(a[5]), "d"(a[6]), "d"(a[7]),
+        "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]));
+}
+
+struct TriBlock {
+  int j0, nb;
+  double *dst;
+  long long ldd;
+};
+__device__ __forceinline__ TriBlock tri_block(int ib, int n, int first, int b, double *out, long long ldo) {
+  TriBlock t;
+  t.j0 = (ib == 0) ? 0 : first + (ib - 1) * b;
+  t.nb = (ib == 0) ? first : min(b, n - t.j0);
+  t.dst = ldo ? out + (long long)t.j0 * ldo + t.j0 : out + (size_t)ib * b * b;
+  t.ldd = ldo ? ldo : t.nb;
+  return t;
+}
+
+// grid.x blocks, grid.y sub-blocks of a block in twos (64 threads)
+__global__ void __launch_bounds__(64)
+trtri16_kernel(int n, const double *L, long long ldl, int first, int b, double *out, long long ldo) {
+  __shared__ double sub_s[2][TI_NB][TI_NB + 1];
+  const TriBlock t = tri_block(blockIdx.x, n, first, b, out, ldo);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, r0 = (2 * blockIdx.y + w) * TI_NB;
+  if (r0 >= t.nb) return;
+  double(*sub)[TI_NB + 1] = sub_s[w];
+  const double *A = L + (long long)(t.j0 + r0) * ldl + t.j0 + r0;
+  const int m = min(TI_NB, t.nb - r0);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {  // padded with the identity
+    const int i = 2 * q + (lane >> 4), j = lane & 15;
+    sub[i][j] = (i < m && j <= i) ? A[(long long)i * ldl + j] : (i == j ? 1.0 : 0.0);
+  }
+  __syncwarp();
+  const int j = lane & 15, h = lane >> 4;
+  double x[8], rd[TI_NB];
+  const double d = 1.0 / sub[j][j];
+#pragma unroll
+  for (int k = 0; k < TI_NB; ++k) rd[k] = __shfl_sync(0xffffffffu, d, k);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) x[u] = (2 * u + h == j) ? 1.0 : 0.0;
+#pragma unroll
+  for (int k = 0; k < TI_NB; ++k) {
+    const double xk = __shfl_sync(0xffffffffu, x[k >> 1], j | ((k & 1) << 4)) * rd[k];
+    if (h == (k & 1)) x[k >> 1] = xk;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (2 * u + 1 <= k) continue;
+      const int i = 2 * u + h;
+      if (i > k) x[u] = fma(-sub[i][k], xk, x[u]);
     }
-    __syncthreads();
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) S(s, ld, i, j) = col[i];
-    if (threadIdx.x == 0) S(s, ld, j, j) = 1.0 / ljj;
-    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = 2 * u + h;
+    if (i < m && j < m) t.dst[(long long)(r0 + i) * t.ldd + r0 + j] = (i >= j) ? x[u] : 0.0;
   }
 }
 
-__device__ void potrf_trtri_body(int nb, double *A, long long lda, double *Winv, long long ldw, int *info,
-                                 int pivot_offset, int factor) {
-  extern __shared__ double smem[];
-  const int ld = nb + 1;
-  __shared__ int fail;
-  if (threadIdx.x == 0) fail = 0;
-  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-    const int i = idx / nb, j = idx - i * nb;
-    S(smem, ld, i, j) = (j <= i) ? A[(long long)i * lda + j] : 0.0;
+__global__ void __launch_bounds__(32 * TI_WARPS, 2)
+trtri_cols_kernel(int n, const double *L, long long ldl, int first, int b, double *out, long long ldo) {
+  __shared__ double dinv[TI_WARPS][TI_NB][TI_NB + 1];
+  __shared__ double rhs[TI_NB][TI_COLS + 1];
+  __shared__ double xs[TI_WARPS][TI_NB][TI_COLS + 1];
+  const TriBlock t = tri_block(blockIdx.x, n, first, b, out, ldo);
+  const int nb = t.nb, c0 = blockIdx.y * TI_COLS;
+  const double *A = L + (long long)t.j0 * ldl + t.j0;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tg = lane & 3;
+  const int k0 = c0 / TI_NB, r0 = w * TI_NB;  // first row block with entries; this warp's rows
+  const bool live = w >= k0 && r0 < nb && c0 < nb;
+  if (live) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = 2 * q + (lane >> 4), j = lane & 15;
+      dinv[w][i][j] = (r0 + i < nb && r0 + j < nb) ? t.dst[(long long)(r0 + i) * t.ldd + r0 + j] : (i == j ? 1.0 : 0.0);
+    }
   }
+  auto load = [&](int K, double(&a)[8]) {  // L_wK as an A fragment
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int row = r0 + g + 8 * (i & 1), col = K * TI_NB + tg + 4 * (i >> 1);
+      a[i] = row < nb ? A[(long long)row * ldl + col] : 0.0;
+    }
+  };
+  double a[8];
+  if (live && w > k0) load(k0, a);
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};  // rows g, g + 8; columns 2 tg, 2 tg + 1
   __syncthreads();
-
-  if (factor) {
-    for (int j = 0; j < nb; ++j) {
-      if (threadIdx.x == 0) {
-        const double p = S(smem, ld, j, j);
-        if (p > 0.0 && p <= 1.79769313486231570e308) {
-          S(smem, ld, j, j) = sqrt(p);
-        } else {
-          fail = 1;
-          if (info && info[1] == 0) {
-            info[0] = pivot_offset + j;
-            info[1] = (p != p || p > 1.79769313486231570e308) ? GPC_ERR_NAN : GPC_ERR_NOT_PD;
-          }
-        }
+  const int last = c0 < nb ? (nb - 1) / TI_NB : k0 - 1;
+  for (int K = k0; K <= last; ++K) {
+    if (w == K) {  // the identity's columns c0 .. c0 + 7 minus the products so far
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int row = g + ((r >> 1) << 3), col = 2 * tg + (r & 1);
+        rhs[row][col] = ((r0 + row == c0 + col) ? 1.0 : 0.0) - acc[r];
       }
-      __syncthreads();
-      if (fail) break;
-      const double d = S(smem, ld, j, j);
-      for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) S(smem, ld, i, j) /= d;
-      __syncthreads();
-      const int m = nb - j - 1;
-      for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-        const int r = idx / m, c = idx - r * m;
-        if (c <= r)
-          S(smem, ld, j + 1 + r, j + 1 + c) -= S(smem, ld, j + 1 + r, j) * S(smem, ld, j + 1 + c, j);
-      }
-      __syncthreads();
     }
-    // L11 back in place, upper part of the block zeroed.
-    for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-      const int i = idx / nb, j = idx - i * nb;
-      A[(long long)i * lda + j] = (j <= i) ? S(smem, ld, i, j) : 0.0;
+    __syncthreads();
+    if (threadIdx.x < TI_NB * TI_COLS) {
+      const int r = threadIdx.x >> 3, c = threadIdx.x & 7;
+      double p[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int q = 0; q < TI_NB; ++q) p[q & 3] = fma(dinv[K][r][q], rhs[q][c], p[q & 3]);
+      xs[K][r][c] = (p[0] + p[1]) + (p[2] + p[3]);
     }
-    if (fail) return;
+    __syncthreads();
+    if (live && w > K) {
+      double bb[4], an[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) bb[i] = xs[K][tg + 4 * i][g];
+      if (K + 1 < w) load(K + 1, an);
+      dmma_16816(acc, a, bb);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) a[i] = an[i];
+    }
   }
-  invert_lower_smem(smem, ld, nb);
-  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-    const int i = idx / nb, j = idx - i * nb;
-    Winv[(long long)i * ldw + j] = (j <= i) ? S(smem, ld, i, j) : 0.0;
+  // every CTA of the block's cluster has read L (a cluster of one unless out is L)
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  for (int idx = threadIdx.x; idx < nb * TI_COLS; idx += blockDim.x) {
+    const int i = idx >> 3, c = idx & 7;
+    // the diagonal sub-blocks are in place already
+    if (c0 + c < nb && i >> 4 != k0) t.dst[(long long)i * t.ldd + c0 + c] = (i >> 4 > k0) ? xs[i >> 4][i & 15][c] : 0.0;
   }
-}
-
-__global__ void __launch_bounds__(DIAG_THREADS)
-potrf_trtri_kernel(int nb, double *A, long long lda, double *Winv, int *info, int pivot_offset,
-                   int factor) {
-  potrf_trtri_body(nb, A, lda, Winv, nb, info, pivot_offset, factor);
-}
-
-// All diagonal-block inverses of L at once, one CTA per block.  Block 0 is
-// rows [0, first), block ib >= 1 is [first + (ib - 1) b, first + ib b).  With
-// ldo == 0 the inverse of block ib goes to out + ib * b * b with leading
-// dimension equal to its size; otherwise to its diagonal position in an
-// n x n matrix out with leading dimension ldo (out may be L itself: each block
-// is read into shared memory before its inverse is written).  (The per-block
-// inverses of Section 3.2, computed as a batch.)
-__global__ void __launch_bounds__(DIAG_THREADS)
-trtri_batched_kernel(int n, const double *L, long long ldl, int first, int b, double *out, long long ldo) {
-  const int ib = blockIdx.x;
-  const int j0 = (ib == 0) ? 0 : first + (ib - 1) * b;
-  const int nb = (ib == 0) ? first : min(b, n - j0);
-  double *dst = ldo ? out + (long long)j0 * ldo + j0 : out + (size_t)ib * b * b;
-  potrf_trtri_body(nb, const_cast<double *>(L) + (long long)j0 * ldl + j0, ldl, dst, ldo ? ldo : nb, nullptr,
-                   0, 0);
 }
 
 // Cholesky factor of one nb x nb diagonal block in shared memory (the small-
@@ -579,54 +633,40 @@ potrf_la_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, i
 
 }  // namespace
 
-static cudaError_t launch_diag(int nb, double *A, long long lda, double *Winv, int *info,
-                               int pivot_offset, int factor, cudaStream_t s) {
-  if (nb <= 0) return cudaSuccess;
-  if (nb > kMaxBlock) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)nb * (nb + 1) * sizeof(double);
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(potrf_trtri_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)((size_t)kMaxBlock * (kMaxBlock + 1) * sizeof(double)));
-    if (e != cudaSuccess) return e;
-    attr_set[dev] = true;
-  }
-  const double nb3 = (double)nb * nb * nb;
-  GPC_LAUNCH(GPC_TRACE_DIAG, (factor ? nb3 / 3.0 : 0.0) + nb3 / 3.0, 8.0 * 1.5 * nb * nb, s,
-             potrf_trtri_kernel<<<1, DIAG_THREADS, smem, s>>>(nb, A, lda, Winv, info, pivot_offset,
-                                                               factor));
-  return cudaGetLastError();
-}
-
-cudaError_t potrf_trtri_diag(int nb, double *A, long long lda, double *Winv, int *info,
-                             int pivot_offset, cudaStream_t s) {
-  return launch_diag(nb, A, lda, Winv, info, pivot_offset, 1, s);
-}
-
-cudaError_t trtri_diag(int nb, const double *D, long long ldd, double *Dinv, cudaStream_t s) {
-  return launch_diag(nb, const_cast<double *>(D), ldd, Dinv, nullptr, 0, 0, s);
-}
-
 cudaError_t trtri_batched(int n, const double *L, long long ldl, int first, int b, double *out,
                           cudaStream_t s, long long ldo) {
   if (n <= 0) return cudaSuccess;
   if (b > kMaxBlock || first < 1 || first > b) return cudaErrorInvalidValue;
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(trtri_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)((size_t)kMaxBlock * (kMaxBlock + 1) * sizeof(double)));
-    if (e != cudaSuccess) return e;
-    attr_set[dev] = true;
-  }
   const int nblk = 1 + (n - first + b - 1) / b;
-  const size_t smem = (size_t)b * (b + 1) * sizeof(double);
+  const bool in_place = (const double *)out == L;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nblk, (unsigned)((b + TI_COLS - 1) / TI_COLS));
+  cfg.blockDim = dim3(32 * TI_WARPS);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  if (in_place) {
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr_set[dev]) {  // up to 16 CTAs per cluster
+      cudaError_t e = cudaFuncSetAttribute(trtri_cols_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+      attr_set[dev] = true;
+    }
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = cfg.gridDim.y;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  GPC_LAUNCH(GPC_TRACE_DIAG, (double)n * TI_NB * TI_NB / 3.0, 16.0 * (double)n * TI_NB, s,
+             trtri16_kernel<<<dim3((unsigned)nblk, (unsigned)((b + 31) / 32)), 64, 0, s>>>(n, L, ldl, first, b, out, ldo));
+  if (b <= TI_NB) return cudaGetLastError();
+  cudaError_t le = cudaSuccess;
   GPC_LAUNCH(GPC_TRACE_DIAG, (double)n * b * b / 3.0, 16.0 * (double)n * b, s,
-             trtri_batched_kernel<<<nblk, DIAG_THREADS, smem, s>>>(n, L, ldl, first, b, out, ldo));
-  return cudaGetLastError();
+             le = cudaLaunchKernelEx(&cfg, trtri_cols_kernel, n, L, ldl, first, b, out, ldo));
+  return le;
 }
 
 cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_offset, cudaStream_t s, bool df) {
