@@ -54,6 +54,7 @@ _SIGNATURES = {
     "gpc_test_split_f64": ([_c_int, _c_vp, _c_vp, _c_vp, _c_vp], _c_int),
     "gpc_version": ([], _c_int),
     "gpc_workspace_size": ([_c_int, _c_int, ctypes.POINTER(_c_size)], _c_int),
+    "gpc_workspace_min_size": ([_c_int, _c_int, ctypes.POINTER(_c_size)], _c_int),
     "gpc_set_tuning": ([_c_int, _c_int], _c_int),
     "gpc_get_tuning": ([_c_int, ctypes.POINTER(_c_int)], _c_int),
     "gpc_se_cov": ([_c_int, _c_int, _c_vp, _c_int, _c_double, _c_double, _c_double, _c_double,
@@ -261,11 +262,12 @@ def check_info(info: torch.Tensor, what: str = "factorisation"):
 
 
 def _ws_for(n: int, precision, ws: torch.Tensor | None, device) -> torch.Tensor:
-    need = workspace_size(n, precision)
     if ws is None:
-        return torch.empty(need, dtype=torch.uint8, device=device)
-    if ws.numel() * ws.element_size() < need or not ws.is_cuda:
-        raise ValueError(f"workspace too small: need {need} bytes")
+        return torch.empty(workspace_size(n, precision), dtype=torch.uint8, device=device)
+    b = ctypes.c_size_t()
+    _check(capi.gpc_workspace_min_size(int(n), precision_code(precision), ctypes.byref(b)), "gpc_workspace_min_size")
+    if ws.numel() * ws.element_size() < b.value or not ws.is_cuda:
+        raise ValueError(f"workspace too small: need {b.value} bytes")
     return ws
 
 
@@ -383,7 +385,10 @@ def trsv(L: torch.Tensor, x: torch.Tensor, trans: bool = False,
     n = L.shape[0]
     ldl = _square(L, "L")
     _vector(x, n, "x")
-    wsb = _ws_for(n, "fp64", ws, L.device)
+    if ws is None:  # the solve's ticket and ready flags
+        wsb = torch.empty(4 * ((n + 63) // 64 + 1) + 256, dtype=torch.uint8, device=L.device)
+    else:
+        wsb = _ws_for(n, "fp64", ws, L.device)
     _check(capi.gpc_trsv(n, _ptr(L), ldl, _ptr(x), 1 if trans else 0, _ptr(wsb), wsb.numel(),
                          _stream()), "gpc_trsv")
     return x

@@ -32,16 +32,20 @@ struct ApiWs {
   double *vec;   // 4 n doubles
   void *refine;  // refinement residual, partial norms and state
   int *flags;    // triangular-solve tickets and ready flags
+  bool slices;   // FP64: products on slices
 };
 
 constexpr int kRefineMaxIters = 10;
 constexpr double kRefineTol = 1e-14;
 constexpr size_t kGemmWorkspace = size_t(256) << 20;  // gpc_gemm_workspace_size; 40 MB (split-K tiles) is accepted
 
-size_t core_bytes(int n, int precision) {
-  size_t c = std::max(chol_workspace_bytes(n, precision), adjoint_workspace_bytes(n, precision));
+// FP64 calls run on slices where the workspace has room for them (gpc_workspace_size)
+// and on the FP64 kernels in the smaller workspace of gpc_workspace_min_size.
+size_t core_bytes(int n, int precision, bool slices) {
+  size_t c = std::max(chol_workspace_bytes(n), adjoint_workspace_bytes(n));
   c = std::max(c, ltv_workspace_bytes(n));
   if (precision == GPC_MIXED) c = std::max(c, mixed_workspace_bytes(n));
+  else if (slices) c = std::max(c, mixed_workspace_bytes(n, true));
   return align_up(c, 256);
 }
 
@@ -53,16 +57,20 @@ size_t flags_bytes(int n) {
   return std::max(trsv_workspace_bytes(std::max(n, 1)), align_up(((size_t)(n + 15) / 16 + 1) * sizeof(int), 256));
 }
 
-size_t total_bytes(int n, int precision) {
-  return core_bytes(n, precision) + align_up(4 * (size_t)std::max(n, 1) * sizeof(double), 256) +
+size_t total_bytes(int n, int precision, bool slices) {
+  return core_bytes(n, precision, slices) + align_up(4 * (size_t)std::max(n, 1) * sizeof(double), 256) +
          refine_workspace_bytes(std::max(n, 1)) + flags_bytes(n);
 }
 
-ApiWs carve(void *ws, int n, int precision) {
+size_t min_bytes(int n, int precision) { return total_bytes(n, precision, false); }
+size_t full_bytes(int n, int precision) { return total_bytes(n, precision, f64_on_slices(n)); }
+
+ApiWs carve(void *ws, size_t ws_bytes, int n, int precision) {
   ApiWs w;
+  w.slices = precision == GPC_FP64 && f64_on_slices(n) && ws_bytes >= full_bytes(n, precision);
   char *p = (char *)ws;
   w.core = p;
-  p += core_bytes(n, precision);
+  p += core_bytes(n, precision, w.slices);
   w.vec = (double *)p;
   p += align_up(4 * (size_t)std::max(n, 1) * sizeof(double), 256);
   w.refine = p;
@@ -182,7 +190,13 @@ int gpc_get_tuning(int key, int *value) {
 
 int gpc_workspace_size(int n, int precision, size_t *bytes) {
   if (!bytes || n < 0 || (precision != GPC_FP64 && precision != GPC_MIXED)) return GPC_ERR_INVALID_ARG;
-  *bytes = total_bytes(n, precision);
+  *bytes = full_bytes(n, precision);
+  return GPC_OK;
+}
+
+int gpc_workspace_min_size(int n, int precision, size_t *bytes) {
+  if (!bytes || n < 0 || !valid_precision(precision)) return GPC_ERR_INVALID_ARG;
+  *bytes = min_bytes(n, precision);
   return GPC_OK;
 }
 
@@ -198,14 +212,14 @@ int gpc_chol(int n, const double *K, int ldk, double *L, int ldl, int precision,
              size_t ws_bytes, int *info, gpc_stream_t stream) {
   if (n < 0 || !valid_precision(precision) || !info) return GPC_ERR_INVALID_ARG;
   if (n == 0) return status_of(reset_info(info, stream));
-  if (bad_square(n, K, ldk) || bad_square(n, L, ldl) || !ws || ws_bytes < total_bytes(n, precision))
+  if (bad_square(n, K, ldk) || bad_square(n, L, ldl) || !ws || ws_bytes < min_bytes(n, precision))
     return GPC_ERR_INVALID_ARG;
   if ((const void *)K == (const void *)L) {
     if (ldk != ldl) return GPC_ERR_INVALID_ARG;
   } else if (overlaps(K, mat_bytes(n, ldk), L, mat_bytes(n, ldl))) {
     return GPC_ERR_INVALID_ARG;
   }
-  ApiWs w = carve(ws, n, precision);
+  ApiWs w = carve(ws, ws_bytes, n, precision);
   cudaError_t e = reset_info(info, stream);
   if (precision == GPC_MIXED) {
     if (e == cudaSuccess) e = to_df_lower(n, K, ldk, L, ldl, stream);
@@ -213,7 +227,7 @@ int gpc_chol(int n, const double *K, int ldk, double *L, int ldl, int precision,
     return status_of(e);
   }
   if (e == cudaSuccess) e = copy_lower(n, K, ldk, L, ldl, stream);
-  if (e == cudaSuccess) e = chol_fp64(n, L, ldl, w.core, info, stream);
+  if (e == cudaSuccess) e = chol_fp64(n, L, ldl, w.core, info, stream, w.slices);
   return status_of(e);
 }
 
@@ -223,7 +237,7 @@ int gpc_chol_adjoint(int n, const double *L, int ldl, const double *Lbar, int ld
   if (n < 0 || !valid_precision(precision)) return GPC_ERR_INVALID_ARG;
   if (n == 0) return GPC_OK;
   if (bad_square(n, L, ldl) || bad_square(n, Lbar, ldlb) || bad_square(n, Kbar, ldkb) || !ws ||
-      ws_bytes < total_bytes(n, precision))
+      ws_bytes < min_bytes(n, precision))
     return GPC_ERR_INVALID_ARG;
   if ((const void *)Lbar == (const void *)Kbar) {
     if (ldlb != ldkb) return GPC_ERR_INVALID_ARG;
@@ -231,14 +245,14 @@ int gpc_chol_adjoint(int n, const double *L, int ldl, const double *Lbar, int ld
     return GPC_ERR_INVALID_ARG;
   }
   if (overlaps(L, mat_bytes(n, ldl), Kbar, mat_bytes(n, ldkb))) return GPC_ERR_INVALID_ARG;
-  ApiWs w = carve(ws, n, precision);
+  ApiWs w = carve(ws, ws_bytes, n, precision);
   cudaError_t e;
   if (precision == GPC_MIXED) {
     e = to_df_lower(n, Lbar, ldlb, Kbar, ldkb, stream);
     if (e == cudaSuccess) e = chol_adjoint_mixed(n, L, ldl, Kbar, ldkb, w.core, w.flags, stream);
   } else {
     e = copy_lower(n, Lbar, ldlb, Kbar, ldkb, stream);
-    if (e == cudaSuccess) e = chol_adjoint_fp64(n, L, ldl, Kbar, ldkb, w.core, stream);
+    if (e == cudaSuccess) e = chol_adjoint_fp64(n, L, ldl, Kbar, ldkb, w.core, w.flags, stream, w.slices);
   }
   if (e == cudaSuccess && symmetric_out) e = lower_to_symmetric_half(n, Kbar, ldkb, stream);
   return status_of(e);
@@ -450,7 +464,7 @@ int gpc_gp_lml(int n, const double *K, int ldk, const double *y, double *L, int 
     return status_of(e);
   }
   if (bad_square(n, K, ldk) || bad_square(n, L, ldl) || !y || !alpha || !ws ||
-      ws_bytes < total_bytes(n, precision))
+      ws_bytes < min_bytes(n, precision))
     return GPC_ERR_INVALID_ARG;
   if ((const void *)K == (const void *)L) {
     if (ldk != ldl || precision == GPC_MIXED) return GPC_ERR_INVALID_ARG;
@@ -460,18 +474,18 @@ int gpc_gp_lml(int n, const double *K, int ldk, const double *y, double *L, int 
   if (overlaps(alpha, n * sizeof(double), L, mat_bytes(n, ldl)) ||
       overlaps(alpha, n * sizeof(double), y, n * sizeof(double)))
     return GPC_ERR_INVALID_ARG;
-  ApiWs w = carve(ws, n, precision);
+  ApiWs w = carve(ws, ws_bytes, n, precision);
   cudaError_t e = reset_info(info, stream);
   if (precision == GPC_MIXED) {
     if (e == cudaSuccess) e = to_df_lower(n, K, ldk, L, ldl, stream);
     if (e == cudaSuccess) e = chol_mixed(n, L, ldl, w.core, info, stream);
   } else {
     if (e == cudaSuccess) e = copy_lower(n, K, ldk, L, ldl, stream);
-    if (e == cudaSuccess) e = chol_fp64(n, L, ldl, w.core, info, stream);
+    if (e == cudaSuccess) e = chol_fp64(n, L, ldl, w.core, info, stream, w.slices);
   }
   // the factorisation left every diagonal-block inverse at the start of the core workspace
   const double *inv = (const double *)w.core;
-  const int b = chol_block_size(precision);
+  const int b = precision == GPC_MIXED || w.slices ? kSliceBlock : tuning().block;
   if (e == cudaSuccess) e = cudaMemcpyAsync(alpha, y, n * sizeof(double), cudaMemcpyDeviceToDevice, stream);
   if (precision == GPC_MIXED) {
     // The mixed path solves in double-float: its factor's own error is far
@@ -480,7 +494,7 @@ int gpc_gp_lml(int n, const double *K, int ldk, const double *y, double *L, int 
     // inverses (free after the factorisation); the solved sub-blocks pass
     // through w.vec.
     const size_t inv_bytes = align_up((size_t)((n + b - 1) / b) * b * b * sizeof(double), 256);
-    const bool room = core_bytes(n, precision) >= inv_bytes + (size_t)n * n * sizeof(float2);
+    const bool room = core_bytes(n, precision, w.slices) >= inv_bytes + (size_t)n * n * sizeof(float2);
     float2 *Ld = room ? (float2 *)((char *)w.core + inv_bytes) : nullptr;
     float2 *xdf = (float2 *)w.vec;
     if (Ld) {
@@ -508,17 +522,17 @@ int gpc_gp_lml_grad(int n, const double *L, int ldl, const double *alpha, double
   if (n < 0 || !valid_precision(precision)) return GPC_ERR_INVALID_ARG;
   if (n == 0) return GPC_OK;
   if (bad_square(n, L, ldl) || bad_square(n, Kbar, ldkb) || !alpha || !ws ||
-      ws_bytes < total_bytes(n, precision))
+      ws_bytes < min_bytes(n, precision))
     return GPC_ERR_INVALID_ARG;
   if (overlaps(L, mat_bytes(n, ldl), Kbar, mat_bytes(n, ldkb))) return GPC_ERR_INVALID_ARG;
-  ApiWs w = carve(ws, n, precision);
+  ApiWs w = carve(ws, ws_bytes, n, precision);
   double *z = w.vec;
   cudaError_t e = ltv(n, L, ldl, alpha, z, w.core, stream);
   if (e == cudaSuccess) e = lml_lbar(n, L, ldl, alpha, z, gbar, Kbar, ldkb, stream, precision == GPC_MIXED);
   if (precision == GPC_MIXED) {
     if (e == cudaSuccess) e = chol_adjoint_mixed(n, L, ldl, Kbar, ldkb, w.core, w.flags, stream);
   } else {
-    if (e == cudaSuccess) e = chol_adjoint_fp64(n, L, ldl, Kbar, ldkb, w.core, stream);
+    if (e == cudaSuccess) e = chol_adjoint_fp64(n, L, ldl, Kbar, ldkb, w.core, w.flags, stream, w.slices);
   }
   return status_of(e);
 }

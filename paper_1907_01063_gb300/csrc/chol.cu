@@ -1,4 +1,6 @@
-// Blocked Cholesky factorisation and blocked reverse-mode adjoint (FP64).
+// Blocked Cholesky factorisation and blocked reverse-mode adjoint on the FP64
+// kernels: small orders, orders too large for slices, and callers whose workspace
+// has no room for them.  Other FP64 calls run on slices (mixed.cu with f64).
 //
 // Forward (Section 3.3, primitive function): right-looking over b-wide block
 // columns.  Each step factors the diagonal block and forms its inverse in one
@@ -76,21 +78,26 @@ AdjWs carve_adj(void *ws, int n) {
 
 }  // namespace
 
-size_t chol_workspace_bytes(int n, int /*precision*/) {
+// Likelihood, adjoint and gradient in one pass (FP64 kernels / slices): 0.78 /
+// 0.81 ms at n = 200, 1.13 / 1.08 at 257, 2.50 / 2.10 at 513, 5.05 / 3.71 at 900,
+// 93 / 22.7 at 4096.  Above 40960 the slices of L^T (14 n^2 bytes) would take
+// more than 23 GB beside the caller's matrices.
+bool f64_on_slices(int n) { return n >= 256 && n <= 40960; }
+
+size_t chol_workspace_bytes(int n) {
   const size_t b = block_sz();
   return align_up(nblocks(n) * b * b * sizeof(double), 256) + align_up((size_t)n * b * sizeof(double), 256) +
          gemm_f64_scratch_bytes();
 }
 
-size_t adjoint_workspace_bytes(int n, int /*precision*/) {
+size_t adjoint_workspace_bytes(int n) {
   const size_t b = block_sz();
   return align_up(nblocks(n) * b * b * sizeof(double), 256) + 2 * align_up(b * b * sizeof(double), 256) +
          align_up((size_t)n * b * sizeof(double), 256) + gemm_f64_scratch_bytes();
 }
 
-int chol_block_size(int precision) { return precision == GPC_MIXED ? 128 : (int)block_sz(); }
-
-cudaError_t chol_fp64(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s) {
+cudaError_t chol_fp64(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s, bool slices) {
+  if (slices) return chol_mixed(n, L, ldl, ws, info, s, true);
   const int b = tuning().block;
   CholWs w = carve_chol(ws, n);
   for (int k0 = 0; k0 < n; k0 += b) {
@@ -113,7 +120,8 @@ cudaError_t chol_fp64(int n, double *L, long long ldl, void *ws, int *info, cuda
 }
 
 cudaError_t chol_adjoint_fp64(int n, const double *L, long long ldl, double *A, long long lda,
-                              void *ws, cudaStream_t s) {
+                              void *ws, int *err, cudaStream_t s, bool slices) {
+  if (slices) return chol_adjoint_mixed(n, L, ldl, A, lda, ws, err, s, true);
   const int b = tuning().block;
   AdjWs w = carve_adj(ws, n);
   const int nblk = (int)nblocks(n), first = n - (nblk - 1) * b;

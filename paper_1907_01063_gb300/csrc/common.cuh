@@ -285,12 +285,13 @@ cudaError_t tri_solve(int n, int m, const double *L, long long ldl, const double
 cudaError_t tri_solve_adjoint(int n, int m, const double *X, long long ldx, const double *C, long long ldc,
                               const double *Cbar, long long ldcb, double *Bbar, long long ldbb, double *Lbar,
                               long long ldlb, void *ws, size_t ws_bytes, cudaStream_t s);
-size_t chol_workspace_bytes(int n, int precision);
-size_t adjoint_workspace_bytes(int n, int precision);
+size_t chol_workspace_bytes(int n);
+size_t adjoint_workspace_bytes(int n);
 size_t trsv_workspace_bytes(int n);
-cudaError_t chol_fp64(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s);
+// slices: products on slices (chol_mixed with f64), ws as for it.
+cudaError_t chol_fp64(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s, bool slices);
 cudaError_t chol_adjoint_fp64(int n, const double *L, long long ldl, double *A, long long lda,
-                              void *ws, cudaStream_t s);
+                              void *ws, int *err, cudaStream_t s, bool slices);
 // skip (device int, may be null): when *skip != 0 the solve does nothing.
 cudaError_t trsv(int n, const double *L, long long ldl, double *x, int trans, void *ws,
                  int *info, cudaStream_t s, const int *skip = nullptr);
@@ -317,9 +318,10 @@ cudaError_t trsv_inv_df(int n, const float2 *Ld, long long ldd, const double *in
 // Lower triangle of the FP64 matrix src as FP32 pairs (hi, lo) into dst; the
 // strict upper triangle of dst is not written.
 cudaError_t to_df_tri(int n, const double *src, long long lds, float2 *dst, long long ldd, cudaStream_t s);
-// Block size the factorisation uses at a precision, and where it leaves its
-// diagonal-block inverses (start of the workspace core).
-int chol_block_size(int precision);
+// Block of the factorisations on slices; their diagonal-block inverses are at the start of the workspace core.
+constexpr int kSliceBlock = 128;
+// Whether FP64 calls of order n run on slices (mixed.cu with f64) or on the FP64 kernels (chol.cu).
+bool f64_on_slices(int n);
 
 // ---------------------------------------------------------------- GP pieces
 constexpr int kMaxDim = 256;
@@ -359,13 +361,28 @@ size_t f64x_slice_bytes(int rows, int kchunks);
 // The slices of split_operand, kF64xSlices of them, of the entries scaled by
 // 2^(kexp_sign kexp[k] - rexp[r]) (either may be null).  saturate: scaled
 // entries above 2^30 become 2^30, otherwise (and for NaN) NaN.
+struct F64xRow {
+  int *rexp_out = nullptr;        // non-null (K within one chunk): rows scaled by their own largest entry, exponents here
+  int *block_out = nullptr;       // non-null: the scale of all entries together, each with row_exps[r] added to its
+  const int *row_exps = nullptr;  // exponent and, in the rows from block_rows on, kexp[k] too
+  int block_rows = 0;
+  int tri = 0;                    // 1: entries with k < r are zero (not read)
+  const int *rexp_sub = nullptr;  // non-null: rexp holds one exponent, row r's is *rexp - rexp_sub[r]
+};
 cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,
                        const int *rexp, const int *kexp, int kexp_sign, bool saturate, cudaStream_t s,
-                       int chunk_offset = 0, int row_offset = 0);
-// C (FP64) -= 2^(ra_i + rb_j) A B^T; the other arguments as for ozaki_gemm.
+                       int chunk_offset = 0, int row_offset = 0, const F64xRow &row = F64xRow());
+// Scale exponents: of the rows of L from K's diagonal (2^e_i >= sqrt(K_ii)); of
+// the rows of a lower triangle by their largest entries and then of its
+// columns; of one block (rows scaled by 2^rexp).
+cudaError_t f64x_diag_exps(int n, const double *K, long long ldk, int *rexp, cudaStream_t s);
+cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, int *cexp, cudaStream_t s);
+cudaError_t f64x_block_exp(int nb, const double *A, long long lda, const int *rexp, int *out, cudaStream_t s);
+// C (FP64) -= 2^(ra_i + rb_j) A B^T (with ra_sub: 2^(*ra - ra_sub_i + rb_j)); the other arguments as for ozaki_gemm.
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
-                      double *partial, int *err, cudaStream_t s, int max_ctas = 0, int kdepth = 0, int max_items = 0);
+                      double *partial, int *err, cudaStream_t s, int max_ctas = 0, int kdepth = 0, int max_items = 0,
+                      const int *ra_sub = nullptr);
 // gemm_f64 through checked split products where the size pays for the split
 // and ws (f64x_scratch_bytes, or less: more passes) allows; otherwise gemm_f64,
 // with ws as its split-K scratch.
@@ -411,8 +428,9 @@ cudaError_t ozaki_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &
 cudaError_t to_df_lower(int n, const double *src, long long lds, double *dst, long long ldd, cudaStream_t s);
 // m x c block in double-float storage -> FP64, in place.
 cudaError_t from_df_rect(int m, int c, double *p, long long ld, cudaStream_t s);
-size_t mixed_workspace_bytes(int n);
-cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s);
+// f64: FP64 storage and accuracy (f64x.cu), the large sizes of precision GPC_FP64.
+size_t mixed_workspace_bytes(int n, bool f64 = false);
+cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s, bool f64 = false);
 // Batched per-GP pass (batched.cu); rowX[i] = first row of GP i in X (d per row) and y.
 // mixed: split-BF16 products for the O(n^3) work and FP64 refinement of alpha.
 size_t batched_workspace_bytes(int batch, int nmax, bool mixed);
@@ -420,7 +438,7 @@ cudaError_t batched_gp_lml_grad(int batch, const int *n, const long long *offK, 
                                 const double *X, const double *y, const double *hyp, double *K, double *value,
                                 double *grad3, int *info, int nmax, bool mixed, void *ws, cudaStream_t s);
 cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A, long long lda, void *ws,
-                               int *err, cudaStream_t s);
+                               int *err, cudaStream_t s, bool f64 = false);
 
 // ---------------------------------------------------------------- launch trace
 // Every kernel launch site brackets its launch with trace_begin/trace_end.

@@ -73,7 +73,8 @@ constexpr int FX_THREADS = 64 + 32 * FX_EPI_WARPS;
 constexpr int FX_GROUPS = 7;
 constexpr int FX_A_PLANE = FX_BM * FX_BK * 2;  // 8 KiB
 constexpr int FX_B_PLANE = FX_BN * FX_BK * 2;  // 4 KiB
-constexpr int FX_EPI_BUF = 32 * 16 * 8;        // 32 rows x 16 columns of FP64 per warp (columns XOR-swizzled)
+constexpr int FX_EPI_COLS = 8;                 // columns per pass of an epilogue buffer
+constexpr int FX_EPI_BUF = 3 * 32 * FX_EPI_COLS * 4;  // three FP32 planes of 32 rows per warp (columns XOR-swizzled)
 constexpr int fx_stages(int S) { return S == 1 ? 4 : 2; }
 constexpr int fx_smem(int S) {
   return fx_stages(S) * S * (FX_A_PLANE + FX_B_PLANE) + (S == 1 ? 0 : FX_EPI_WARPS * FX_EPI_BUF) + 1024 + 1024;
@@ -95,9 +96,12 @@ struct FxParams {
   int lower, lower_off;            // entries with col + lower_off <= row
   int kskip, ksh_m, ksh_n;         // known-zero K ranges (Gemm::kskip), shifted by the panel's offsets
   int splits, tiles_m, tiles_n, per_batch, num_work;
+  int sub;                         // 4: four CTAs per tile, each with 8 columns of every epilogue warp's 32 (else 1)
   int a_rows, b_rows;              // slice rows per batch entry
   int accumulate;
   const int *ra, *rb;              // scale exponents of the output's rows and columns (null: 0), ...
+  int ra_mul;                      // 0: one exponent for all rows, less ra_sub[row]
+  const int *ra_sub;
   int ra_codes, rb_codes;          // ... or row_codes_kernel codes
   int ra_stride, rb_stride;        // per batch entry
   double *C;
@@ -115,7 +119,7 @@ struct FxParams {
 __device__ __forceinline__ int row_exp(const int *e, int codes, int i) {
   if (!e) return 0;
   const int v = __ldg(e + i);
-  return codes ? code_exponent(v) : v;
+  return codes ? code_exponent(v) : (v < -100000 ? 0 : v);
 }
 
 // ------------------------------------------------------------------ work list
@@ -286,6 +290,18 @@ __device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&r)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) r[i] = __uint_as_float(v[i]);
 }
+__device__ __forceinline__ void tmem_ld8(uint32_t addr, float (&r)[8]) {
+  uint32_t v[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(addr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r[i] = __uint_as_float(v[i]);
+}
+__device__ __forceinline__ void pin8(float (&r)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) asm volatile("" : "+f"(r[i]));
+}
 __device__ __forceinline__ void pin32(float (&r)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) asm volatile("" : "+f"(r[i]));
@@ -317,7 +333,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char *sA = smem;
   unsigned char *sB = smem + STAGES * A_STAGE;
-  double *epi_buf = (double *)(sB + STAGES * B_STAGE);
+  float *epi_buf = (float *)(sB + STAGES * B_STAGE);
   uint64_t *bars = (uint64_t *)((unsigned char *)epi_buf + (CHECK ? 0 : FX_EPI_WARPS * FX_EPI_BUF));
   // bars: full[STAGES], empty[STAGES], tfull, gfree[NG], drain
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), tfull = smem_u32(bars + 2 * STAGES);
@@ -363,7 +379,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       long long issued = 0;
       bool ok = true;
       for (int w = blockIdx.x; w < p.num_work && ok && !p.no_loads; w += gridDim.x) {
-        const Work k = work_item<CHECK>(p, w);
+        const Work k = work_item<CHECK>(p, CHECK ? w : w / p.sub);
         if (k.skip) continue;
         if (!CHECK && p.accumulate && !p.partial) prefetch_output(p, k);
         const int ya = p.a_row0 + k.b * p.a_rows + k.tm * FX_BM, yb = p.b_row0 + k.b * p.b_rows + k.tn * FX_BN;
@@ -395,7 +411,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       uint32_t phase = 0, tphase = 0;
       bool ok = true, any = false;
       for (int w = blockIdx.x; w < p.num_work && ok; w += gridDim.x) {
-        const Work k = work_item<CHECK>(p, w);
+        const Work k = work_item<CHECK>(p, CHECK ? w : w / p.sub);
         if (k.skip) continue;
         for (int c = k.c0; c < k.c1 && ok; ++c) {
           const int ns = chunk_stages(p, c);
@@ -462,13 +478,16 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   } else {
     // ---------------- epilogue: warps 2..9; lane quarter = warp % 4, column half by warp pair
     const int q = warp & 3, half = (warp - 2) >> 2;
-    double *tb = epi_buf + (size_t)(warp - 2) * (FX_EPI_BUF / 8);
-    const int rl_lo = lane >> 4, cl = lane & 15;
+    // Buffer element (row, c) of a plane at row 8 + (c ^ (row / 4) % 8): both a
+    // thread per row (the TMEM layout) and 4 rows x 8 columns per access (64-byte
+    // row pieces of global memory) are free of bank conflicts.
+    float *tb = epi_buf + (size_t)(warp - 2) * (FX_EPI_BUF / 4);
+    const int rl = lane >> 3, cl = lane & 7;
     const uint32_t taddr = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32);
     uint32_t tphase = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < p.num_work && ok; w += gridDim.x) {
-      const Work k = work_item<CHECK>(p, w);
+      const Work k = work_item<CHECK>(p, CHECK ? w : w / p.sub);
       if (k.skip) continue;
       const int row0 = k.tm * FX_BM + q * 32, colh = k.tn * FX_BN + half * 32;
       if constexpr (CHECK) {
@@ -520,37 +539,140 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             row0 + 32 <= p.M && colh + 32 <= p.N && (!p.lower || colh + 31 + p.lower_off <= row0);
         const bool live = !p.flags || row0 >= p.M || colh >= p.N ||
                           p.flags[(size_t)k.b * p.flag_stride + (size_t)(4 * k.tm + q) * p.flag_ld + 2 * k.tn + half];
-        const int ea = row0 + lane < p.M ? row_exp(p.ra, p.ra_codes, k.b * p.ra_stride + row0 + lane) : 0;
+        const int ea = row0 + lane < p.M ? row_exp(p.ra, p.ra_codes, k.b * p.ra_stride + (row0 + lane) * p.ra_mul) -
+                                              (p.ra_sub ? __ldg(p.ra_sub + row0 + lane) : 0)
+                                        : 0;
         const int ebl = colh + lane < p.N ? row_exp(p.rb, p.rb_codes, k.b * p.rb_stride + colh + lane) : 0;
-        f2x fa[16], fb[16], fc[16];
-        uint32_t late = 0;  // columns whose old value does not fit the triple: added in FP64 at the end
-        if (add) {
+        if (p.sub == 4) {
+          // Few tiles (the factorisation's chain): every CTA forms the whole tile
+          // but folds and writes only columns 8 cg .. + 7 of each warp's 32.  The
+          // whole epilogue is some 5000 instructions per warp and 60 KB of code,
+          // mostly fetched for this one pass.
+          const int cg = w & 3, col = colh + cg * FX_EPI_COLS + cl;
+          const int eb = __shfl_sync(0xffffffffu, ebl, cg * FX_EPI_COLS + cl);
+          f2x A[4], B[4], C[4];
+          uint32_t off = 0;
 #pragma unroll
-          for (int hc = 0; hc < 2; ++hc) {
-            double v[16];
+          for (int i = 0; i < 4; ++i) A[i] = B[i] = C[i] = 0ull;
+          if (add) {
+            double v[8];
 #pragma unroll
-            for (int it = 0; it < 16; ++it) {
-              const int rl = 2 * it + rl_lo, row = row0 + rl, col = colh + hc * 16 + cl;
-              const bool in = interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row));
+            for (int it = 0; it < 8; ++it) {
+              const int row = row0 + 4 * it + rl;
+              const bool in = row < p.M && col < p.N && !(p.lower && col + p.lower_off > row);
               v[it] = in ? base[(long long)row * ld + col] : 0.0;
             }
 #pragma unroll
-            for (int it = 0; it < 16; ++it) {
-              const int rl = 2 * it + rl_lo;
-              tb[rl * 16 + (cl ^ (rl & 15))] = v[it];
+            for (int it = 0; it < 8; ++it) {
+              float t0 = 0.f, t1 = 0.f, t2 = 0.f;
+              const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
+              if (!f64_to_triple(v[it], sh, t0, t1, t2)) off |= 1u << it;
+              const int at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
+              tb[at] = t0;
+              tb[at + 256] = t1;
+              tb[at + 512] = t2;
             }
             __syncwarp();
 #pragma unroll
-            for (int i = 0; i < 16; i += 2) {
-              float t0[3] = {0.f, 0.f, 0.f}, t1[3] = {0.f, 0.f, 0.f};
-              const double x0 = tb[lane * 16 + (i ^ (lane & 15))], x1 = tb[lane * 16 + ((i + 1) ^ (lane & 15))];
-              const int s0 = ea + __shfl_sync(0xffffffffu, ebl, hc * 16 + i);
-              const int s1 = ea + __shfl_sync(0xffffffffu, ebl, hc * 16 + i + 1);
-              if (!f64_to_triple(x0, s0, t0[0], t0[1], t0[2])) late |= 1u << (hc * 16 + i);
-              if (!f64_to_triple(x1, s1, t1[0], t1[1], t1[2])) late |= 1u << (hc * 16 + i + 1);
-              fa[hc * 8 + i / 2] = pk2(t0[0], t1[0]);
-              fb[hc * 8 + i / 2] = pk2(t0[1], t1[1]);
-              fc[hc * 8 + i / 2] = pk2(t0[2], t1[2]);
+            for (int i = 0; i < 8; i += 2) {
+              const int a0 = lane * FX_EPI_COLS + (i ^ (lane >> 2)), a1 = lane * FX_EPI_COLS + ((i + 1) ^ (lane >> 2));
+              A[i / 2] = pk2(tb[a0], tb[a1]);
+              B[i / 2] = pk2(tb[a0 + 256], tb[a1 + 256]);
+              C[i / 2] = pk2(tb[a0 + 512], tb[a1 + 512]);
+            }
+            __syncwarp();
+          }
+#pragma unroll 1
+          for (int c = k.c0; c < k.c1; ++c) {
+            if (!mbar_wait(tfull, tphase, abort_flag, p.wait_ns)) { ok = false; break; }
+            tphase ^= 1;
+            fence_after();
+            float g[FX_GROUPS][8];
+#pragma unroll
+            for (int grp = 0; grp < FX_GROUPS; ++grp) tmem_ld8(taddr + (uint32_t)(grp * FX_BN + cg * 8), g[grp]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int grp = 0; grp < FX_GROUPS; ++grp) pin8(g[grp]);
+            fence_before();
+            __syncwarp();
+            if (lane < FX_GROUPS) mbar_arrive(gfree0 + 8 * lane);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              f2x e, f;
+              auto part = [&](int q) {
+                const f2x x = pk2(g[q][2 * i], g[q][2 * i + 1]);
+                return NEG ? x ^ 0x8000000080000000ull : x;
+              };
+              C[i] = add2(C[i], part(6));
+              C[i] = add2(C[i], part(5));
+#pragma unroll
+              for (int q = 4; q >= 1; --q) {
+                two_sum2(B[i], part(q), B[i], e);
+                C[i] = add2(C[i], e);
+              }
+              two_sum2(A[i], part(0), A[i], e);
+              two_sum2(B[i], e, B[i], f);
+              C[i] = add2(C[i], f);
+            }
+          }
+          if (!ok) break;
+          if (!live) continue;
+#pragma unroll
+          for (int i = 0; i < 8; i += 2) {
+            const int a0 = lane * FX_EPI_COLS + (i ^ (lane >> 2)), a1 = lane * FX_EPI_COLS + ((i + 1) ^ (lane >> 2));
+            upk2(A[i / 2], tb[a0], tb[a1]);
+            upk2(B[i / 2], tb[a0 + 256], tb[a1 + 256]);
+            upk2(C[i / 2], tb[a0 + 512], tb[a1 + 512]);
+          }
+          __syncwarp();
+#pragma unroll 4
+          for (int it = 0; it < 8; ++it) {
+            const int row = row0 + 4 * it + rl, at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
+            const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
+            if (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row)) {
+              double *dst = base + (long long)row * ld + col;
+              double v = triple_to_f64(tb[at], tb[at + 256], tb[at + 512], sh);
+              if (off >> it & 1u) v = *dst + v;
+              *dst = v;
+            }
+          }
+          __syncwarp();
+          continue;
+        }
+        f2x fa[16], fb[16], fc[16];
+        uint32_t late = 0;  // values (8 per column group) that do not fit the triple: added in FP64 at the end
+        if (add) {
+          double v[4][8];  // all loads in flight before the first is used
+#pragma unroll
+          for (int cg = 0; cg < 4; ++cg)
+#pragma unroll
+            for (int it = 0; it < 8; ++it) {
+              const int row = row0 + 4 * it + rl, col = colh + cg * FX_EPI_COLS + cl;
+              const bool in = interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row));
+              v[cg][it] = in ? base[(long long)row * ld + col] : 0.0;
+            }
+#pragma unroll
+          for (int cg = 0; cg < 4; ++cg) {
+            const int eb = __shfl_sync(0xffffffffu, ebl, cg * FX_EPI_COLS + cl);
+            uint32_t off = 0;  // which of this thread's eight values do not fit
+#pragma unroll
+            for (int it = 0; it < 8; ++it) {
+              float t0 = 0.f, t1 = 0.f, t2 = 0.f;
+              const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
+              if (!f64_to_triple(v[cg][it], sh, t0, t1, t2)) off |= 1u << it;
+              const int at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
+              tb[at] = t0;
+              tb[at + 256] = t1;
+              tb[at + 512] = t2;
+            }
+            if (off) late |= off << (8 * cg);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+              const int a0 = lane * FX_EPI_COLS + (i ^ (lane >> 2)), a1 = lane * FX_EPI_COLS + ((i + 1) ^ (lane >> 2));
+              fa[cg * 4 + i / 2] = pk2(tb[a0], tb[a1]);
+              fb[cg * 4 + i / 2] = pk2(tb[a0 + 256], tb[a1 + 256]);
+              fc[cg * 4 + i / 2] = pk2(tb[a0 + 512], tb[a1 + 512]);
             }
             __syncwarp();
           }
@@ -607,30 +729,29 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (!ok) break;
         if (!live) continue;
 #pragma unroll
-        for (int hc = 0; hc < 2; ++hc) {
+        for (int cg = 0; cg < 4; ++cg) {
 #pragma unroll
-          for (int i = 0; i < 16; i += 2) {
-            float a0, a1, b0, b1, c0, c1;
-            upk2(fa[hc * 8 + i / 2], a0, a1);
-            upk2(fb[hc * 8 + i / 2], b0, b1);
-            upk2(fc[hc * 8 + i / 2], c0, c1);
-            const int s0 = ea + __shfl_sync(0xffffffffu, ebl, hc * 16 + i);
-            const int s1 = ea + __shfl_sync(0xffffffffu, ebl, hc * 16 + i + 1);
-            double v0 = triple_to_f64(a0, b0, c0, s0), v1 = triple_to_f64(a1, b1, c1, s1);
-            if (late >> (hc * 16 + i) & 3u) {
-              const double *src = base + (long long)(row0 + lane) * ld + colh + hc * 16 + i;
-              if (late >> (hc * 16 + i) & 1u) v0 = src[0] + v0;
-              if (late >> (hc * 16 + i + 1) & 1u) v1 = src[1] + v1;
-            }
-            tb[lane * 16 + (i ^ (lane & 15))] = v0;
-            tb[lane * 16 + ((i + 1) ^ (lane & 15))] = v1;
+          for (int i = 0; i < 8; i += 2) {
+            const int a0 = lane * FX_EPI_COLS + (i ^ (lane >> 2)), a1 = lane * FX_EPI_COLS + ((i + 1) ^ (lane >> 2));
+            upk2(fa[cg * 4 + i / 2], tb[a0], tb[a1]);
+            upk2(fb[cg * 4 + i / 2], tb[a0 + 256], tb[a1 + 256]);
+            upk2(fc[cg * 4 + i / 2], tb[a0 + 512], tb[a1 + 512]);
           }
           __syncwarp();
-#pragma unroll
-          for (int it = 0; it < 16; ++it) {
-            const int rl = 2 * it + rl_lo, row = row0 + rl, col = colh + hc * 16 + cl;
-            if (interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row)))
-              base[(long long)row * ld + col] = tb[rl * 16 + (cl ^ (rl & 15))];
+          const int col = colh + cg * FX_EPI_COLS + cl;
+          const int eb = __shfl_sync(0xffffffffu, ebl, cg * FX_EPI_COLS + cl);
+          // partly rolled: 32 copies of the rounding made the kernel's code so long
+          // that a launch of one tile took 34 us, mostly fetching instructions
+#pragma unroll 4
+          for (int it = 0; it < 8; ++it) {
+            const int row = row0 + 4 * it + rl, at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
+            const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
+            if (interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row))) {
+              double *dst = base + (long long)row * ld + col;
+              double v = triple_to_f64(tb[at], tb[at + 256], tb[at + 512], sh);
+              if (late >> (8 * cg + it) & 1u) v = *dst + v;
+              *dst = v;
+            }
           }
           __syncwarp();
         }
@@ -662,6 +783,12 @@ struct FxOperand {
   long long rs, ks, src_stride;
   int M, K, row_end, kpad;
   const int *rexp;
+  int rexp_mul;          // 0: one exponent for all rows, less rexp_sub[r]
+  const int *rexp_sub;
+  int *rexp_out;         // non-null (one chunk): rows are scaled by their own largest entry, exponents written here
+  int *block_out;        // non-null: largest exponent of all entries, each plus row_exps[r] and, in the rows from
+  int block_rows;        // block_rows on, the entry's kexp; less kBlockMargin
+  const int *row_exps;
   int *counts;           // per row: entries of at least 2^-5 of the row's scale (null: not counted)
   int rexp_stride, tri, tri_off;
   unsigned short *dst;
@@ -675,6 +802,12 @@ struct FxSplit {
   int codes, kexp_sign, sat;
 };
 constexpr int kCountExp = -5;
+// A block column's common scale lies 2^50 below its largest entry: entries up to
+// 2^100 above the scale and chunks down to 2^-70 below it keep all their slices
+// in FP32's range, so columns 2^-120 below the largest lose nothing and the
+// finished diagonal block may be 2^50 above it.
+constexpr int kBlockMargin = 50;
+constexpr int kNoExp = -100000;  // exponent of nothing but zeros
 template <int S, bool ABS>
 __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__ FxSplit p) {
   __shared__ double tile[8][129];
@@ -701,11 +834,13 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   if (r >= o.row_end) return;  // past the last barrier
   int E = 0;
   if (o.rexp && r < o.M) {
-    E = __ldg(o.rexp + (size_t)blockIdx.z * o.rexp_stride + r);
+    E = __ldg(o.rexp + (size_t)blockIdx.z * o.rexp_stride + (size_t)r * o.rexp_mul);
     if (p.codes) E = code_exponent(E);
+    if (E < kNoExp) E = 0;  // no entry at all
+    if (o.rexp_sub) E -= __ldg(o.rexp_sub + r);
   }
   unsigned long long mant[4];
-  int ex[4], emax = -100000;
+  int ex[4], emax = kNoExp, raw = kNoExp;
   uint32_t neg = 0, nan = 0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -721,15 +856,16 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     ex[i] = e - 1023 - E + kx;
     if (e == 0 || (e == 2047 && p.codes)) {
       mant[i] = 0;
-      ex[i] = -100000;
-    } else if (e == 2047 || ex[i] >= 30) {
+      ex[i] = kNoExp;
+    } else if (e == 2047 || (ex[i] >= 30 && !o.rexp_out)) {
       const bool isnan = e == 2047 && (u << 12) != 0;
-      if (isnan || (!p.sat && (e == 2047 || ex[i] >= 60))) nan |= 1u << i;
+      if (isnan || (!p.sat && (e == 2047 || ex[i] >= 100))) nan |= 1u << i;
       if (p.sat || nan >> i & 1u) {
         mant[i] = 1ull << 52;
         ex[i] = 30;
       }
     }
+    if (e != 0 && e != 2047) raw = max(raw, e - 1022 + (r < o.block_rows ? 0 : kx));
     emax = max(emax, ex[i]);
   }
   if (o.counts) {
@@ -740,6 +876,15 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     if (lane == 0 && n > 0) atomicAdd(o.counts + (size_t)blockIdx.z * o.rexp_stride + r, n);
   }
   emax = __reduce_max_sync(0xffffffffu, emax);
+  if (o.block_out) {
+    raw = __reduce_max_sync(0xffffffffu, raw);
+    if (lane == 0 && raw > kNoExp && r < o.M) atomicMax(o.block_out, raw + __ldg(o.row_exps + r) - kBlockMargin);
+  }
+  int shift = 0;  // the row's own exponent, when it is found here
+  if (o.rexp_out && r < o.M) {
+    shift = emax > kNoExp ? emax + 1 : 0;
+    if (lane == 0) o.rexp_out[r] = shift;
+  }
   unsigned short *dst =
       o.dst + (long long)blockIdx.z * o.dst_stride + (long long)r * o.kpad + (long long)c * FX_CHUNK + lane * 4;
   if (ABS) {  // magnitudes, rounded toward zero to BF16
@@ -767,7 +912,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   }
 #pragma unroll
   for (int pp = 0; pp < S; ++pp) {
-    const int fexp = emax + 1 - 8 * (pp + 1) + 127;
+    const int fexp = emax - shift + 1 - 8 * (pp + 1) + 127;
     const uint32_t sb = fexp >= 1 ? (uint32_t)fexp << 23 : 0u;
     uint32_t h[4];
 #pragma unroll
@@ -936,7 +1081,7 @@ size_t f64x_slice_bytes(int rows, int kchunks) {
 
 cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,
                        const int *rexp, const int *kexp, int kexp_sign, bool saturate, cudaStream_t s,
-                       int chunk_offset, int row_offset) {
+                       int chunk_offset, int row_offset, const F64xRow &row) {
   if (M <= 0 || K <= 0) return cudaSuccess;
   const int op_chunks = (K <= first) ? 1 : 1 + (K - first + FX_CHUNK - 1) / FX_CHUNK;
   const int chunks = std::min(op_chunks, out.kpad / FX_CHUNK - chunk_offset);
@@ -954,6 +1099,16 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
   o.row_end = row_offset > 0 ? M : out.rows_pad;
   o.kpad = out.kpad;
   o.rexp = rexp;
+  o.rexp_mul = row.rexp_sub ? 0 : 1;
+  o.rexp_sub = row.rexp_sub;
+  o.rexp_out = row.rexp_out;
+  o.block_out = row.block_out;
+  o.block_rows = row.block_rows;
+  o.row_exps = row.row_exps;
+  o.tri = row.tri;
+  if (row.rexp_out && chunks != 1) return cudaErrorInvalidValue;
+  if (row.block_out)
+    if (cudaError_t e = cudaMemsetAsync(row.block_out, 0x80, sizeof(int), s); e != cudaSuccess) return e;
   o.dst = (unsigned short *)out.base + (long long)row_offset * out.kpad + (long long)chunk_offset * FX_CHUNK;
   o.plane = (long long)out.rows_pad * out.kpad;
   p.first = first;
@@ -969,7 +1124,7 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
 
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
-                      double *partial, int *err, cudaStream_t s, int max_ctas, int kdepth, int max_items) {
+                      double *partial, int *err, cudaStream_t s, int max_ctas, int kdepth, int max_items, const int *ra_sub) {
   if (M <= 0 || N <= 0 || chunks <= 0) return cudaSuccess;
   if (kdepth <= 0) kdepth = FX_CHUNK;
   if (kdepth > FX_CHUNK || kdepth % FX_BK) return cudaErrorInvalidValue;
@@ -994,6 +1149,8 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
   p.num_work = p.per_batch * p.splits;
   p.accumulate = 1;
   p.ra = ra;
+  p.ra_mul = ra_sub ? 0 : 1;
+  p.ra_sub = ra_sub;
   p.rb = rb;
   p.C = C;
   p.ldc = ldc;
@@ -1006,6 +1163,11 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
                            : (M >= N ? 0.5 * (double)N * (N + 1) + (double)(M - N) * N : 0.5 * (double)M * (M + 1));
   const double flops = 2.0 * mn * (double)chunks * kdepth * 28.0;  // 28 slice products
   const double bytes = 16.0 * mn + (double)(M + N) * chunks * kdepth * 2 * kF64xSlices;
+  p.sub = 1;
+  if (max_ctas == 0 && 4 * p.num_work <= sm_count()) {
+    p.sub = 4;
+    p.num_work *= 4;
+  }
   int grid = std::min(p.num_work, max_ctas > 0 ? std::min(max_ctas, sm_count()) : sm_count());
   if (max_items > 0) grid = std::max(grid, (p.num_work + max_items - 1) / max_items);
   cudaError_t e = launch_product<kF64xSlices, true, false>(ma, mb, p, grid, flops, bytes, s);
@@ -1014,6 +1176,89 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 8.0 * (p.splits + 2) * mn, s,
              launch_k(f64x_reduce_kernel, (unsigned)((total + 255) / 256), 256, 0, s, M, N, p.splits, (const double *)partial,
                       C, ldc, lower ? 1 : 0, 1, (const unsigned char *)nullptr, 0));
+  return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------ scales of the factorisation and its adjoint
+namespace {
+
+// e_i with K_ii < 4^e_i (|L_ij| <= sqrt(K_ii) < 2^e_i); 0 where K_ii is no
+// positive normal number (the factorisation fails there).
+__global__ void diag_exps_kernel(int n, const double *K, long long ldk, int *rexp) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const unsigned long long u = (unsigned long long)__double_as_longlong(K[(long long)i * ldk + i]);
+  const int e = (int)(u >> 52);  // the sign bit too: negative entries are above 2047
+  rexp[i] = (e > 0 && e < 2047) ? (e - 1022 + 1) >> 1 : 0;
+}
+// rexp[i]: exponent E, 2^E above the largest entry of row i of the lower triangle.  A warp per row.
+__global__ void __launch_bounds__(256) lower_row_exps_kernel(int n, const double *L, long long ldl, int *rexp) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;
+  int m = 0;
+#pragma unroll 4
+  for (int k = lane; k <= i; k += 32) {
+    const int e = (int)((unsigned long long)__double_as_longlong(L[(long long)i * ldl + k]) >> 52) & 0x7FF;
+    m = max(m, e == 2047 ? 0 : e);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) rexp[i] = m > 0 ? m - 1022 : 0;
+}
+// cexp[c]: the same for column c of the rows scaled by 2^-rexp.  32 columns and
+// 64 rows per CTA; cexp holds large negative numbers on entry.
+__global__ void __launch_bounds__(256)
+lower_col_exps_kernel(int n, const double *L, long long ldl, const int *rexp, int *cexp) {
+  const int c = blockIdx.x * 32 + (threadIdx.x & 31), t0 = blockIdx.y * 64;
+  if (c >= n || t0 + 63 < blockIdx.x * 32) return;
+  int m = kNoExp;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int t = t0 + (threadIdx.x >> 5) + 8 * q;
+    if (t < n && t >= c) {
+      const int e = (int)((unsigned long long)__double_as_longlong(L[(long long)t * ldl + c]) >> 52) & 0x7FF;
+      if (e != 0 && e != 2047) m = max(m, e - 1022 - __ldg(rexp + t));
+    }
+  }
+  if (m > kNoExp) atomicMax(&cexp[c], m);
+}
+// *out: 2^(*out + kBlockMargin) above the largest entry of the nb x nb block with row r scaled by 2^rexp[r].
+__global__ void __launch_bounds__(256)
+block_exp_kernel(int nb, const double *A, long long lda, const int *rexp, int *out) {
+  __shared__ int red[8];
+  int m = kNoExp;
+  for (int idx = threadIdx.x; idx < nb * nb; idx += 256) {
+    const int r = idx / nb, c = idx - r * nb;
+    const int e = (int)((unsigned long long)__double_as_longlong(A[(long long)r * lda + c]) >> 52) & 0x7FF;
+    if (e != 0 && e != 2047) m = max(m, e - 1022 + rexp[r]);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+    *out = m > kNoExp ? m - kBlockMargin : 0;
+  }
+}
+
+}  // namespace
+
+cudaError_t f64x_diag_exps(int n, const double *K, long long ldk, int *rexp, cudaStream_t s) {
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 12.0 * n, s,
+             launch_k(diag_exps_kernel, (unsigned)((n + 255) / 256), 256, 0, s, n, K, ldk, rexp));
+  return cudaGetLastError();
+}
+cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, int *cexp, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(cexp, 0x80, (size_t)n * sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 4.0 * n * (n + 1.0), s,
+             launch_k(lower_row_exps_kernel, (unsigned)((n + 7) / 8), 256, 0, s, n, L, ldl, rexp));
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 4.0 * n * (n + 1.0), s,
+             launch_k(lower_col_exps_kernel, dim3((unsigned)((n + 31) / 32), (unsigned)((n + 63) / 64)), 256, 0, s, n, L,
+                      ldl, (const int *)rexp, cexp));
+  return cudaGetLastError();
+}
+cudaError_t f64x_block_exp(int nb, const double *A, long long lda, const int *rexp, int *out, cudaStream_t s) {
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 8.0 * nb * nb, s, launch_k(block_exp_kernel, 1, 256, 0, s, nb, A, lda, rexp, out));
   return cudaGetLastError();
 }
 
@@ -1088,6 +1333,7 @@ cudaError_t one_panel(const Gemm &g, const Panels &pn, int mo, int no, int ko, c
     o.row_end = pad;
     o.kpad = kpad;
     o.rexp = code;
+    o.rexp_mul = 1;
     o.rexp_stride = pad;
     o.tri = tri;  // element (r, k) is zero for k + ko < r + panel offset (1) or > (2)
     o.tri_off = tri_off;
@@ -1150,6 +1396,7 @@ cudaError_t one_panel(const Gemm &g, const Panels &pn, int mo, int no, int ko, c
   p.accumulate = (ko > 0 || g.beta != 0.0) ? 1 : 0;
   p.ra = cA;
   p.rb = cB;
+  p.ra_mul = 1;
   p.ra_codes = p.rb_codes = 1;
   p.ra_stride = mpad;
   p.rb_stride = npad;
@@ -1172,8 +1419,14 @@ cudaError_t one_panel(const Gemm &g, const Panels &pn, int mo, int no, int ko, c
   e = launch_product<1, false, true>(ma1, mb1, p, grid, 2.0 * mnk, 0.0, s);
   if (e != cudaSuccess) return e;
   p.partial = p.splits > 1 ? partial : nullptr;
-  e = g.alpha < 0.0 ? launch_product<GX_S, true, false>(ma, mb, p, grid, 72.0 * mnk, 0.0, s)
-                    : launch_product<GX_S, false, false>(ma, mb, p, grid, 72.0 * mnk, 0.0, s);
+  p.sub = 1;
+  if (4 * p.num_work <= sm_count()) {
+    p.sub = 4;
+    p.num_work *= 4;
+  }
+  const int pgrid = std::min(p.num_work, sm_count());
+  e = g.alpha < 0.0 ? launch_product<GX_S, true, false>(ma, mb, p, pgrid, 72.0 * mnk, 0.0, s)
+                    : launch_product<GX_S, false, false>(ma, mb, p, pgrid, 72.0 * mnk, 0.0, s);
   if (e != cudaSuccess) return e;
   if (p.splits > 1) {
     const long long total = (long long)M * N;

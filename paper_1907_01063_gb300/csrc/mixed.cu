@@ -1,7 +1,8 @@
 // Mixed-precision blocked Cholesky and blocked adjoint (precision GPC_MIXED).
 //
-// Same block algorithms as the FP64 path (Section 3.3; see chol.cu), with the
-// O(n^3) products moved to split-BF16 tensor-core products (ozaki.cu):
+// Same block algorithms as chol.cu (Section 3.3), with the O(n^3) products
+// moved to split-BF16 tensor-core products (ozaki.cu).  The FP64 path runs the
+// same code on FP64 storage with the FP64-accurate products of f64x.cu (f64).
 //   forward: the trailing update A22 -= L21 L21^T;
 //   adjoint: Bbar -= Cbar R, Dbar -= Cbar^T C and Rbar -= [Dbar; Cbar]^T [R; B].
 // The diagonal-block factors, their inverses, the panel solves and the Dbar
@@ -40,6 +41,7 @@ struct MixWs {
   double *inv, *m, *t, *panel, *scratch;  // FP64 pieces (scratch doubles as the split-K partials)
   void *sc, *sdc, *lt;                    // slices: panel rows, block-column columns, L^T
   void *grp, *tmp;                        // factorisation: two group buffers, per-step temporaries
+  int *rexp, *cexp, *xexp, *bexp;         // FP64 path: scale exponents (rows of L, columns, panel rows, block column)
 };
 constexpr int kMaxDefer = 8;
 int defer_depth() { return std::max(1, std::min(tuning().mixed_defer, kMaxDefer)); }
@@ -73,7 +75,13 @@ cudaError_t aux_for_device(Aux **out) {
 size_t scratch_bytes() { return std::max(gemm_f64_scratch_bytes(), kPartialCap); }
 int nchunks(int n) { return std::max(1, (n + MB - 1) / MB); }
 
-MixWs carve(void *ws, int n, bool adjoint) {
+// Slices per operand: five on the mixed path (ozaki.cu), seven on the FP64 path (f64x.cu).
+size_t sbytes(int rows, int kchunks, bool f64) {
+  return f64 ? f64x_slice_bytes(rows, kchunks) : slice_bytes(rows, kchunks);
+}
+size_t exps_bytes(int n) { return align_up((size_t)n * sizeof(int), 256); }
+
+MixWs carve(void *ws, int n, bool adjoint, bool f64) {
   char *p = (char *)ws;
   MixWs w{};
   w.inv = (double *)p; p += (size_t)nchunks(n) * b2();  // every diagonal-block inverse
@@ -81,25 +89,29 @@ MixWs carve(void *ws, int n, bool adjoint) {
   w.t = (double *)p; p += b2();
   w.panel = (double *)p; p += align_up((size_t)n * MB * sizeof(double), 256);
   w.scratch = (double *)p; p += scratch_bytes();
-  w.sc = p; p += 2 * slice_bytes(n, 1);  // two buffers: the next panel's slices while the last are in use
+  w.sc = p; p += 2 * sbytes(n, 1, f64);  // two buffers: the next panel's slices while the last are in use
   if (adjoint) {
-    w.sdc = p; p += slice_bytes(MB, nchunks(n));
-    w.lt = p; p += slice_bytes(n, nchunks(n));
+    w.sdc = p; p += sbytes(MB, nchunks(n), f64);
+    w.lt = p; p += sbytes(n, nchunks(n), f64);
   } else {
-    w.grp = p; p += 2 * slice_bytes(n, defer_depth());
-    w.tmp = p; p += slice_bytes(n, 1);
+    w.grp = p; p += 2 * sbytes(n, defer_depth(), f64);
+    w.tmp = p; p += sbytes(n, 1, f64);
   }
+  w.rexp = (int *)p; p += exps_bytes(n);
+  w.cexp = (int *)p; p += exps_bytes(n);
+  w.xexp = (int *)p; p += exps_bytes(n);
+  w.bexp = (int *)p;
   return w;
 }
 
 }  // namespace
 
-size_t mixed_workspace_bytes(int n) {
+size_t mixed_workspace_bytes(int n, bool f64) {
   n = std::max(n, 1);
   const size_t common = ((size_t)nchunks(n) + 2) * b2() + align_up((size_t)n * MB * sizeof(double), 256) +
-                        scratch_bytes() + 2 * slice_bytes(n, 1) + 1024;
-  const size_t adj = slice_bytes(MB, nchunks(n)) + slice_bytes(n, nchunks(n));
-  const size_t fwd = 2 * slice_bytes(n, defer_depth()) + slice_bytes(n, 1);
+                        scratch_bytes() + 2 * sbytes(n, 1, f64) + 3 * exps_bytes(n) + 256 + 1024;
+  const size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64);
+  const size_t fwd = 2 * sbytes(n, defer_depth(), f64) + sbytes(n, 1, f64);
   return common + std::max(adj, fwd);
 }
 
@@ -125,15 +137,35 @@ size_t mixed_workspace_bytes(int n) {
 // region -- and group buffers alternate, so a split never overwrites slices
 // still being read.  D = 1 is the one-block lookahead (rest of every step in
 // the background).
-cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s) {
-  MixWs w = carve(ws, n, false);
+//
+// f64 (precision GPC_FP64): the same schedule with the products of f64x.cu on
+// FP64 storage.  Row i of L is scaled by 2^-e_i, e_i from K's diagonal
+// (|L_ij| <= sqrt(K_ii)); the slices' error is then relative to
+// sqrt(K_ii K_jj), the form of the FP64 factorisation's own error bound.
+cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cudaStream_t s, bool f64) {
+  MixWs w = carve(ws, n, false, f64);
+  if (f64) TRY(f64x_diag_exps(n, L, ldl, w.rexp, s));
+  const bool df = !f64;  // the matrices the products update are in double-float storage
+  // slices of M rows of L, the first at global row `row`, K columns
+  auto split = [&](const double *src, int M, int K, const SliceBuf &out, int row, int chunk = 0, int roff = 0) {
+    return f64 ? f64x_split(src, ldl, 1, M, K, K, out, w.rexp + row, nullptr, 0, true, s, chunk, roff)
+               : split_operand(src, ldl, 1, M, K, K, out, s, chunk, roff);
+  };
+  // C -= A B^T; C's first row and column are global rows gi and gj of L
+  auto product = [&](const SliceBuf &A, int ar, const SliceBuf &B, int br, int M, int N, int chunks, bool lower,
+                     double *C, int gi, int gj, cudaStream_t st, int ctas, int kdepth, int items) {
+    int *e = info ? info + 1 : nullptr;
+    return f64 ? f64x_gemm(A, ar, 0, B, br, 0, M, N, chunks, lower, w.rexp + gi, w.rexp + gj, C, ldl, 1, nullptr, e,
+                           st, ctas, kdepth, items)
+               : ozaki_gemm(A, ar, 0, B, br, 0, M, N, chunks, lower, -1.0f, (float2 *)C, ldl, 1, nullptr, e, st, ctas,
+                            kdepth, items);
+  };
   Aux *aux = nullptr;
   TRY(aux_for_device(&aux));
   const int D = defer_depth();
   const int nbc = nchunks(n);
   const int bg_ctas = std::max(1, sm_count() - std::max(0, std::min(tuning().mixed_free_sms, sm_count() / 2)));
   const int bg_items = std::max(0, tuning().mixed_cta_items);
-  int *err = info ? info + 1 : nullptr;
   // the caller's stream carries the critical chain: its launches go first
   PriorityScope chain(tuning().mixed_priority ? greatest_priority() : 0);
   bool strip_pending = false, rest_pending = false;
@@ -153,9 +185,8 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
     if (e == cudaSuccess) e = cudaStreamWaitEvent(aux->st, aux->ev_fork, 0);
     PriorityScope background(0);
     if (e == cudaSuccess && c1 > c0)
-      e = ozaki_gemm(slabs.G, c0 - slabs.p0, 0, slabs.G, c0 - slabs.p0, 0, n - c0, c1 - c0, slabs.chunks, true,
-                     -1.0f, (float2 *)(L + (long long)c0 * ldl + c0), ldl, 1, nullptr, err, aux->st, bg_ctas, 0,
-                     bg_items);
+      e = product(slabs.G, c0 - slabs.p0, slabs.G, c0 - slabs.p0, n - c0, c1 - c0, slabs.chunks, true,
+                  L + (long long)c0 * ldl + c0, c0, c0, aux->st, bg_ctas, 0, bg_items);
     if (e == cudaSuccess && slabs.next == slabs.count) e = cudaEventRecord(aux->ev_rest, aux->st);
     return e;
   };
@@ -164,7 +195,7 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
     const int p0 = g * D * MB, p1 = std::min(n, p0 + D * MB);
     const int k0 = bc * MB, nb = std::min(MB, n - k0), m = n - k0 - nb;
     double *A11 = L + (long long)k0 * ldl + k0;
-    SliceBuf G = slice_view((char *)w.grp + (size_t)(g & 1) * slice_bytes(n, D), n - p0, D);
+    SliceBuf G = slice_view((char *)w.grp + (size_t)(g & 1) * sbytes(n, D, f64), n - p0, D);
     // ---- FP64 steps of this block column (its updates are all applied)
     if (nb > MH) {
       // Two 64-wide steps: factor and solve the left half, update the right
@@ -175,30 +206,29 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
       const int hb = nb - MH;
       double *Aba = A11 + (long long)MH * ldl;  // right half's rows, left half's columns
       double *Ab = Aba + MH;                    // right half's diagonal block
-      const size_t sb_small = slice_bytes(MH, 1);
-      SliceBuf Sba = slice_view((char *)w.tmp + slice_bytes(n, 1) - sb_small, hb, 1);
-      TRY(potrf_diag(MH, A11, ldl, info, k0, s, true));
-      TRY(trsm_rows(hb, MH, Aba, ldl, A11, ldl, 0, s, true));
-      TRY(split_operand(Aba, ldl, 1, hb, MH, MH, Sba, s));
-      TRY(ozaki_gemm(Sba, 0, 0, Sba, 0, 0, hb, hb, 1, true, -1.0f, (float2 *)Ab, ldl, 1, nullptr, err, s, 0, MH));
-      TRY(potrf_diag(hb, Ab, ldl, info, k0 + MH, s, true));
+      const size_t sb_small = sbytes(MH, 1, f64);
+      SliceBuf Sba = slice_view((char *)w.tmp + sbytes(n, 1, f64) - sb_small, hb, 1);
+      TRY(potrf_diag(MH, A11, ldl, info, k0, s, df));
+      TRY(trsm_rows(hb, MH, Aba, ldl, A11, ldl, 0, s, df));
+      TRY(split(Aba, hb, MH, Sba, k0 + MH));
+      TRY(product(Sba, 0, Sba, 0, hb, hb, 1, true, Ab, k0 + MH, k0 + MH, s, 0, MH, 0));
+      TRY(potrf_diag(hb, Ab, ldl, info, k0 + MH, s, df));
       if (m > 0) {
         double *Ca = A11 + (long long)nb * ldl;  // panel rows below the diagonal block, left half
-        TRY(trsm_rows(m, MH, Ca, ldl, A11, ldl, 0, s, true));
+        TRY(trsm_rows(m, MH, Ca, ldl, A11, ldl, 0, s, df));
         SliceBuf Sc = slice_view(w.tmp, m, 1);
-        TRY(split_operand(Ca, ldl, 1, m, MH, MH, Sc, s));
-        TRY(ozaki_gemm(Sc, 0, 0, Sba, 0, 0, m, hb, 1, false, -1.0f, (float2 *)(Ca + MH), ldl, 1, nullptr, err, s, 0,
-                       MH));
-        TRY(trsm_rows(m, hb, Ca + MH, ldl, Ab, ldl, 0, s, true));
+        TRY(split(Ca, m, MH, Sc, k0 + nb));
+        TRY(product(Sc, 0, Sba, 0, m, hb, 1, false, Ca + MH, k0 + nb, k0 + MH, s, 0, MH, 0));
+        TRY(trsm_rows(m, hb, Ca + MH, ldl, Ab, ldl, 0, s, df));
       }
     } else {
-      TRY(potrf_diag(nb, A11, ldl, info, k0, s, true));
-      if (m > 0) TRY(trsm_rows(m, nb, A11 + (long long)nb * ldl, ldl, A11, ldl, 0, s, true));  // L21 = A21 L11^{-T}
+      TRY(potrf_diag(nb, A11, ldl, info, k0, s, df));
+      if (m > 0) TRY(trsm_rows(m, nb, A11 + (long long)nb * ldl, ldl, A11, ldl, 0, s, df));  // L21 = A21 L11^{-T}
     }
     if (m <= 0) continue;
     // ---- this block column's slices: chunk t of the group buffer, rows from k0 + nb
     const int r0 = k0 + nb - p0;  // first panel row, relative to the group
-    TRY(split_operand(A11 + (long long)nb * ldl, ldl, 1, m, nb, nb, G, s, t, r0));
+    TRY(split(A11 + (long long)nb * ldl, m, nb, G, k0 + nb, t, r0));
     // ---- next block column minus all of the group's block columns so far
     const int nb2 = std::min(MB, m);
     const bool last_in_group = (k0 + nb == p1);
@@ -211,8 +241,7 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
       TRY(cudaStreamWaitEvent(s, aux->ev_rest, 0));
       rest_pending = false;
     }
-    TRY(ozaki_gemm(G, r0, 0, G, r0, 0, m, nb2, t + 1, true, -1.0f, (float2 *)(A11 + (long long)nb * ldl + nb), ldl,
-                   1, nullptr, err, s));
+    TRY(product(G, r0, G, r0, m, nb2, t + 1, true, A11 + (long long)nb * ldl + nb, k0 + nb, k0 + nb, s, 0, 0, 0));
     if (rest_pending && slabs.next < slabs.count) TRY(launch_slab());
     if (!last_in_group || m <= nb2) continue;
     // ---- the group's deferred update of the columns right of the next block column
@@ -223,9 +252,8 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
     TRY(cudaStreamWaitEvent(aux->st, aux->ev_fork, 0));
     PriorityScope background(0);
     if (p2 > q1) {
-      TRY(ozaki_gemm(G, q1 - p0, 0, G, q1 - p0, 0, n - q1, p2 - q1, chunks, true, -1.0f,
-                     (float2 *)(L + (long long)q1 * ldl + q1), ldl, 1, nullptr, err, aux->st, bg_ctas, 0,
-                     bg_items));
+      TRY(product(G, q1 - p0, G, q1 - p0, n - q1, p2 - q1, chunks, true, L + (long long)q1 * ldl + q1, q1, q1,
+                  aux->st, bg_ctas, 0, bg_items));
       TRY(cudaEventRecord(aux->ev_split, aux->st));
       strip_pending = true;
     }
@@ -256,14 +284,30 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
   return trtri_batched(n, L, ldl, std::min(MB, n), MB, w.inv, s);
 }
 
+// f64 (precision GPC_FP64): the same sweep with the products of f64x.cu on FP64
+// storage.  The rows of L are equilibrated by powers of two first, L' = S^-1 L
+// with S = diag(2^s_t), 2^s_t above row t's largest entry: every product sums
+// over rows t of L (or columns t of the adjoint), L's entries entering with
+// 2^-s_t and the adjoint's with 2^s_t, so a diagonal scaling of K changes no
+// rounding.  Operand rows are then scaled by their largest entry: columns of
+// L' (cexp), panel rows of the adjoint (xexp, found by the split itself) and, for
+// its columns c, the block column's largest entry in equilibrated units less s_c
+// (bexp; each chunk of 128 keeps its own exponent, so this one only has to keep
+// FP32's range).
 cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A, long long lda, void *ws,
-                               int *err, cudaStream_t s) {
-  MixWs w = carve(ws, n, true);
+                               int *err, cudaStream_t s, bool f64) {
+  MixWs w = carve(ws, n, true, f64);
+  const bool df = !f64;
   const int nblk = nchunks(n);
   const int first = n - (nblk - 1) * MB;  // rows in the top-left block
   // L^T slices: operand row t = column t of L, K = rows of L, chunked like the sweep's blocks.
   SliceBuf LT = slice_view(w.lt, n, nblk);
-  TRY(split_operand(L, 1, ldl, n, n, first, LT, s));
+  if (f64) {
+    TRY(f64x_lower_exps(n, L, ldl, w.rexp, w.cexp, s));
+    TRY(f64x_split(L, 1, ldl, n, n, first, LT, w.cexp, w.rexp, -1, false, s, 0, 0, F64xRow{nullptr, nullptr, nullptr, 0, 1, nullptr}));
+  } else {
+    TRY(split_operand(L, 1, ldl, n, n, first, LT, s));
+  }
   TRY(trtri_batched(n, L, ldl, first, MB, w.inv, s));  // independent of the sweep: one launch
   Aux *aux = nullptr;
   TRY(aux_for_device(&aux));
@@ -294,38 +338,67 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
         const int hb = nb - MH;
         double *Cb = Cbar + MH;
         const double *Dba = D + (long long)MH * ldl;
-        TRY(trsm_rows(m, hb, Cb, lda, Dba + MH, ldl, 1, s, true));
-        SliceBuf SX = slice_view((char *)w.sc + slice_bytes(n, 1), m, 1);
+        TRY(trsm_rows(m, hb, Cb, lda, Dba + MH, ldl, 1, s, df));
+        SliceBuf SX = slice_view((char *)w.sc + sbytes(n, 1, f64), m, 1);
         SliceBuf SD = slice_view(w.sdc, MH, 1);
-        TRY(split_operand(Cb, lda, 1, m, hb, hb, SX, s));
-        TRY(split_operand(Dba, 1, ldl, MH, hb, hb, SD, s));  // row c, K index t: Dba[t][c]
-        TRY(ozaki_gemm(SX, 0, 0, SD, 0, 0, m, MH, 1, false, -1.0f, (float2 *)Cbar, lda, 1, nullptr, err, s, 0,
-                       (hb + 31) / 32 * 32));
-        TRY(trsm_rows(m, MH, Cbar, lda, D, ldl, 1, s, true));
+        const int depth = (hb + 31) / 32 * 32;
+        if (f64) {
+          TRY(f64x_split(Cb, lda, 1, m, hb, hb, SX, nullptr, w.rexp + j + MH, 1, false, s, 0, 0,
+                         F64xRow{w.xexp, nullptr, nullptr, 0, 0, nullptr}));
+          TRY(f64x_split(Dba, 1, ldl, MH, hb, hb, SD, w.cexp + j, w.rexp + j + MH, -1, false, s));
+          TRY(f64x_gemm(SX, 0, 0, SD, 0, 0, m, MH, 1, false, w.xexp, w.cexp + j, Cbar, lda, 1, nullptr, err, s, 0,
+                        depth));
+        } else {
+          TRY(split_operand(Cb, lda, 1, m, hb, hb, SX, s));
+          TRY(split_operand(Dba, 1, ldl, MH, hb, hb, SD, s));  // row c, K index t: Dba[t][c]
+          TRY(ozaki_gemm(SX, 0, 0, SD, 0, 0, m, MH, 1, false, -1.0f, (float2 *)Cbar, lda, 1, nullptr, err, s, 0,
+                         depth));
+        }
+        TRY(trsm_rows(m, MH, Cbar, lda, D, ldl, 1, s, df));
       } else {
-        TRY(trsm_rows(m, nb, Cbar, lda, D, ldl, 1, s, true));  // Cbar <- Cbar D^{-1} (FP64)
+        TRY(trsm_rows(m, nb, Cbar, lda, D, ldl, 1, s, df));  // Cbar <- Cbar D^{-1} (FP64)
       }
-      // Dbar -= Cbar^T C on slices, Dbar still in double-float storage: the
-      // columns of Cbar (K = rows k..n) fill chunks 1.. of the block column's
-      // slices; C^T is rows j..k of the L^T slices.
-      TRY(split_operand(Cbar, 1, lda, nb, m, MB, SDC, s, 1));
+      // Dbar -= Cbar^T C on slices (mixed: Dbar still in double-float storage):
+      // the columns of Cbar (K = rows k..n) fill chunks 1.. of the block
+      // column's slices; C^T is rows j..k of the L^T slices.
+      SliceBuf SC = slice_view(w.sc, f64 ? m + nb : m, 1);
+      if (f64) {
+        // panel rows of the block column with their exponents, and bexp in
+        // equilibrated units: Kbar' = S Kbar S for Cbar, Lbar' = S Lbar for Dbar's
+        // rows, which only count here
+        TRY(f64x_split(Dbar, lda, 1, m + nb, nb, nb, SC, nullptr, w.rexp + j, 1, false, s, 0, 0,
+                       F64xRow{w.xexp, w.bexp, w.rexp + j, nb, 0, nullptr}));
+        TRY(f64x_split(Cbar, 1, lda, nb, m, MB, SDC, w.bexp, w.rexp + k, 1, false, s, 1, 0,
+                       F64xRow{nullptr, nullptr, nullptr, 0, 0, w.rexp + j}));
+      } else {
+        TRY(split_operand(Cbar, 1, lda, nb, m, MB, SDC, s, 1));
+      }
       const int dch = chunks - 1;
       int dsplits = std::max(1, std::min(dch, (2 * sm_count() + 1) / 2));
       while (dsplits > 1 && ozaki_partial_bytes(nb, nb, dsplits) > kPartialCap) --dsplits;
-      TRY(ozaki_gemm(SDC, 0, MB, LT, j, (ib + 1) * MB, nb, nb, dch, true, -1.0f, (float2 *)Dbar, lda, dsplits,
-                     (float2 *)w.scratch, err, s));
-      if (j > 0) {  // Bbar -= Cbar R on slices (Bbar in double-float storage)
-        SliceBuf SC = slice_view(w.sc, m, 1);
-        TRY(split_operand(Cbar, lda, 1, m, nb, nb, SC, s));
+      if (f64)
+        TRY(f64x_gemm(SDC, 0, MB, LT, j, (ib + 1) * MB, nb, nb, dch, true, w.bexp, w.cexp + j, Dbar, lda, dsplits,
+                      w.scratch, err, s, 0, 0, 0, w.rexp + j));
+      else
+        TRY(ozaki_gemm(SDC, 0, MB, LT, j, (ib + 1) * MB, nb, nb, dch, true, -1.0f, (float2 *)Dbar, lda, dsplits,
+                       (float2 *)w.scratch, err, s));
+      if (j > 0) {  // Bbar -= Cbar R on slices
+        if (!f64) TRY(split_operand(Cbar, lda, 1, m, nb, nb, SC, s));
         TRY(cudaEventRecord(aux->ev_split, s));
         TRY(cudaStreamWaitEvent(aux->st, aux->ev_split, 0));
-        TRY(ozaki_gemm(SC, 0, 0, LT, 0, ib * MB, m, j, 1, false, -1.0f, (float2 *)(A + (long long)k * lda),
-                       lda, 1, nullptr, err, aux->st, sm_count() - side));
+        if (f64)
+          TRY(f64x_gemm(SC, nb, 0, LT, 0, ib * MB, m, j, 1, false, w.xexp + nb, w.cexp, A + (long long)k * lda, lda, 1,
+                        nullptr, err, aux->st, sm_count() - side));
+        else
+          TRY(ozaki_gemm(SC, 0, 0, LT, 0, ib * MB, m, j, 1, false, -1.0f, (float2 *)(A + (long long)k * lda),
+                         lda, 1, nullptr, err, aux->st, sm_count() - side));
         TRY(cudaEventRecord(aux->ev_rest, aux->st));
         bbar_pending = true;
       }
+    } else if (f64) {
+      TRY(f64x_block_exp(nb, Dbar, lda, w.rexp + j, w.bexp, s));
     }
-    TRY(from_df_rect(nb, nb, Dbar, lda, s));
+    if (!f64) TRY(from_df_rect(nb, nb, Dbar, lda, s));
     {
       Gemm p;  // M = sym(tril(D^T Dbar))
       p.M = nb; p.N = nb; p.K = nb;
@@ -355,12 +428,20 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
       TRY(gemm_f64(d, w.scratch, s));
     }
     if (j > 0) {  // Rbar -= [Dbar; Cbar]^T [R; B] on slices (Rbar in double-float storage)
-      TRY(split_operand(Dbar, 1, lda, nb, nb, nb, SDC, s, 0));  // chunk 0: the finished Dbar
+      if (f64)  // chunk 0: the finished Dbar
+        TRY(f64x_split(Dbar, 1, lda, nb, nb, nb, SDC, w.bexp, w.rexp + j, 1, false, s, 0, 0,
+                       F64xRow{nullptr, nullptr, nullptr, 0, 0, w.rexp + j}));
+      else
+        TRY(split_operand(Dbar, 1, lda, nb, nb, nb, SDC, s, 0));
       const int tiles = (j + 63) / 64;
       int splits = std::max(1, std::min(chunks, (2 * sm_count() + tiles - 1) / tiles));
       while (splits > 1 && ozaki_partial_bytes(nb, j, splits) > kPartialCap) --splits;
-      TRY(ozaki_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, -1.0f, (float2 *)(A + (long long)j * lda),
-                     lda, splits, (float2 *)w.scratch, err, s));
+      if (f64)
+        TRY(f64x_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, w.bexp, w.cexp, A + (long long)j * lda, lda,
+                      splits, w.scratch, err, s, 0, 0, 0, w.rexp + j));
+      else
+        TRY(ozaki_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, -1.0f, (float2 *)(A + (long long)j * lda),
+                       lda, splits, (float2 *)w.scratch, err, s));
     }
     TRY(phi_block(nb, Dbar, lda, s));
     if (bbar_pending) {

@@ -5,12 +5,15 @@ most K 2^-53 S (S = sum |a||b|, first order) and so is the product under test
 (its own bound is no larger than the FP64 chain's), so they differ by at most
 2 (K + 2) 2^-53 S.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 import paper_1907_01063_gb300 as gp
 from oracle import oracle as O
+from paper_1907_01063_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +88,97 @@ def test_reverse_mode():
     Ab, Bb = gp.gemm_adjoint(*(torch.as_tensor(x, device="cuda") for x in (A, B, Cb)))
     check(Ab.cpu().numpy(), Cb, B.T.copy())
     check(Bb.cpu().numpy(), A.T.copy(), Cb)
+
+
+# ---- the factorisation and its adjoint on slices (orders from 256)
+def dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+
+
+def problem(n, seed=0):
+    X = W.gp_inputs(n, 3, seed)
+    return O.se_cov(X, 1.0, 1.0, 0.3, 1e-6), W.random_lower(n, seed + 1)
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("n", [256, 257, 319, 384, 449, 640, 769, 1025])
+def test_factor_and_adjoint_match_the_oracle(n):
+    # 1e-12: condition about 1e4 times the unit roundoff, as for the FP64 kernels
+    K, Wt = problem(n, n)
+    L = O.chol(K)
+    assert rel(gp.chol(dev(K)).cpu().numpy(), L) <= 1e-12
+    assert rel(gp.chol_adjoint(dev(L), dev(Wt)).cpu().numpy(), O.chol_adjoint(L, Wt)) <= 1e-12
+
+
+def test_minimal_workspace_takes_the_fp64_kernels():
+    n = 500
+    K, Wt = problem(n, 3)
+    b = ctypes.c_size_t()
+    assert gp.capi.gpc_workspace_min_size(n, gp.GPC_FP64, ctypes.byref(b)) == gp.GPC_OK
+    assert b.value < gp.workspace_size(n)
+    ws = torch.empty(b.value, dtype=torch.uint8, device="cuda")
+    L = O.chol(K)
+    assert rel(gp.chol(dev(K), ws=ws).cpu().numpy(), L) <= 1e-12
+    assert rel(gp.chol_adjoint(dev(L), dev(Wt), ws=ws).cpu().numpy(), O.chol_adjoint(L, Wt)) <= 1e-12
+    y = W.gp_inputs(n, 1, 5)[:, 0]
+    assert rel(gp.gp_lml(dev(K), dev(y), ws=ws)["alpha"].cpu().numpy(), O.gp_lml(K, y)["alpha"]) <= 1e-11
+
+
+@pytest.mark.parametrize("spread", [0, 12, 40])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -660, 2.0 ** 660])
+def test_diagonal_scaling_changes_nothing(spread, scale):
+    # K -> D K D with powers of two: L -> D L and Kbar -> D^-1 Kbar D^-1 exactly, so
+    # the slices must see the same digits
+    n = 450
+    K, Wt = problem(n, 7)
+    d = 2.0 ** np.round(spread * np.random.default_rng(1).standard_normal(n)) * np.sqrt(scale)
+    L = gp.chol(dev(K)).cpu().numpy()
+    G = gp.chol_adjoint(dev(L), dev(Wt)).cpu().numpy()
+    L2 = gp.chol(dev(d[:, None] * K * d[None, :])).cpu().numpy()
+    assert np.abs(L2 / d[:, None] - L).max() <= 1e-13
+    G2 = gp.chol_adjoint(dev(d[:, None] * L), dev(Wt / d[:, None])).cpu().numpy()
+    assert np.abs(G2 * d[:, None] * d[None, :] - G).max() <= 1e-12 * np.abs(G).max()
+
+
+def test_adjoint_of_independent_blocks_keeps_the_small_one():
+    n, h = 500, 300
+    K, Wt = problem(n, 9)
+    K[h:, :h] = K[:h, h:] = 0.0
+    Wt[h:, :h] = 0.0
+    Wt[h:, h:] *= 1e-30
+    L = O.chol(K)
+    G = gp.chol_adjoint(dev(L), dev(Wt)).cpu().numpy()
+    ref = O.chol_adjoint(L, Wt)
+    assert rel(G[h:, h:], ref[h:, h:]) <= 1e-12 and rel(G[:h, :h], ref[:h, :h]) <= 1e-12
+
+
+@pytest.mark.parametrize("bad,value,status", [(300, -1.0, gp.GPC_ERR_NOT_PD), (450, np.nan, gp.GPC_ERR_NAN),
+                                              (450, np.inf, gp.GPC_ERR_NAN)])
+def test_failing_pivots(bad, value, status):
+    K, _ = problem(640, 11)
+    K[bad, bad] = value
+    info = gp.new_info()
+    gp.chol(dev(K), info=info, check=False)
+    assert info.tolist() == [bad, status]
+
+
+@pytest.mark.parametrize("value,status", [(1e9, gp.GPC_ERR_NOT_PD), (1e200, gp.GPC_ERR_NOT_PD), (np.nan, gp.GPC_ERR_NAN)])
+def test_row_above_its_diagonal_fails_at_that_row(value, status):
+    K, _ = problem(640, 12)
+    K[400, 20] = value
+    info = gp.new_info()
+    gp.chol(dev(K), info=info, check=False)
+    assert info.tolist() == [400, status]
+
+
+def test_nan_in_the_adjoint_spreads():
+    n = 400
+    K, Wt = problem(n, 13)
+    Wt[350, 200] = np.nan
+    L = O.chol(K)
+    G = gp.chol_adjoint(dev(L), dev(Wt)).cpu().numpy()
+    ref = O.chol_adjoint(L, Wt)
+    assert np.isnan(G[350, 100]) and np.isnan(ref[350, 100])
