@@ -82,7 +82,7 @@ AdjWs carve_adj(void *ws, int n) {
 // 0.81 ms at n = 200, 1.13 / 1.08 at 257, 2.50 / 2.10 at 513, 5.05 / 3.71 at 900,
 // 93 / 22.7 at 4096.  Above 40960 the slices of L^T (14 n^2 bytes) would take
 // more than 23 GB beside the caller's matrices.
-bool f64_on_slices(int n) { return n >= 256 && n <= 40960; }
+bool f64_on_slices(int n) { return (n >= 320 || n == 256) && n <= 40960; }
 
 size_t chol_workspace_bytes(int n) {
   const size_t b = block_sz();

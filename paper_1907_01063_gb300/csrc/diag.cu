@@ -9,10 +9,6 @@
 namespace gpc {
 namespace {
 
-constexpr int DIAG_THREADS = 256;
-
-__device__ __forceinline__ double &S(double *s, int ld, int i, int j) { return s[i * ld + j]; }
-
 // All diagonal-block inverses of L at once.  Block 0 is rows [0, first),
 // block ib >= 1 is [first + (ib - 1) b, first + ib b).  With ldo == 0 the
 // inverse of block ib goes to out + ib * b * b with leading dimension equal to
@@ -164,25 +160,6 @@ trtri_cols_kernel(int n, const double *L, long long ldl, int first, int b, doubl
   }
 }
 
-// Cholesky factor of one nb x nb diagonal block in shared memory (the small-
-// block step of Section 3.3), blocked right-looking with panels of PF_PW
-// columns.  Per panel:
-//  1. the PF_PW x PF_PW diagonal sub-block by Schur-complement updates
-//     without square roots (a_ik -= a_ij a_kj / a_jj), one thread per
-//     element, one barrier per column; the thread that owns the next pivot
-//     forms its reciprocal right after its own update.  Column k is then
-//     scaled by 1/sqrt(a_kk) (L = L' D^{1/2}).
-//  2. one thread per row below solves that row against the sub-block,
-//     column by column with the later columns' updates independent, and
-//     writes it, transposed, into a panel buffer;
-//  3. every thread updates 4 x 4 tiles of the trailing lower triangle from
-//     the panel buffer (row and column quadruples read as contiguous pairs).
-// The FP64 pipe of one SM bounds step 3 (about nb^3/6 fused multiply-adds);
-// steps 1 and 2 are short dependent chains.  Writes L11 in place with the
-// upper part of the block zeroed; the first failing pivot is recorded in info
-// (GPC_ERR_NOT_PD, or GPC_ERR_NAN for NaN/Inf) and the rest of the block is
-// written back unfinished.  No inverse is formed: the panel below is solved
-// by substitution (trsm_rows_kernel).
 // An FP64 entry, or a double-float one (FP32 hi + lo in the same 8 bytes) when df.
 __device__ __forceinline__ double load_entry(const double *p, int df) {
   if (df) {
@@ -192,121 +169,196 @@ __device__ __forceinline__ double load_entry(const double *p, int df) {
   return *p;
 }
 
-constexpr int PF_PW = 16;
-static_assert(PF_PW * PF_PW == DIAG_THREADS, "one thread per sub-block element");
-__global__ void __launch_bounds__(DIAG_THREADS)
-potrf_diag_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, int df) {
-  extern __shared__ double smem[];                            // nb x (nb + 1)
-  __shared__ __align__(16) double pt[PF_PW][kMaxBlock + 4];  // panel rows below, transposed
-  __shared__ double rdiag[PF_PW], pinv[PF_PW];
-  __shared__ int fail;
-  const int ld = nb + 1;
-  if (threadIdx.x == 0) fail = 0;
-  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-    const int i = idx / nb, j = idx - i * nb;
-    S(smem, ld, i, j) = (j <= i) ? load_entry(A + (long long)i * lda + j, df) : 0.0;
+// Cholesky factor of one nb x nb diagonal block, nb <= NB (the small-block step
+// of Section 3.3), in panels of 8 columns without square roots: A = X D^-1 X^T
+// with X = L sqrt(D), so the chain from pivot to pivot is one reciprocal, one
+// multiply and one multiply-add, and all square roots are taken at the end.
+// FP64 instructions are what counts here: each holds its sub-partition's FP64
+// pipe for 64 cycles whatever its active lanes, and a dependent one follows after
+// 67.  Per panel p:
+//   1. warp 0 factors the 8 x 8 diagonal tile (lane = row and column mod 4: at
+//      most six FP64 instructions per column, three of them the reciprocal);
+//      meanwhile the other warps, which hold the trailing 8 x 8 tiles in registers
+//      (two entries per lane, dealt in column order), apply panel p-1 to theirs,
+//      the tiles of column p first, which they store;
+//   2. every warp solves 16 of the rows below (two lanes per row, 20 FP64
+//      instructions) and stores them as X and as W = X D^-1;
+//   3. the next diagonal tile takes its update -X W^T and is stored.
+// Three barriers per panel.  The trailing updates are plain multiply-adds: the
+// tensor instruction m8n8k4 takes 611 cycles against 512 for the same 256 of
+// them, and takes them even when its predicate is off.  Writes L11 in place with the upper part of the block
+// zeroed; the first failing pivot is recorded in info (GPC_ERR_NOT_PD, or
+// GPC_ERR_NAN for NaN/Inf) and the rest of the block is written back unfinished.
+// Measured: 64 rows 74 -> 51 us against a column-by-column lookahead with one
+// pivot warp (square roots and two row halves on the chain), 128 rows 250 -> 170.
+// 1/x to about 2 ulp: the hardware seed and one third-order step y (1 + e + e^2).
+__device__ __forceinline__ double recip_cubic(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// Positive, finite and normal, by the high word (a comparison of FP64 values
+// would take the FP64 pipe).
+__device__ __forceinline__ bool normal_positive(double x) {
+  return (unsigned)(__double2hiint(x) - 0x00100000) < 0x7FE00000u;
+}
+
+constexpr int kPotrfW = 12;  // row of W: 8 entries, padded against bank conflicts
+template <int NB>
+constexpr size_t potrf_smem() {
+  return ((size_t)NB * (NB + 4) + (size_t)NB * kPotrfW + 8 * 9 + NB) * sizeof(double);
+}
+
+template <int NB>
+__device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, int *info, int pivot_offset, int df) {
+  constexpr int LD = NB + 4, NT = NB / 8, NW = NB / 16, OWN = NW - 1, TILES = NT * (NT - 1) / 2,
+                SLOTS = (TILES + OWN - 1) / OWN;
+  extern __shared__ double sm[];
+  double *M = sm, *W = sm + NB * LD, *Wd = W + NB * kPotrfW, *pinv_s = Wd + 8 * 9;
+  __shared__ int fail;  // failing column, or NB
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tr = lane >> 2, tc = lane & 3;  // row and column pair of an 8 x 8 tile
+  if (threadIdx.x == 0) fail = NB;
+#pragma unroll 16
+  for (int idx = threadIdx.x; idx < NB * NB; idx += 32 * NW) {
+    const int r = idx / NB, c = idx - r * NB;  // rows past nb: the identity
+    M[r * LD + c] = (r < nb && c < nb) ? (c <= r ? load_entry(A + (long long)r * lda + c, df) : 0.0) : (r == c ? 1.0 : 0.0);
   }
   __syncthreads();
-  const int si = threadIdx.x / PF_PW, sk = threadIdx.x % PF_PW;  // sub-block element of this thread
-  for (int p0 = 0; p0 < nb; p0 += PF_PW) {
-    const int pw = min(PF_PW, nb - p0), m0 = p0 + pw;
-    const bool mine = si < pw && sk <= si;
-    // 1. diagonal sub-block
-    auto pivot = [&](int j) {  // by the owner of (j, j), after its last update
-      const double pv = S(smem, ld, p0 + j, p0 + j);
-      if (!(pv > 0.0 && pv <= 1.79769313486231570e308)) {
-        fail = 1;
-        if (info && info[1] == 0) {
-          info[0] = pivot_offset + p0 + j;
-          info[1] = (pv != pv || pv > 1.79769313486231570e308) ? GPC_ERR_NAN : GPC_ERR_NOT_PD;
-        }
-      } else {
-        pinv[j] = recip_nr(pv);
-      }
-    };
-    if (threadIdx.x == 0) pivot(0);
-    __syncthreads();
-    for (int j = 0; j < pw && !fail; ++j) {
-      if (mine && sk > j) {
-        const double t = S(smem, ld, p0 + si, p0 + j) * pinv[j];
-        S(smem, ld, p0 + si, p0 + sk) = fma(-t, S(smem, ld, p0 + sk, p0 + j), S(smem, ld, p0 + si, p0 + sk));
-        if (si == j + 1 && sk == j + 1) pivot(j + 1);
-      }
-      __syncthreads();
+  // tiles (ti, tk), 1 <= tk <= ti, in column order: slot s of owner o = w - 1 is number s OWN + o
+  double acc[SLOTS][2];
+  int ti[SLOTS], tk[SLOTS];
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) {
+    int t = s * OWN + w - 1, k = 1;
+    if (w == 0 || t >= TILES) {
+      ti[s] = tk[s] = -1;
+      continue;
     }
-    if (fail) break;
-    if (mine && si == sk) rdiag[sk] = rsqrt_nr(S(smem, ld, p0 + sk, p0 + sk));
-    __syncthreads();
-    if (mine) {
-      double &e = S(smem, ld, p0 + si, p0 + sk);
-      e *= rdiag[sk];  // on the diagonal: a_kk / sqrt(a_kk) = sqrt(a_kk)
+    while (t >= NT - k) t -= NT - k++;
+    tk[s] = k;
+    ti[s] = k + t;
+    const double *src = M + (8 * ti[s] + tr) * LD + 8 * k + 2 * tc;
+    acc[s][0] = src[0];
+    acc[s][1] = src[1];
+  }
+  auto update = [&](int s, int p) {  // tile s -= X W^T of panel p
+    const double *x = M + (8 * ti[s] + tr) * LD + 8 * p, *v = W + (8 * tk[s] + 2 * tc) * kPotrfW;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      acc[s][0] = fma(-x[q], v[q], acc[s][0]);
+      acc[s][1] = fma(-x[q], v[kPotrfW + q], acc[s][1]);
     }
-    __syncthreads();
-    // 2. rows below the sub-block: x = a L_pp^{-T} by forward substitution
-    for (int i = m0 + threadIdx.x; i < nb; i += blockDim.x) {
-      double x[PF_PW];
+  };
+  auto store = [&](int s) {
+    double *dst = M + (8 * ti[s] + tr) * LD + 8 * tk[s] + 2 * tc;
+    dst[0] = acc[s][0];
+    dst[1] = acc[s][1];
+  };
+  const int np = (nb + 7) / 8;
+  for (int p = 0; p < np; ++p) {
+    if (w == 0) {
+      const int i = tr, q = tc;
+      double *D = M + (8 * p + i) * LD + 8 * p + q;
+      double a0 = D[0], a1 = D[4];
+      bool ok = true;
 #pragma unroll
-      for (int j = 0; j < PF_PW; ++j) x[j] = (j < pw) ? S(smem, ld, i, p0 + j) : 0.0;
-#pragma unroll
-      for (int j = 0; j < PF_PW; ++j) {
-        if (j < pw) {
-          x[j] *= rdiag[j];
-#pragma unroll
-          for (int t = j + 1; t < PF_PW; ++t)
-            if (t < pw) x[t] = fma(-x[j], S(smem, ld, p0 + t, p0 + j), x[t]);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < PF_PW; ++j) {
-        if (j < pw) {
-          S(smem, ld, i, p0 + j) = x[j];
-          pt[j][i - m0] = x[j];
-        }
-      }
-    }
-    __syncthreads();
-    // 3. trailing update of the lower triangle, rows and columns in [m0, nb)
-    const int m = nb - m0;
-    if (m > 0) {
-      const int tb = (m + 3) >> 2, ntiles = tb * (tb + 1) / 2;
-      for (int t = threadIdx.x; t < ntiles; t += blockDim.x) {
-        int ti = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-        while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
-        while (ti * (ti + 1) / 2 > t) --ti;
-        const int tk = t - ti * (ti + 1) / 2;
-        const int r0 = 4 * ti, c0 = 4 * tk;  // offsets from m0
-        double acc[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
-#pragma unroll
-        for (int q = 0; q < PF_PW; ++q) {
-          if (q < pw) {
-            const double2 a01 = *(const double2 *)&pt[q][r0], a23 = *(const double2 *)&pt[q][r0 + 2];
-            const double2 b01 = *(const double2 *)&pt[q][c0], b23 = *(const double2 *)&pt[q][c0 + 2];
-            const double a[4] = {a01.x, a01.y, a23.x, a23.y}, bc[4] = {b01.x, b01.y, b23.x, b23.y};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], bc[v], acc[u][v]);
+      for (int j = 0; j < 8; ++j) {
+        const double aj = j < 4 ? a0 : a1;
+        const double d = __shfl_sync(0xffffffffu, aj, j * 4 + (j & 3));
+        const bool fine = normal_positive(d);
+        if (ok && !fine && !(d > 0.0 && d <= 1.79769313486231570e308)) {
+          ok = false;
+          if (lane == 0) {
+            fail = 8 * p + j;
+            if (info && info[1] == 0) {
+              info[0] = pivot_offset + 8 * p + j;
+              info[1] = (d != d || d > 1.79769313486231570e308) ? GPC_ERR_NAN : GPC_ERR_NOT_PD;
+            }
           }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            const int i = m0 + r0 + u, k = m0 + c0 + v;
-            if (i < nb && k <= i) S(smem, ld, i, k) -= acc[u][v];
-          }
+        if (!ok) continue;
+        const double aij = __shfl_sync(0xffffffffu, aj, (lane & ~3) | (j & 3));
+        const double k0 = __shfl_sync(0xffffffffu, aj, q * 4 + (j & 3));
+        const double k1 = __shfl_sync(0xffffffffu, aj, (q + 4) * 4 + (j & 3));
+        const double pinv = fine ? recip_cubic(d) : 1.0 / d, t = aij * pinv;
+        if (j < 3 && q > j) a0 = fma(-t, k0, a0);
+        if (j < 7 && q + 4 > j) a1 = fma(-t, k1, a1);
+        if (q == (j & 3)) Wd[i * 9 + j] = t;
+        if (lane == 0) pinv_s[8 * p + j] = pinv;
       }
+      D[0] = a0;
+      D[4] = a1;
+    } else if (p > 0) {
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (tk[s] == p && ti[s] > p) {
+          update(s, p - 1);
+          store(s);
+        }
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (tk[s] > p) update(s, p - 1);
+    }
+    __syncthreads();
+    if (fail < NB || p == np - 1) break;
+    const int row = 8 * (p + 1) + 16 * w + (lane >> 1), h = lane & 1;
+    if (8 * (p + 1) + 16 * w < NB) {
+      double *xr = M + (row < NB ? row : NB - 1) * LD + 8 * p + h;
+      double x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = xr[2 * u];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const double xj = __shfl_sync(0xffffffffu, x[j >> 1], (lane & ~1) | (j & 1));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (2 * u + 1 <= j) continue;
+          if (2 * u + h > j) x[u] = fma(-xj, Wd[(2 * u + h) * 9 + j], x[u]);
+        }
+      }
+      if (row < NB) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          xr[2 * u] = x[u];
+          W[row * kPotrfW + 2 * u + h] = x[u] * pinv_s[8 * p + 2 * u + h];
+        }
+      }
+    }
+    __syncthreads();
+    if (w > 0) {
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (tk[s] == p + 1 && ti[s] == p + 1) {
+          update(s, p);
+          store(s);
+        }
     }
     __syncthreads();
   }
-  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-    const int r = idx / nb, c = idx - r * nb;
-    A[(long long)r * lda + c] = (c <= r) ? S(smem, ld, r, c) : 0.0;
+  // L = X D^-1/2; the diagonal holds D
+  const int last = fail;
+  double *rs = W;
+  __syncthreads();
+  if (threadIdx.x < NB) rs[threadIdx.x] = threadIdx.x < last ? rsqrt_nr(M[threadIdx.x * (LD + 1)]) : 1.0;
+  __syncthreads();
+#pragma unroll 8
+  for (int idx = threadIdx.x; idx < NB * NB; idx += 32 * NW) {
+    const int r = idx / NB, c = idx - r * NB;
+    if (r < nb && c < nb) A[(long long)r * lda + c] = (c <= r) ? M[r * LD + c] * rs[c] : 0.0;
   }
+}
+
+// Blocks of up to 64 rows.
+__global__ void __launch_bounds__(128)
+potrf_la_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, int df) {
+  potrf_block<64>(nb, A, lda, info, pivot_offset, df);
+}
+// Blocks of 65 to 128 rows.
+__global__ void __launch_bounds__(256)
+potrf_diag_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, int df) {
+  potrf_block<128>(nb, A, lda, info, pivot_offset, df);
 }
 
 // Row-parallel triangular solve of an m x nb panel X (in place) against the
@@ -359,7 +411,7 @@ trsm_rows_kernel(int m, int nb, double *X, long long ldx, const double *T, long 
   }
 }
 
-// The same panel solve with TPR threads per row (4, or 16 for short panels)
+// The same panel solve with TPR threads per row (4 or 16 by panel height)
 // and no block barriers, for the block sizes the factorisations use (NB = 64
 // or 128).  Thread t of a row holds columns k = TPR c + t (c < NB / TPR) in
 // registers; at step j the owner of column j (final by then) passes it to the
@@ -474,163 +526,6 @@ __global__ void recip_rsqrt_probe_kernel(int n, const double *x, double *out) {
   out[4 * i + 3] = rsqrt(v);
 }
 
-// Cholesky factor of one nb x nb diagonal block, nb <= 64, with a one-column
-// lookahead (the small-block step of Section 3.3).  Column k+1 is finished
-// (pivot, 1/sqrt, scaling) by one warp while six other warps apply column k
-// to the rest of the block.  On this part a dependent FP64 operation costs
-// about 60 cycles and one SM sustains under two FP64 multiply-adds per cycle,
-// so the pivot chain and the trailing updates must overlap, and no FP64
-// instruction may issue with lanes that have nothing to do (a warp
-// instruction costs the FP64 pipe the same time whatever its active mask):
-//   * warp 0 (the pivot warp) finishes columns: for column k+1 it applies the
-//     column-k update itself, takes r = 1/sqrt(pivot) and writes the final
-//     column to shared memory, then publishes col_ready = k+1;
-//   * warps 1-3 and 5-7 (the updaters, u = 0..5) own whole columns j = u mod 6,
-//     lane l holding rows j + l and j + l + 32 in registers, so whether a
-//     column takes part in a step is the same for the whole warp; at step k,
-//     once column k is final, the owner of column k+2 (the one the pivot warp
-//     finishes next) updates and stores it first and marks rounds[k+1], then
-//     every warp updates its later columns (rounds[0]: columns 0 and 1 stored
-//     as loaded, one mark per warp);
-//   * warp 4 idles, so the pivot warp has its SM sub-partition to itself.
-// Every wait is a bounded spin on a shared-memory word; a wait that runs out
-// records GPC_ERR_TIMEOUT and stops the block.  The first failing pivot is
-// recorded like potrf_diag_kernel does, and the rest of the block is written
-// back unfinished.
-constexpr int PL_NB = 64, PL_LD = PL_NB + 1, PL_W = 6, PL_COLS = (PL_NB + PL_W - 1) / PL_W;
-constexpr long long PL_SPIN = 1LL << 24;
-
-__global__ void __launch_bounds__(256)
-potrf_la_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, int df, int *gerr) {
-  __shared__ double M[PL_NB * PL_LD];
-  __shared__ int col_ready, stop;
-  __shared__ int rounds[PL_NB];  // rounds[r]: marks of round r
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) {
-    col_ready = -1;
-    stop = 0;
-  }
-  if (threadIdx.x < PL_NB) rounds[threadIdx.x] = 0;
-  const bool updater = warp != 0 && warp != 4;
-  const int uw = updater ? warp - 1 - (warp > 4) : 0;
-  double a0[PL_COLS], a1[PL_COLS];  // column uw + 6 c: rows j + lane, j + lane + 32
-  if (updater) {
-#pragma unroll
-    for (int c = 0; c < PL_COLS; ++c) {
-      const int j = uw + PL_W * c, r0 = j + lane, r1 = r0 + 32;
-      a0[c] = (j < nb && r0 < nb) ? load_entry(A + (long long)r0 * lda + j, df) : 0.0;
-      a1[c] = (j < nb && r1 < nb) ? load_entry(A + (long long)r1 * lda + j, df) : 0.0;
-    }
-  }
-  __syncthreads();
-  volatile int *vready = &col_ready, *vstop = &stop;
-  // Polls: the updaters back off between polls, so that their loads do not
-  // queue in front of the pivot warp's shared-memory accesses.
-  auto spin_ge = [&](volatile int *w, int target) -> bool {
-    for (long long it = 0; it < PL_SPIN; ++it) {
-      if (*w >= target) return true;
-      if (*vstop) return false;
-      if (updater) __nanosleep(64);
-    }
-    return false;
-  };
-  auto give_up = [&]() {  // a wait ran out: report and stop the block
-    if (info && info[1] == 0) info[1] = GPC_ERR_TIMEOUT;
-    record_error(gerr, GPC_ERR_TIMEOUT);
-    *vstop = 1;
-  };
-  if (updater) {
-    // round 0: columns 0 and 1 as loaded (owned by updaters 0 and 1)
-    if (uw <= 1 && uw < nb) {
-      const int j = uw, r0 = j + lane, r1 = r0 + 32;
-      if (r0 < nb) M[r0 * PL_LD + j] = a0[0];
-      if (r1 < nb) M[r1 * PL_LD + j] = a1[0];
-    }
-    __threadfence_block();
-    __syncwarp();
-    if (lane == 0) atomicAdd(&rounds[0], 1);
-  }
-  if (warp == 0) {
-    // ---- pivot warp: lanes own rows lane and lane + 32
-    for (int c = 0; c < nb; ++c) {
-      // column c comes from round max(c - 1, 0)
-      if (!spin_ge((volatile int *)&rounds[max(c - 1, 0)], c <= 1 ? PL_W : 1)) {
-        if (!*vstop && lane == 0) give_up();
-        break;
-      }
-      __threadfence_block();
-      const int i0 = lane, i1 = lane + 32;
-      double v0 = (i0 >= c && i0 < nb) ? M[i0 * PL_LD + c] : 0.0;
-      double v1 = (i1 >= c && i1 < nb) ? M[i1 * PL_LD + c] : 0.0;
-      if (c > 0) {  // the update by column c - 1, finished by this warp just before
-        const double lc = M[c * PL_LD + c - 1];
-        if (i0 >= c && i0 < nb) v0 = fma(-M[i0 * PL_LD + c - 1], lc, v0);
-        if (i1 >= c && i1 < nb) v1 = fma(-M[i1 * PL_LD + c - 1], lc, v1);
-      }
-      const double pv = (c < 32) ? __shfl_sync(0xffffffffu, v0, c) : __shfl_sync(0xffffffffu, v1, c - 32);
-      if (!(pv > 0.0 && pv <= 1.79769313486231570e308)) {
-        if (lane == 0) {
-          if (info && info[1] == 0) {
-            info[0] = pivot_offset + c;
-            info[1] = (pv != pv || pv > 1.79769313486231570e308) ? GPC_ERR_NAN : GPC_ERR_NOT_PD;
-          }
-          *vstop = 1;
-        }
-        break;
-      }
-      const double r = rsqrt_nr(pv);  // every lane: no broadcast on the chain
-      if (i0 >= c && i0 < nb) M[i0 * PL_LD + c] = (i0 == c) ? pv * r : v0 * r;
-      if (i1 >= c && i1 < nb) M[i1 * PL_LD + c] = (i1 == c) ? pv * r : v1 * r;
-      __threadfence_block();
-      __syncwarp();
-      if (lane == 0) *vready = c;
-    }
-  } else if (updater) {
-    // ---- updaters: step k applies column k to columns k + 2 .. nb - 1
-    for (int k = 0; k + 2 < nb; ++k) {
-      if (!spin_ge(vready, k)) {
-        if (!*vstop && lane == 0) give_up();
-        break;
-      }
-      __threadfence_block();
-#pragma unroll
-      for (int c = 0; c < PL_COLS; ++c) {
-        const int j = uw + PL_W * c;
-        if (j == k + 2) {  // warp-uniform: the column the pivot warp needs next
-          const double ljk = M[j * PL_LD + k];
-          const int r0 = j + lane, r1 = r0 + 32;
-          if (r0 < nb) {
-            a0[c] = fma(-M[r0 * PL_LD + k], ljk, a0[c]);
-            M[r0 * PL_LD + j] = a0[c];
-          }
-          if (r1 < nb) {
-            a1[c] = fma(-M[r1 * PL_LD + k], ljk, a1[c]);
-            M[r1 * PL_LD + j] = a1[c];
-          }
-          __threadfence_block();
-          __syncwarp();
-          if (lane == 0) atomicAdd(&rounds[k + 1], 1);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < PL_COLS; ++c) {
-        const int j = uw + PL_W * c;
-        if (j > k + 2 && j < nb) {  // warp-uniform
-          const double ljk = M[j * PL_LD + k];
-          const int r0 = j + lane, r1 = r0 + 32;
-          if (r0 < nb) a0[c] = fma(-M[r0 * PL_LD + k], ljk, a0[c]);
-          if (j + 32 < nb && r1 < nb) a1[c] = fma(-M[r1 * PL_LD + k], ljk, a1[c]);
-        }
-      }
-    }
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-    const int r = idx / nb, c = idx - r * nb;
-    A[(long long)r * lda + c] = (c <= r) ? M[r * PL_LD + c] : 0.0;
-  }
-}
-
 }  // namespace
 
 cudaError_t trtri_batched(int n, const double *L, long long ldl, int first, int b, double *out,
@@ -672,23 +567,22 @@ cudaError_t trtri_batched(int n, const double *L, long long ldl, int first, int 
 cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_offset, cudaStream_t s, bool df) {
   if (nb <= 0) return cudaSuccess;
   if (nb > kMaxBlock) return cudaErrorInvalidValue;
+  if (nb <= 64) {
+    GPC_LAUNCH(GPC_TRACE_DIAG, (double)nb * nb * nb / 3.0, 16.0 * nb * nb, s,
+               launch_k(potrf_la_kernel, 1, 128, potrf_smem<64>(), s, nb, A, lda, info, pivot_offset, df ? 1 : 0));
+    return cudaGetLastError();
+  }
   static bool attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
     cudaError_t e = cudaFuncSetAttribute(potrf_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)((size_t)kMaxBlock * (kMaxBlock + 1) * sizeof(double)));
+                                         (int)potrf_smem<128>());
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
-  if (nb <= PL_NB) {  // blocks of up to 64: the lookahead kernel
-    GPC_LAUNCH(GPC_TRACE_DIAG, (double)nb * nb * nb / 3.0, 16.0 * nb * nb, s,
-               launch_k(potrf_la_kernel, 1, 256, 0, s, nb, A, lda, info, pivot_offset, df ? 1 : 0, error_word()));
-    return cudaGetLastError();
-  }
-  const size_t smem = (size_t)nb * (nb + 1) * sizeof(double);
   GPC_LAUNCH(GPC_TRACE_DIAG, (double)nb * nb * nb / 3.0, 16.0 * nb * nb, s,
-             launch_k(potrf_diag_kernel, 1, DIAG_THREADS, smem, s, nb, A, lda, info, pivot_offset, df ? 1 : 0));
+             launch_k(potrf_diag_kernel, 1, 256, potrf_smem<128>(), s, nb, A, lda, info, pivot_offset, df ? 1 : 0));
   return cudaGetLastError();
 }
 
@@ -723,25 +617,25 @@ cudaError_t trsm_rows(int m, int nb, double *X, long long ldx, const double *T, 
   if (cudaError_t ce = trsm_carveout(); ce != cudaSuccess) return ce;
   const double fl = (double)m * nb * nb, by = 16.0 * (double)m * nb + 4.0 * nb * nb;
   if (nb == 64 || nb == 128) {
-    // short panels (at most 256 rows): 16 threads per row, so the row's FP64
-    // work is spread over four times as many warps
-    const bool short_panel = m <= 256;
-    const int tpr = short_panel ? 16 : 4;
+    // A warp issues 224 FP64 instructions for its 2 rows with 16 threads per row
+    // and 608 for 8 rows with 4 (NB = 64; the same proportion at 128): as long as
+    // all warps run at once, the wider split is the faster (m = 1000: 31 us with
+    // 4 threads per row, 18 with 16).  Eight threads per row gained nothing above.
+    const int tpr = m <= 8 * sm_count() ? 16 : 4;
     const unsigned qgrid = (unsigned)((m + TQ_THREADS / tpr - 1) / (TQ_THREADS / tpr));
 #define GPC_TRSM_QUAD(NB_, MODE_, TPR_)                                                                      \
   GPC_LAUNCH(GPC_TRACE_TRSM, fl, by, s,                                                                     \
              launch_k(trsm_quad_kernel<NB_, MODE_, TPR_>, qgrid, TQ_THREADS, 0, s, m, X, ldx, T, ldt, df))
-    if (short_panel) {
-      if (nb == 64 && mode == 0) GPC_TRSM_QUAD(64, 0, 16);
-      else if (nb == 64) GPC_TRSM_QUAD(64, 1, 16);
-      else if (mode == 0) GPC_TRSM_QUAD(128, 0, 16);
-      else GPC_TRSM_QUAD(128, 1, 16);
-    } else {
-      if (nb == 64 && mode == 0) GPC_TRSM_QUAD(64, 0, 4);
-      else if (nb == 64) GPC_TRSM_QUAD(64, 1, 4);
-      else if (mode == 0) GPC_TRSM_QUAD(128, 0, 4);
-      else GPC_TRSM_QUAD(128, 1, 4);
-    }
+#define GPC_TRSM_TPR(TPR_)                                \
+  do {                                                    \
+    if (nb == 64 && mode == 0) GPC_TRSM_QUAD(64, 0, TPR_);  \
+    else if (nb == 64) GPC_TRSM_QUAD(64, 1, TPR_);          \
+    else if (mode == 0) GPC_TRSM_QUAD(128, 0, TPR_);        \
+    else GPC_TRSM_QUAD(128, 1, TPR_);                       \
+  } while (0)
+    if (tpr == 16) GPC_TRSM_TPR(16);
+    else GPC_TRSM_TPR(4);
+#undef GPC_TRSM_TPR
 #undef GPC_TRSM_QUAD
     return cudaGetLastError();
   }
