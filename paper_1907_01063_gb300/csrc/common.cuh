@@ -351,13 +351,14 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // ---------------------------------------------------------------- FP64-accurate split products (f64x.cu)
 struct SliceBuf;
 constexpr int kF64xSlices = 7;                     // BF16 slices per operand of the factorisation's products
+constexpr int kF64xWide = 8;                       // of a general product, and of the adjoint's panel x inverse
 constexpr size_t kF64xScratchCap = size_t(1) << 30;  // a general product's slices per pass
 // A checked product (8 slices) of K terms loses at most K 2^-62.5 relative to
 // its operands' row scales; the FP64 chain's bound is K 2^-53 S with S = sum
 // |a'||b'| in the same units, so S >= 2^-9.5 suffices.  S is formed from the
 // leading eight bits of the magnitudes (rounded toward zero: never too large).
 constexpr float kF64xTheta = 0x1.7p-10f;
-size_t f64x_slice_bytes(int rows, int kchunks);
+size_t f64x_slice_bytes(int rows, int kchunks, bool wide = false);
 // The slices of split_operand, kF64xSlices of them, of the entries scaled by
 // 2^(kexp_sign kexp[k] - rexp[r]) (either may be null).  saturate: scaled
 // entries above 2^30 become 2^30, otherwise (and for NaN) NaN.
@@ -368,6 +369,8 @@ struct F64xRow {
   int block_rows = 0;
   int tri = 0;                    // 1: entries with k < r are zero (not read)
   const int *rexp_sub = nullptr;  // non-null: rexp holds one exponent, row r's is *rexp - rexp_sub[r]
+  bool df = false;                // the entries are FP32 pairs (double-float storage)
+  bool wide = false;              // kF64xWide slices
 };
 cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,
                        const int *rexp, const int *kexp, int kexp_sign, bool saturate, cudaStream_t s,
@@ -378,11 +381,18 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
 cudaError_t f64x_diag_exps(int n, const double *K, long long ldk, int *rexp, cudaStream_t s);
 cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, int *cexp, cudaStream_t s);
 cudaError_t f64x_block_exp(int nb, const double *A, long long lda, const int *rexp, int *out, cudaStream_t s);
-// C (FP64) -= 2^(ra_i + rb_j) A B^T (with ra_sub: 2^(*ra - ra_sub_i + rb_j)); the other arguments as for ozaki_gemm.
+// C (FP64) -= 2^(ra_i + rb_j) A B^T (with ra_sub: 2^(*ra - ra_sub_i + rb_j)),
+// or with `wide` C = that product on kF64xWide slices; the other arguments as for ozaki_gemm.
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
                       double *partial, int *err, cudaStream_t s, int max_ctas = 0, int kdepth = 0, int max_items = 0,
-                      const int *ra_sub = nullptr);
+                      const int *ra_sub = nullptr, bool wide = false);
+// Slices of the transposes of lower-triangular diagonal blocks (the first of order `first` at src with leading
+// dimension ld0, the others of order 128, `stride` apart from src + off1, with ld): operand row c = column c, scaled
+// by its own largest entry; block ib's kF64xWide slices at out + ib f64x_slice_bytes(128, 1, true), its scale
+// exponents at exps + 128 ib.
+cudaError_t f64x_split_blocks(int nblk, int first, const double *src, long long ld0, long long ld, long long off1,
+                              long long stride, void *out, int *exps, cudaStream_t s);
 // gemm_f64 through checked split products where the size pays for the split
 // and ws (f64x_scratch_bytes, or less: more passes) allows; otherwise gemm_f64,
 // with ws as its split-K scratch.

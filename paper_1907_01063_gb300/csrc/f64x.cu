@@ -791,6 +791,7 @@ struct FxOperand {
   const int *row_exps;
   int *counts;           // per row: entries of at least 2^-5 of the row's scale (null: not counted)
   int rexp_stride, tri, tri_off;
+  int df;                // entries are FP32 pairs (hi, lo)
   unsigned short *dst;
   long long plane, dst_stride;
 };
@@ -826,7 +827,15 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     bool in = r < o.M && kk < klen;
     if (o.tri == 1) in = in && k >= r + o.tri_off;
     if (o.tri == 2) in = in && k <= r + o.tri_off;
-    tile[rr][kk] = in ? src[(long long)r * o.rs + (long long)k * o.ks] : 0.0;
+    const double *at = src + (long long)r * o.rs + (long long)k * o.ks;
+    double v = 0.0;
+    if (in && o.df) {
+      const float2 q = *reinterpret_cast<const float2 *>(at);
+      v = exact_f64(q.x) + exact_f64(q.y);
+    } else if (in) {
+      v = *at;
+    }
+    tile[rr][kk] = v;
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -883,7 +892,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   int shift = 0;  // the row's own exponent, when it is found here
   if (o.rexp_out && r < o.M) {
     shift = emax > kNoExp ? emax + 1 : 0;
-    if (lane == 0) o.rexp_out[r] = shift;
+    if (lane == 0) o.rexp_out[(size_t)blockIdx.z * o.rexp_stride + r] = shift;
   }
   unsigned short *dst =
       o.dst + (long long)blockIdx.z * o.dst_stride + (long long)r * o.kpad + (long long)c * FX_CHUNK + lane * 4;
@@ -1074,9 +1083,9 @@ cudaError_t carveout_max(const void *fn, bool (&done)[64]) {
 
 }  // namespace
 
-size_t f64x_slice_bytes(int rows, int kchunks) {
+size_t f64x_slice_bytes(int rows, int kchunks, bool wide) {
   const size_t rp = align_up((size_t)std::max(rows, 1), FX_BM);
-  return align_up((size_t)kF64xSlices * rp * (size_t)kchunks * FX_CHUNK * 2, 1024);
+  return align_up((size_t)(wide ? kF64xWide : kF64xSlices) * rp * (size_t)kchunks * FX_CHUNK * 2, 1024);
 }
 
 cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,
@@ -1086,9 +1095,9 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
   const int op_chunks = (K <= first) ? 1 : 1 + (K - first + FX_CHUNK - 1) / FX_CHUNK;
   const int chunks = std::min(op_chunks, out.kpad / FX_CHUNK - chunk_offset);
   if (chunks <= 0 || row_offset < 0 || row_offset + M > out.rows_pad) return cudaErrorInvalidValue;
-  static bool carve[64] = {};
-  if (cudaError_t e = carveout_max((const void *)f64x_split_kernel<kF64xSlices, false>, carve); e != cudaSuccess)
-    return e;
+  static bool carve[2][64] = {};
+  const auto fx_split_kernel = row.wide ? f64x_split_kernel<kF64xWide, false> : f64x_split_kernel<kF64xSlices, false>;
+  if (cudaError_t e = carveout_max((const void *)fx_split_kernel, carve[row.wide]); e != cudaSuccess) return e;
   FxSplit p = {};
   FxOperand &o = p.op[0];
   o.src = src;
@@ -1106,6 +1115,7 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
   o.block_rows = row.block_rows;
   o.row_exps = row.row_exps;
   o.tri = row.tri;
+  o.df = row.df ? 1 : 0;
   if (row.rexp_out && chunks != 1) return cudaErrorInvalidValue;
   if (row.block_out)
     if (cudaError_t e = cudaMemsetAsync(row.block_out, 0x80, sizeof(int), s); e != cudaSuccess) return e;
@@ -1117,20 +1127,54 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
   p.sat = saturate ? 1 : 0;
   p.blocks0 = (o.row_end + 7) / 8;
   dim3 grid((unsigned)chunks, (unsigned)p.blocks0);
-  GPC_LAUNCH(GPC_TRACE_SPLIT, 0.0, 8.0 * M * K + 2.0 * kF64xSlices * (double)o.row_end * chunks * FX_CHUNK, s,
-             launch_k(f64x_split_kernel<kF64xSlices, false>, grid, 256, 0, s, p));
+  const int S = row.wide ? kF64xWide : kF64xSlices;
+  GPC_LAUNCH(GPC_TRACE_SPLIT, 0.0, 8.0 * M * K + 2.0 * S * (double)o.row_end * chunks * FX_CHUNK, s,
+             launch_k(fx_split_kernel, grid, 256, 0, s, p));
+  return cudaGetLastError();
+}
+
+cudaError_t f64x_split_blocks(int nblk, int first, const double *src, long long ld0, long long ld, long long off1,
+                              long long stride, void *out, int *exps, cudaStream_t s) {
+  constexpr int b = FX_CHUNK;
+  const size_t bytes = f64x_slice_bytes(b, 1, true);
+  F64xRow row;
+  row.wide = true;
+  row.rexp_out = exps;
+  row.tri = 1;
+  if (cudaError_t e = f64x_split(src, 1, ld0, first, first, first, slice_view(out, b, 1), nullptr, nullptr, 0, false, s,
+                                 0, 0, row);
+      e != cudaSuccess || nblk == 1)
+    return e;
+  FxSplit p = {};
+  FxOperand &o = p.op[0];
+  o.src = src + off1;
+  o.rs = 1;
+  o.ks = ld;
+  o.src_stride = stride;
+  o.M = o.K = o.row_end = o.kpad = b;
+  o.rexp_out = exps + b;
+  o.rexp_stride = b;
+  o.tri = 1;
+  o.dst = (unsigned short *)((char *)out + bytes);
+  o.plane = (long long)b * b;
+  o.dst_stride = (long long)(bytes / 2);
+  p.first = b;
+  p.blocks0 = b / 8;
+  GPC_LAUNCH(GPC_TRACE_SPLIT, 0.0, (8.0 + 2.0 * kF64xWide) * b * b * (nblk - 1), s,
+             launch_k(f64x_split_kernel<kF64xWide, false>, dim3(1, b / 8, (unsigned)(nblk - 1)), 256, 0, s, p));
   return cudaGetLastError();
 }
 
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
-                      double *partial, int *err, cudaStream_t s, int max_ctas, int kdepth, int max_items, const int *ra_sub) {
+                      double *partial, int *err, cudaStream_t s, int max_ctas, int kdepth, int max_items, const int *ra_sub,
+                      bool wide) {
   if (M <= 0 || N <= 0 || chunks <= 0) return cudaSuccess;
   if (kdepth <= 0) kdepth = FX_CHUNK;
-  if (kdepth > FX_CHUNK || kdepth % FX_BK) return cudaErrorInvalidValue;
+  if (kdepth > FX_CHUNK || kdepth % FX_BK || (wide && splits > 1)) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, A.base, A.kpad, A.rows_pad, kF64xSlices, FX_BM) ||
-      !make_map(&mb, B.base, B.kpad, B.rows_pad, kF64xSlices, FX_BN))
+  const int S = wide ? kF64xWide : kF64xSlices;
+  if (!make_map(&ma, A.base, A.kpad, A.rows_pad, S, FX_BM) || !make_map(&mb, B.base, B.kpad, B.rows_pad, S, FX_BN))
     return cudaErrorInvalidValue;
   FxParams p = {};
   p.M = M;
@@ -1147,7 +1191,7 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
   p.tiles_n = (N + FX_BN - 1) / FX_BN;
   p.per_batch = (int)count_tiles(p);
   p.num_work = p.per_batch * p.splits;
-  p.accumulate = 1;
+  p.accumulate = wide ? 0 : 1;
   p.ra = ra;
   p.ra_mul = ra_sub ? 0 : 1;
   p.ra_sub = ra_sub;
@@ -1161,8 +1205,8 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
   p.no_loads = faults().ozaki_no_loads;
   const double mn = !lower ? (double)M * N
                            : (M >= N ? 0.5 * (double)N * (N + 1) + (double)(M - N) * N : 0.5 * (double)M * (M + 1));
-  const double flops = 2.0 * mn * (double)chunks * kdepth * 28.0;  // 28 slice products
-  const double bytes = 16.0 * mn + (double)(M + N) * chunks * kdepth * 2 * kF64xSlices;
+  const double flops = 2.0 * mn * (double)chunks * kdepth * (S * (S + 1) / 2);
+  const double bytes = 16.0 * mn + (double)(M + N) * chunks * kdepth * 2 * S;
   p.sub = 1;
   if (max_ctas == 0 && 4 * p.num_work <= sm_count()) {
     p.sub = 4;
@@ -1170,7 +1214,8 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
   }
   int grid = std::min(p.num_work, max_ctas > 0 ? std::min(max_ctas, sm_count()) : sm_count());
   if (max_items > 0) grid = std::max(grid, (p.num_work + max_items - 1) / max_items);
-  cudaError_t e = launch_product<kF64xSlices, true, false>(ma, mb, p, grid, flops, bytes, s);
+  cudaError_t e = wide ? launch_product<kF64xWide, false, false>(ma, mb, p, grid, flops, bytes, s)
+                       : launch_product<kF64xSlices, true, false>(ma, mb, p, grid, flops, bytes, s);
   if (e != cudaSuccess || p.splits == 1) return e;
   const long long total = (long long)M * N;
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 8.0 * (p.splits + 2) * mn, s,
@@ -1265,7 +1310,7 @@ cudaError_t f64x_block_exp(int nb, const double *A, long long lda, const int *re
 // ------------------------------------------------------------------ general products
 namespace {
 
-constexpr int GX_S = 8;                // slices of a checked product
+constexpr int GX_S = kF64xWide;        // slices of a checked product
 constexpr int GX_PLANES = GX_S + 1;    // and the plane of leading magnitudes
 constexpr size_t kGxMinScratch = size_t(8) << 20;
 

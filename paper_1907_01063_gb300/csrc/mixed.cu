@@ -41,7 +41,8 @@ struct MixWs {
   double *inv, *m, *t, *panel, *scratch;  // FP64 pieces (scratch doubles as the split-K partials)
   void *sc, *sdc, *lt;                    // slices: panel rows, block-column columns, L^T
   void *grp, *tmp;                        // factorisation: two group buffers, per-step temporaries
-  int *rexp, *cexp, *xexp, *bexp;         // FP64 path: scale exponents (rows of L, columns, panel rows, block column)
+  void *sx, *si;                          // adjoint, eight slices: panel rows, diagonal-block inverses
+  int *rexp, *cexp, *xexp, *iexp, *bexp;  // scale exponents: rows of L, its columns, panel rows, inverses, block column
 };
 constexpr int kMaxDefer = 8;
 int defer_depth() { return std::max(1, std::min(tuning().mixed_defer, kMaxDefer)); }
@@ -93,6 +94,8 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
   if (adjoint) {
     w.sdc = p; p += sbytes(MB, nchunks(n), f64);
     w.lt = p; p += sbytes(n, nchunks(n), f64);
+    w.sx = p; p += f64x_slice_bytes(n, 1, true);
+    w.si = p; p += (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
   } else {
     w.grp = p; p += 2 * sbytes(n, defer_depth(), f64);
     w.tmp = p; p += sbytes(n, 1, f64);
@@ -100,6 +103,7 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
   w.rexp = (int *)p; p += exps_bytes(n);
   w.cexp = (int *)p; p += exps_bytes(n);
   w.xexp = (int *)p; p += exps_bytes(n);
+  w.iexp = (int *)p; p += exps_bytes(nchunks(n) * MB);
   w.bexp = (int *)p;
   return w;
 }
@@ -109,8 +113,10 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
 size_t mixed_workspace_bytes(int n, bool f64) {
   n = std::max(n, 1);
   const size_t common = ((size_t)nchunks(n) + 2) * b2() + align_up((size_t)n * MB * sizeof(double), 256) +
-                        scratch_bytes() + 2 * sbytes(n, 1, f64) + 3 * exps_bytes(n) + 256 + 1024;
-  const size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64);
+                        scratch_bytes() + 2 * sbytes(n, 1, f64) + 3 * exps_bytes(n) + exps_bytes(nchunks(n) * MB) + 256 +
+                        1024;
+  const size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64) + f64x_slice_bytes(n, 1, true) +
+                     (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
   const size_t fwd = 2 * sbytes(n, defer_depth(), f64) + sbytes(n, 1, f64);
   return common + std::max(adj, fwd);
 }
@@ -308,7 +314,8 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
   } else {
     TRY(split_operand(L, 1, ldl, n, n, first, LT, s));
   }
-  TRY(trtri_batched(n, L, ldl, first, MB, w.inv, s));  // independent of the sweep: one launch
+  TRY(trtri_batched(n, L, ldl, first, MB, w.inv, s));  // independent of the sweep
+  TRY(f64x_split_blocks(nblk, first, w.inv, first, MB, (long long)MB * MB, (long long)MB * MB, w.si, w.iexp, s));
   Aux *aux = nullptr;
   TRY(aux_for_device(&aux));
   // Within a step the Bbar update (rows below, columns left: the largest
@@ -331,33 +338,16 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
     bool bbar_pending = false;
     if (m > 0) {
       double *Cbar = A + (long long)k * lda + j;
-      if (nb > MH) {
-        // Cbar <- Cbar D^{-1} as two 64-wide steps, right half first: with
-        // D = [Da 0; Dba Db], Xb = Cb Db^{-1}, then Ca -= Xb Dba (split-BF16,
-        // K = nb - 64) and Xa = Ca Da^{-1}.  The FP64 solves halve.
-        const int hb = nb - MH;
-        double *Cb = Cbar + MH;
-        const double *Dba = D + (long long)MH * ldl;
-        TRY(trsm_rows(m, hb, Cb, lda, Dba + MH, ldl, 1, s, df));
-        SliceBuf SX = slice_view((char *)w.sc + sbytes(n, 1, f64), m, 1);
-        SliceBuf SD = slice_view(w.sdc, MH, 1);
-        const int depth = (hb + 31) / 32 * 32;
-        if (f64) {
-          TRY(f64x_split(Cb, lda, 1, m, hb, hb, SX, nullptr, w.rexp + j + MH, 1, false, s, 0, 0,
-                         F64xRow{w.xexp, nullptr, nullptr, 0, 0, nullptr}));
-          TRY(f64x_split(Dba, 1, ldl, MH, hb, hb, SD, w.cexp + j, w.rexp + j + MH, -1, false, s));
-          TRY(f64x_gemm(SX, 0, 0, SD, 0, 0, m, MH, 1, false, w.xexp, w.cexp + j, Cbar, lda, 1, nullptr, err, s, 0,
-                        depth));
-        } else {
-          TRY(split_operand(Cb, lda, 1, m, hb, hb, SX, s));
-          TRY(split_operand(Dba, 1, ldl, MH, hb, hb, SD, s));  // row c, K index t: Dba[t][c]
-          TRY(ozaki_gemm(SX, 0, 0, SD, 0, 0, m, MH, 1, false, -1.0f, (float2 *)Cbar, lda, 1, nullptr, err, s, 0,
-                         depth));
-        }
-        TRY(trsm_rows(m, MH, Cbar, lda, D, ldl, 1, s, df));
-      } else {
-        TRY(trsm_rows(m, nb, Cbar, lda, D, ldl, 1, s, df));  // Cbar <- Cbar D^{-1} (FP64)
-      }
+      // Cbar <- Cbar D^{-1}, FP64 in and out on both paths: one product with the
+      // block's inverse on eight slices (with seven the adjoint's error grows to
+      // twice that of a substitution).  (Two 64-wide substitutions with a
+      // product between them took 132 us at m = 8000 and 65 us at m = 500, this
+      // 40 and 22: the substitution is FP64 work, m 128^2 / 2 multiply-adds.)
+      SliceBuf SX = slice_view(w.sx, m, 1);
+      TRY(f64x_split(Cbar, lda, 1, m, nb, nb, SX, nullptr, nullptr, 0, false, s, 0, 0,
+                     F64xRow{w.xexp, nullptr, nullptr, 0, 0, nullptr, df, true}));
+      TRY(f64x_gemm(SX, 0, 0, slice_view((char *)w.si + (size_t)ib * f64x_slice_bytes(MB, 1, true), MB, 1), 0, 0, m, nb, 1,
+                    false, w.xexp, w.iexp + (size_t)ib * MB, Cbar, lda, 1, nullptr, err, s, 0, 0, 0, nullptr, true));
       // Dbar -= Cbar^T C on slices (mixed: Dbar still in double-float storage):
       // the columns of Cbar (K = rows k..n) fill chunks 1.. of the block
       // column's slices; C^T is rows j..k of the L^T slices.

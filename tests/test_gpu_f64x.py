@@ -113,6 +113,19 @@ def test_factor_and_adjoint_match_the_oracle(n):
     assert rel(gp.chol_adjoint(dev(L), dev(Wt)).cpu().numpy(), O.chol_adjoint(L, Wt)) <= 1e-12
 
 
+@pytest.mark.parametrize("n", [321, 383, 447, 513])
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("mixed", 1e-8)])
+def test_panel_times_inverse_at_ragged_first_blocks(n, precision, tol):
+    # top-left blocks of 65, 127, 63 and 1 rows; a row of the upstream gradient far
+    # above the others must not cost them digits (each row has its own scale).
+    # fp64: as above; mixed: 2^-40 of a row's scale times condition about 1e4
+    K, Wt = problem(n, n)
+    Wt[n - 3] *= 2.0 ** 20
+    Wt[n - 2] *= 2.0 ** -20
+    L = O.chol(K)
+    assert rel(gp.chol_adjoint(dev(L), dev(Wt), precision).cpu().numpy(), O.chol_adjoint(L, Wt)) <= tol
+
+
 def test_minimal_workspace_takes_the_fp64_kernels():
     n = 500
     K, Wt = problem(n, 3)
