@@ -114,7 +114,7 @@ int gpc_workspace_min_size(int n, int precision, size_t *bytes);
 #define GPC_TUNE_BLOCK 0
 #define GPC_TUNE_SLICES 1
 #define GPC_TUNE_SPLITK_MIN 2
-#define GPC_TUNE_BATCH_BLOCK 3  /* block size inside gpc_batched_gp_lml_grad: 32 or 64 */
+#define GPC_TUNE_BATCH_BLOCK 3  /* block size inside the persistent launch of gpc_batched_gp_lml_grad: 32 or 64 */
 /* Mixed factorisation (GPC_MIXED): block columns (128 wide) whose trailing
  * updates are merged into one product with K = 128 x value (1..8, default 6;
  * enters the mixed workspace size); SMs its background products leave to the
@@ -438,12 +438,15 @@ int gpc_se_hyper_grad_workspace_size(int n, size_t *bytes);
 
 /*
  * Batched Gaussian-process likelihood and gradient for many independent GPs of
- * uneven size in one persistent launch.  The paper's batched diagonal
- * inverses (Section 3.2) give each small problem its own thread block; here
- * each thread block takes whole GPs from a device queue ordered by size,
- * largest first, and runs for each: the SE covariance of gpc_se_cov (jitter 0),
- * the Cholesky factorisation, the two solves, the log marginal likelihood of
- * gpc_gp_lml, Kbar of gpc_gp_lml_grad and the gradient of gpc_se_hyper_grad.
+ * uneven size: the SE covariance of gpc_se_cov (jitter 0), the Cholesky
+ * factorisation, the two solves, the log marginal likelihood of gpc_gp_lml,
+ * Kbar of gpc_gp_lml_grad and the gradient of gpc_se_hyper_grad.  It runs in one
+ * of two ways, chosen from batch and nmax.  Many small GPs: one persistent launch
+ * (the paper's batched diagonal inverses, Section 3.2, give each small problem its
+ * own thread block; here each thread block takes whole GPs from a device queue
+ * ordered by size, largest first).  Larger GPs, and batches of no more GPs than
+ * SMs: in lockstep, every member taking the same 128-wide block step in one launch,
+ * with its products on BF16 slices at FP64 accuracy in both precisions.
  * All arrays are device arrays:
  *   n[i]       order of GP i (1 <= n[i] <= nmax; larger sizes set info[i] to
  *              {-1, GPC_ERR_INVALID_ARG} on the device and skip the GP)
@@ -454,14 +457,16 @@ int gpc_se_hyper_grad_workspace_size(int n, size_t *bytes);
  *   value[i], grad3[3i..3i+2], info[2i..2i+1]  outputs per GP (info as for
  *              gpc_chol; a GP whose factorisation fails gets NaN outputs)
  * nmax: host int, at most 4096; workspace from gpc_batched_workspace_size
- * for the same precision (per SM room for Kbar, the kernel values, the
- * diagonal-block inverses and three vectors of order nmax; the mixed path
- * adds BF16 slice buffers of about 10 nmax^2 bytes, so an FP64 workspace is
- * too small for it).
+ * for the same precision.  The persistent launch needs, per SM, room for Kbar, the
+ * kernel values, the diagonal-block inverses and three vectors of order nmax; the
+ * mixed path adds BF16 slice buffers of about 10 nmax^2 bytes.  The lockstep way
+ * takes about 36 nmax^2 bytes per member, for the whole batch or for as many
+ * members per pass as 8 GB hold; a workspace that is too small for 64 members
+ * (and the batch) but large enough for the persistent launch gives that.
  * The panel solves of the factorisation and of the adjoint are products with
  * the inverses of the diagonal blocks (formed once per block, right after it
  * is factored), and the forward and backward solves apply the same inverses.
- * precision GPC_FP64: every step in FP64.  GPC_MIXED: the O(n^3) products
+ * precision GPC_FP64: every step at FP64 accuracy.  GPC_MIXED, persistent launch: the O(n^3) products
  * (trailing updates of the factorisation and the adjoint's block products)
  * run on the tensor cores as split-BF16 slice products with FP32 group sums
  * folded into double-float accumulators (Section 3.3's blocked algorithms

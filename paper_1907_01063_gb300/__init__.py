@@ -673,7 +673,7 @@ class Batch:
     sizes: host sequence of n_i; the covariance/factor of GP i occupies
     n_i^2 doubles of K at offK[i]; its inputs are rows rowX[i] .. of X and y.
     precision: "fp64" or "mixed"; the workspace is sized for it, and a batch
-    made for "fp64" cannot run the mixed path (its workspace is smaller).
+    made for "fp64" cannot run the mixed path (its workspace may be smaller).
     """
 
     def __init__(self, sizes, device=None, precision="fp64"):
@@ -712,7 +712,7 @@ class Batch:
 def batched_gp_lml_grad(batch: Batch, X: torch.Tensor, y: torch.Tensor, hyp: torch.Tensor,
                         precision=None):
     """Log marginal likelihood and (alpha, rho, sigma) gradient of every GP in
-    the batch in one launch; returns (value [batch], grad3 [batch, 3], info [batch, 2]).
+    the batch (one persistent launch, or block steps in lockstep); returns (value [batch], grad3 [batch, 3], info [batch, 2]).
     precision defaults to the batch's own."""
     precision = batch.precision if precision is None else precision
     if not (X.is_cuda and X.dtype == torch.float64 and X.dim() == 2 and X.is_contiguous()):
@@ -722,6 +722,8 @@ def batched_gp_lml_grad(batch: Batch, X: torch.Tensor, y: torch.Tensor, hyp: tor
     hyp = hyp.to(device=X.device, dtype=torch.float64).contiguous()
     if hyp.numel() != 3 * batch.batch:
         raise ValueError("hyp must have shape (batch, 3)")
+    if batch.batch and precision_code(precision) == GPC_MIXED != precision_code(batch.precision):
+        _check(GPC_ERR_INVALID_ARG, "gpc_batched_gp_lml_grad")  # made for fp64
     _check(capi.gpc_batched_gp_lml_grad(batch.batch, batch.nmax, batch.n.data_ptr(), batch.offK.data_ptr(),
                                         batch.rowX.data_ptr(), X.shape[1], X.data_ptr(), y.data_ptr(),
                                         hyp.data_ptr(), precision_code(precision), batch.K.data_ptr(),

@@ -552,7 +552,7 @@ constexpr int kBatchMaxN = 4096;
 
 int gpc_batched_workspace_size(int batch, int nmax, int precision, size_t *bytes) {
   if (!bytes || batch < 0 || nmax < 1 || nmax > kBatchMaxN || !valid_precision(precision)) return GPC_ERR_INVALID_ARG;
-  *bytes = batched_workspace_bytes(std::max(batch, 1), nmax, precision == GPC_MIXED);
+  *bytes = batched_full_workspace_bytes(std::max(batch, 1), nmax, precision == GPC_MIXED);
   return GPC_OK;
 }
 
@@ -568,7 +568,7 @@ int gpc_batched_gp_lml_grad(int batch, int nmax, const int *n, const long long *
       ws_bytes < batched_workspace_bytes(batch, nmax, mixed))
     return GPC_ERR_INVALID_ARG;
   return status_of(batched_gp_lml_grad(batch, n, offK, rowX, d, X, y, hyp, Kws, value, grad3, info, nmax, mixed,
-                                       ws, stream));
+                                       ws, ws_bytes, stream));
 }
 
 int gpc_se_hyper_grad_workspace_size(int n, size_t *bytes) {

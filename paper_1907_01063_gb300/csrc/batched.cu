@@ -1,5 +1,6 @@
 // Batched Gaussian-process likelihood and gradient: many independent GPs of
-// uneven size in one persistent launch.
+// uneven size in one persistent launch.  (Batches of larger GPs, and those with
+// less GPs than SMs, run in lockstep instead: batched_steps.cu; in_steps() below.)
 //
 // Each CTA takes whole GPs from a device queue ordered by size, largest
 // first (longest-processing-time-first), and runs the complete pass for that
@@ -47,6 +48,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 
 namespace gpc {
 namespace {
@@ -1047,6 +1049,29 @@ __global__ void order_kernel(int batch, const int *n, int *order) {
 
 }  // namespace
 
+// Whether the lockstep path (batched_steps.cu) is the faster one, from what the
+// host knows: the number of members and the largest order.  The kernel above
+// takes at least as long as its largest member (FP64: 26 ms at order 512, as the
+// cube; mixed: 12 ms, as the power 2.2), the lockstep path at least 4 us per
+// member, whatever its order.  With a member per SM or less the line is at order
+// 96: 152 members of orders 32 .. 96 take 0.62 ms here and 0.63 ms in lockstep,
+// 32 .. 128 1.04 and 0.72, 32 .. 512 26.6 and 4.8 (mixed 12.8 and 4.8).  With
+// more, small members fill the SMs: 400 of orders 32 .. 128 take 1.57 and 1.88,
+// 32 .. 200 3.10 and 3.12, 32 .. 300 7.2 and 5.0 (mixed 5.2 and 5.0), 32 .. 800
+// 93 and 22 (36 and 22); 512 of orders 64 .. 1024 200 and 45.
+bool in_steps(int batch, int nmax, bool mixed) {
+  if (batch <= sm_count()) return nmax > 96;
+  const double r = nmax / 512.0, alone_us = mixed ? 12.4e3 * std::pow(r, 2.2) : 26e3 * r * r * r;
+  return nmax >= 256 && 4.0 * batch <= alone_us;
+}
+constexpr int kMinPass = 64;  // a workspace for less members per pass (and less than the batch) keeps the kernel above
+
+size_t batched_full_workspace_bytes(int batch, int nmax, bool mixed) {
+  const size_t base = batched_workspace_bytes(batch, nmax, mixed);
+  if (!in_steps(batch, nmax, mixed)) return base;
+  return std::max(base, align_up((size_t)batch * sizeof(int), 1024) + 1024 + batched_steps_bytes(batch, nmax, base));
+}
+
 size_t batched_workspace_bytes(int batch, int nmax, bool mixed) {
   const size_t slot = (size_t)slot_elems(nmax, mixed);
   return align_up((size_t)sm_count() * slot * sizeof(double), 256) + align_up((size_t)batch * sizeof(int), 256) + 256;
@@ -1054,8 +1079,18 @@ size_t batched_workspace_bytes(int batch, int nmax, bool mixed) {
 
 cudaError_t batched_gp_lml_grad(int batch, const int *n, const long long *offK, const long long *rowX, int d,
                                 const double *X, const double *y, const double *hyp, double *K, double *value,
-                                double *grad3, int *info, int nmax, bool mixed, void *ws, cudaStream_t s) {
+                                double *grad3, int *info, int nmax, bool mixed, void *ws, size_t ws_bytes,
+                                cudaStream_t s) {
   if (batch <= 0) return cudaSuccess;
+  const size_t order_bytes = align_up((size_t)batch * sizeof(int), 1024);
+  if (in_steps(batch, nmax, mixed) && ws_bytes > order_bytes + 1024 &&
+      batched_steps_members(batch, nmax, ws_bytes - order_bytes - 1024) >= std::min(batch, kMinPass)) {
+    char *base = (char *)align_up((size_t)ws, 1024);
+    int *order = (int *)base;
+    GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 8.0 * batch, s, order_kernel<<<1, 256, 0, s>>>(batch, n, order));
+    return batched_steps(batch, n, offK, rowX, d, X, y, hyp, K, value, grad3, info, nmax, order, base + order_bytes,
+                         ws_bytes - order_bytes - 1024, s);
+  }
   const int nb = std::min(std::max(tuning().batch_block, 16), MAXB);
   const size_t slot = (size_t)slot_elems(nmax, mixed);
   char *p = (char *)ws;

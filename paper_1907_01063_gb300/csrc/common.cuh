@@ -393,6 +393,52 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
 // exponents at exps + 128 ib.
 cudaError_t f64x_split_blocks(int nblk, int first, const double *src, long long ld0, long long ld, long long off1,
                               long long stride, void *out, int *exps, cudaStream_t s);
+// The same two steps for `count` matrices of whole 128 blocks in one launch:
+// member z has nblk[z] block rows and takes part while nblk[z] > act; its rows
+// (columns, K) end 128 (nblk[z] - mb) (nb, kb) after the operand's start where mb
+// (nb, kb) is not negative.
+struct F64xBatch {
+  int count = 0;
+  const int *nblk = nullptr, *n = nullptr;  // n: rows (diag_batch; a block's other rows are the identity)
+  int act = 0, mb = -1, nb = -1, kb = -1;
+};
+struct F64xBatchSplit {
+  const double *src;              // element (r, k) of member z: src[z stride + r rs + k ks]
+  long long rs, ks, stride;
+  int M, K;
+  void *out;                      // member z's slices: rows z rows .. of a buffer of count rows x kpad
+  int rows, kpad, chunk0;
+  int tri;                        // as in F64xRow; 2: entries with k > r are zero, 3: symmetric, read from k <= r
+  bool wide;
+  int vec;                        // entries per member of the exponent arrays below
+  int *rexp_out;                  // as in F64xRow
+  const int *rexp;                // one exponent per member, rexp[z], less rexp_sub[r]
+  const int *rexp_sub, *kexp;
+  const int *rexps;               // ... or one per row
+  bool kexp_minus;                // kexp enters with -1
+  int *block_out;                 // one per member
+  bool skip_zero;                 // chunks left of the diagonal (tri = 1) are not written
+  const int *row_exps;
+};
+cudaError_t f64x_split_batch(const F64xBatch &b, const F64xBatchSplit &q, cudaStream_t s);
+struct F64xBatchGemm {
+  const void *A, *B;              // slices as f64x_split_batch leaves them
+  int a_rows, a_kpad, a_row0, a_k0, b_rows, b_kpad, b_row0, b_k0;
+  int M, N, chunks;
+  bool lower, wide;               // wide: C = the product, else C -= it
+  const int *ra, *ra_sub, *rb;    // ra_sub: ra has one exponent per member
+  int vec;
+  double *C;
+  long long ldc, sC;
+};
+cudaError_t f64x_gemm_batch(const F64xBatch &b, const F64xBatchGemm &g, int *err, cudaStream_t s);
+// rexp and cexp of f64x_lower_exps for every member (n rows and `vec` exponents at most).
+cudaError_t f64x_lower_exps_batch(const F64xBatch &b, int n, const double *L, long long ldl, long long stride, int vec,
+                                  int *rexp, int *cexp, cudaStream_t s);
+// Diagonal block ib of every member, whole 128 blocks: factor in place (failing pivots as potrf_diag into
+// info + 2 order[z]) and inverse (128 x 128 at out + z so).
+cudaError_t diag_batch(const F64xBatch &b, double *A, long long lda, long long sA, int ib, double *out, long long so,
+                       const int *order, int *info, cudaStream_t s);
 // gemm_f64 through checked split products where the size pays for the split
 // and ws (f64x_scratch_bytes, or less: more passes) allows; otherwise gemm_f64,
 // with ws as its split-K scratch.
@@ -444,9 +490,20 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
 // Batched per-GP pass (batched.cu); rowX[i] = first row of GP i in X (d per row) and y.
 // mixed: split-BF16 products for the O(n^3) work and FP64 refinement of alpha.
 size_t batched_workspace_bytes(int batch, int nmax, bool mixed);
+// Workspace that lets batched_gp_lml_grad run in lockstep where that is the faster way.
+size_t batched_full_workspace_bytes(int batch, int nmax, bool mixed);
 cudaError_t batched_gp_lml_grad(int batch, const int *n, const long long *offK, const long long *rowX, int d,
                                 const double *X, const double *y, const double *hyp, double *K, double *value,
-                                double *grad3, int *info, int nmax, bool mixed, void *ws, cudaStream_t s);
+                                double *grad3, int *info, int nmax, bool mixed, void *ws, size_t ws_bytes,
+                                cudaStream_t s);
+// The same in lockstep (batched_steps.cu): the workspace for one pass over the
+// batch, or for as many members as `floor` bytes (or 8 GB) hold; order: the
+// members' indices, largest first.
+size_t batched_steps_bytes(int batch, int nmax, size_t floor);
+int batched_steps_members(int batch, int nmax, size_t bytes);
+cudaError_t batched_steps(int batch, const int *n, const long long *offK, const long long *rowX, int d, const double *X,
+                          const double *y, const double *hyp, double *K, double *value, double *grad3, int *info,
+                          int nmax, const int *order, void *ws, size_t ws_bytes, cudaStream_t s);
 cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A, long long lda, void *ws,
                                int *err, cudaStream_t s, bool f64 = false);
 

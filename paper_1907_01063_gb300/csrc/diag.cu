@@ -39,6 +39,13 @@ __device__ __forceinline__ void dmma_16816(double (&c)[4], const double (&a)[8],
         "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]));
 }
 
+struct TriBatch {  // grid.z members (zero: one)
+  const int *n;
+  int ib;
+  long long sL, so;
+};
+// Rows of block ib of a member of order n: the rest of its 128 is the identity.
+__device__ __forceinline__ int member_rows(const int *n, int z, int ib) { return min(kMaxBlock, __ldg(n + z) - ib * kMaxBlock); }
 struct TriBlock {
   int j0, nb;
   double *dst;
@@ -55,7 +62,11 @@ __device__ __forceinline__ TriBlock tri_block(int ib, int n, int first, int b, d
 
 // grid.x blocks, grid.y sub-blocks of a block in twos (64 threads)
 __global__ void __launch_bounds__(64)
-trtri16_kernel(int n, const double *L, long long ldl, int first, int b, double *out, long long ldo) {
+trtri16_kernel(int n, const double *L, long long ldl, int first, int b, double *out, long long ldo, TriBatch q) {
+  if (q.n) n = first = member_rows(q.n, blockIdx.z, q.ib);
+  if (n <= 0) return;
+  L += blockIdx.z * q.sL;
+  out += blockIdx.z * q.so;
   __shared__ double sub_s[2][TI_NB][TI_NB + 1];
   const TriBlock t = tri_block(blockIdx.x, n, first, b, out, ldo);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, r0 = (2 * blockIdx.y + w) * TI_NB;
@@ -95,7 +106,11 @@ trtri16_kernel(int n, const double *L, long long ldl, int first, int b, double *
 }
 
 __global__ void __launch_bounds__(32 * TI_WARPS, 2)
-trtri_cols_kernel(int n, const double *L, long long ldl, int first, int b, double *out, long long ldo) {
+trtri_cols_kernel(int n, const double *L, long long ldl, int first, int b, double *out, long long ldo, TriBatch q) {
+  if (q.n) n = first = member_rows(q.n, blockIdx.z, q.ib);
+  if (n <= 0) return;
+  L += blockIdx.z * q.sL;
+  out += blockIdx.z * q.so;
   __shared__ double dinv[TI_WARPS][TI_NB][TI_NB + 1];
   __shared__ double rhs[TI_NB][TI_COLS + 1];
   __shared__ double xs[TI_WARPS][TI_NB][TI_COLS + 1];
@@ -158,6 +173,11 @@ trtri_cols_kernel(int n, const double *L, long long ldl, int first, int b, doubl
     // the diagonal sub-blocks are in place already
     if (c0 + c < nb && i >> 4 != k0) t.dst[(long long)i * t.ldd + c0 + c] = (i >> 4 > k0) ? xs[i >> 4][i & 15][c] : 0.0;
   }
+  if (q.n)  // the identity past the member's order
+    for (int idx = threadIdx.x; idx < kMaxBlock * TI_COLS; idx += blockDim.x) {
+      const int i = idx >> 3, c = c0 + (idx & 7);
+      if (i >= nb || c >= nb) t.dst[(long long)i * t.ldd + c] = i == c ? 1.0 : 0.0;
+    }
 }
 
 // An FP64 entry, or a double-float one (FP32 hi + lo in the same 8 bytes) when df.
@@ -361,6 +381,14 @@ potrf_diag_kernel(int nb, double *A, long long lda, int *info, int pivot_offset,
   potrf_block<128>(nb, A, lda, info, pivot_offset, df);
 }
 
+// Whole 128 blocks, one per member (grid.x).
+__global__ void __launch_bounds__(256)
+potrf_batch_kernel(double *A, long long lda, long long sA, const int *n, int ib, const int *order, int *info) {
+  const int z = blockIdx.x, nb = member_rows(n, z, ib);
+  if (nb <= 0) return;
+  potrf_block<128>(nb, A + z * sA, lda, info + 2 * __ldg(order + z), ib * 128, 0);
+}
+
 // Row-parallel triangular solve of an m x nb panel X (in place) against the
 // nb x nb lower block T (Section 3.3's panel step, by substitution instead of
 // a product with the inverse):
@@ -556,11 +584,12 @@ cudaError_t trtri_batched(int n, const double *L, long long ldl, int first, int 
     cfg.numAttrs = 1;
   }
   GPC_LAUNCH(GPC_TRACE_DIAG, (double)n * TI_NB * TI_NB / 3.0, 16.0 * (double)n * TI_NB, s,
-             trtri16_kernel<<<dim3((unsigned)nblk, (unsigned)((b + 31) / 32)), 64, 0, s>>>(n, L, ldl, first, b, out, ldo));
+             trtri16_kernel<<<dim3((unsigned)nblk, (unsigned)((b + 31) / 32)), 64, 0, s>>>(n, L, ldl, first, b, out, ldo,
+                                                                                                 TriBatch{}));
   if (b <= TI_NB) return cudaGetLastError();
   cudaError_t le = cudaSuccess;
   GPC_LAUNCH(GPC_TRACE_DIAG, (double)n * b * b / 3.0, 16.0 * (double)n * b, s,
-             le = cudaLaunchKernelEx(&cfg, trtri_cols_kernel, n, L, ldl, first, b, out, ldo));
+             le = cudaLaunchKernelEx(&cfg, trtri_cols_kernel, n, L, ldl, first, b, out, ldo, TriBatch{}));
   return le;
 }
 
@@ -583,6 +612,30 @@ cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_of
   }
   GPC_LAUNCH(GPC_TRACE_DIAG, (double)nb * nb * nb / 3.0, 16.0 * nb * nb, s,
              launch_k(potrf_diag_kernel, 1, 256, potrf_smem<128>(), s, nb, A, lda, info, pivot_offset, df ? 1 : 0));
+  return cudaGetLastError();
+}
+
+cudaError_t diag_batch(const F64xBatch &b, double *A, long long lda, long long sA, int ib, double *out, long long so,
+                       const int *order, int *info, cudaStream_t s) {
+  static bool attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+    cudaError_t e =
+        cudaFuncSetAttribute(potrf_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)potrf_smem<128>());
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = true;
+  }
+  constexpr int nb = kMaxBlock;
+  const double work = (double)b.count * nb * nb * nb / 3.0, bytes = 16.0 * b.count * nb * nb;
+  const TriBatch q{b.n, ib, sA, so};
+  GPC_LAUNCH(GPC_TRACE_DIAG, work, bytes, s,
+             potrf_batch_kernel<<<b.count, 256, potrf_smem<128>(), s>>>(A, lda, sA, b.n, ib, order, info));
+  GPC_LAUNCH(GPC_TRACE_DIAG, 0.0, bytes, s,
+             trtri16_kernel<<<dim3(1, nb / 32, (unsigned)b.count), 64, 0, s>>>(nb, A, lda, nb, nb, out, nb, q));
+  GPC_LAUNCH(GPC_TRACE_DIAG, work, bytes, s,
+             trtri_cols_kernel<<<dim3(1, nb / TI_COLS, (unsigned)b.count), 32 * TI_WARPS, 0, s>>>(nb, A, lda, nb, nb, out,
+                                                                                                  nb, q));
   return cudaGetLastError();
 }
 

@@ -102,7 +102,10 @@ struct FxParams {
   const int *ra, *rb;              // scale exponents of the output's rows and columns (null: 0), ...
   int ra_mul;                      // 0: one exponent for all rows, less ra_sub[row]
   const int *ra_sub;
+  int sub_stride;
   int ra_codes, rb_codes;          // ... or row_codes_kernel codes
+  const int *nblk;                 // non-null: F64xBatch
+  int act, mb, nb, kb;
   int ra_stride, rb_stride;        // per batch entry
   double *C;
   long long ldc, sC;
@@ -156,11 +159,17 @@ __device__ __forceinline__ Work work_item(const FxParams &p, int w) {
   if (p.kskip == KSKIP_ROWS_END) hi = min(hi, max(0, m0 + FX_BM + p.ksh_m + FX_CHUNK - 1) / FX_CHUNK);
   if (p.kskip == KSKIP_COLS_END) hi = min(hi, max(0, n0 + FX_BN + p.ksh_n + FX_CHUNK - 1) / FX_CHUNK);
   lo = min(lo, hi);
+  k.skip = false;
+  if (p.nblk) {
+    const int blocks = __ldg(p.nblk + k.b);
+    if (p.kb >= 0) hi = min(hi, max(0, blocks - p.kb));
+    k.skip = blocks <= p.act || (p.mb >= 0 && m0 >= FX_CHUNK * (blocks - p.mb)) ||
+             (p.nb >= 0 && n0 >= FX_CHUNK * (blocks - p.nb));
+  }
   const int per = (hi - lo + p.splits - 1) / p.splits;
   k.c0 = min(hi, lo + k.split * per);
   k.c1 = min(hi, k.c0 + per);
   k.none = lo >= hi;
-  k.skip = false;
   // The check skips tiles the row counts show to be safe (bit 0, not written by
   // this launch, so every warp of every K range decides alike), the product the
   // tiles left to the FP64 kernel.
@@ -217,6 +226,7 @@ __device__ __forceinline__ double triple_to_f64(float a, float b, float c, int s
   two_sum1(h, m, h, m);
   two_sum1(m, l, m, l);
   const uint32_t hb = __float_as_uint(h);
+  if (h == 0.f) return __longlong_as_double((long long)((unsigned long long)hb << 32));
   const int eb = (int)(hb >> 23) & 0xFF;
   if (eb >= 54 && eb <= 254 && (unsigned)(eb + 896 + sh - 2) <= 2042u) {
     const uint32_t sign = hb & 0x80000000u;
@@ -235,6 +245,13 @@ __device__ __forceinline__ double triple_to_f64(float a, float b, float c, int s
     return __longlong_as_double((long long)bits + (long long)d);
   }
   return scalbn((double)h + ((double)m + (double)l), sh);
+}
+
+// s + e == a + b, or a - b, exactly.
+template <bool NEG>
+__device__ __forceinline__ void fold2(f2x a, f2x b, f2x &s, f2x &e) {
+  if (NEG) two_diff2(a, b, s, e);
+  else two_sum2(a, b, s, e);
 }
 
 // ------------------------------------------------------------------ MMAs
@@ -540,103 +557,116 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const bool live = !p.flags || row0 >= p.M || colh >= p.N ||
                           p.flags[(size_t)k.b * p.flag_stride + (size_t)(4 * k.tm + q) * p.flag_ld + 2 * k.tn + half];
         const int ea = row0 + lane < p.M ? row_exp(p.ra, p.ra_codes, k.b * p.ra_stride + (row0 + lane) * p.ra_mul) -
-                                              (p.ra_sub ? __ldg(p.ra_sub + row0 + lane) : 0)
+                                              (p.ra_sub ? __ldg(p.ra_sub + k.b * p.sub_stride + row0 + lane) : 0)
                                         : 0;
         const int ebl = colh + lane < p.N ? row_exp(p.rb, p.rb_codes, k.b * p.rb_stride + colh + lane) : 0;
-        if (p.sub == 4) {
-          // Few tiles (the factorisation's chain): every CTA forms the whole tile
-          // but folds and writes only columns 8 cg .. + 7 of each warp's 32.  The
-          // whole epilogue is some 5000 instructions per warp and 60 KB of code,
-          // mostly fetched for this one pass.
-          const int cg = w & 3, col = colh + cg * FX_EPI_COLS + cl;
-          const int eb = __shfl_sync(0xffffffffu, ebl, cg * FX_EPI_COLS + cl);
-          f2x A[4], B[4], C[4];
-          uint32_t off = 0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) A[i] = B[i] = C[i] = 0ull;
-          if (add) {
-            double v[8];
+        if (p.sub == 4 || p.chunks == 1) {
+          // 8 columns of each warp's 32 at a time.  With few tiles (sub: the
+          // factorisation's chain) every CTA forms the whole tile but folds and
+          // writes only one such group; with one chunk the groups take turns.  Folding
+          // all 32 columns together needs some 5000 instructions per warp and 60 KB of
+          // code, which pays only where a tile's chunks run through it many times.
+          // (One chunk, 9.2e3 accumulated tiles of a batch: 38 -> 29 us per tile and SM.)
+          const int cg0 = p.sub == 4 ? w & 3 : 0, cg1 = p.sub == 4 ? cg0 + 1 : 4;
+          double v[8];
+          auto load = [&](int cg) {
+            const int col = colh + cg * FX_EPI_COLS + cl;
 #pragma unroll
             for (int it = 0; it < 8; ++it) {
               const int row = row0 + 4 * it + rl;
-              const bool in = row < p.M && col < p.N && !(p.lower && col + p.lower_off > row);
+              const bool in = interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row));
               v[it] = in ? base[(long long)row * ld + col] : 0.0;
             }
+          };
+          if (add) load(cg0);
+#pragma unroll 1
+          for (int cg = cg0; cg < cg1; ++cg) {
+            const int col = colh + cg * FX_EPI_COLS + cl;
+            const int eb = __shfl_sync(0xffffffffu, ebl, cg * FX_EPI_COLS + cl);
+            f2x A[4], B[4], C[4];
+            uint32_t off = 0;
 #pragma unroll
-            for (int it = 0; it < 8; ++it) {
-              float t0 = 0.f, t1 = 0.f, t2 = 0.f;
-              const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
-              if (!f64_to_triple(v[it], sh, t0, t1, t2)) off |= 1u << it;
-              const int at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
-              tb[at] = t0;
-              tb[at + 256] = t1;
-              tb[at + 512] = t2;
+            for (int i = 0; i < 4; ++i) A[i] = B[i] = C[i] = 0ull;
+            if (add) {
+#pragma unroll
+              for (int it = 0; it < 8; ++it) {
+                float t0 = 0.f, t1 = 0.f, t2 = 0.f;
+                const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
+                if (!f64_to_triple(v[it], sh, t0, t1, t2)) off |= 1u << it;
+                const int at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
+                tb[at] = t0;
+                tb[at + 256] = t1;
+                tb[at + 512] = t2;
+              }
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 8; i += 2) {
+                const int a0 = lane * FX_EPI_COLS + (i ^ (lane >> 2)), a1 = lane * FX_EPI_COLS + ((i + 1) ^ (lane >> 2));
+                A[i / 2] = pk2(tb[a0], tb[a1]);
+                B[i / 2] = pk2(tb[a0 + 256], tb[a1 + 256]);
+                C[i / 2] = pk2(tb[a0 + 512], tb[a1 + 512]);
+              }
+              __syncwarp();
+              if (cg + 1 < cg1) load(cg + 1);  // in flight while this group is folded
             }
-            __syncwarp();
+#pragma unroll 1
+            for (int c = k.c0; c < k.c1; ++c) {
+              if (cg == cg0) {
+                if (!mbar_wait(tfull, tphase, abort_flag, p.wait_ns)) { ok = false; break; }
+                tphase ^= 1;
+                fence_after();
+              }
+              float g[FX_GROUPS][8];
+#pragma unroll
+              for (int grp = 0; grp < FX_GROUPS; ++grp) tmem_ld8(taddr + (uint32_t)(grp * FX_BN + cg * 8), g[grp]);
+              tmem_wait_ld();
+#pragma unroll
+              for (int grp = 0; grp < FX_GROUPS; ++grp) pin8(g[grp]);
+              if (cg + 1 == cg1) {
+                fence_before();
+                __syncwarp();
+                if (lane < FX_GROUPS) mbar_arrive(gfree0 + 8 * lane);
+              }
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                f2x e, f;
+                auto part = [&](int q) { return pk2(g[q][2 * i], g[q][2 * i + 1]); };
+                C[i] = NEG ? sub2(C[i], part(6)) : add2(C[i], part(6));
+                C[i] = NEG ? sub2(C[i], part(5)) : add2(C[i], part(5));
+#pragma unroll
+                for (int q = 4; q >= 1; --q) {
+                  fold2<NEG>(B[i], part(q), B[i], e);
+                  C[i] = add2(C[i], e);
+                }
+                fold2<NEG>(A[i], part(0), A[i], e);
+                two_sum2(B[i], e, B[i], f);
+                C[i] = add2(C[i], f);
+              }
+            }
+            if (!ok) break;
+            if (!live) continue;
 #pragma unroll
             for (int i = 0; i < 8; i += 2) {
               const int a0 = lane * FX_EPI_COLS + (i ^ (lane >> 2)), a1 = lane * FX_EPI_COLS + ((i + 1) ^ (lane >> 2));
-              A[i / 2] = pk2(tb[a0], tb[a1]);
-              B[i / 2] = pk2(tb[a0 + 256], tb[a1 + 256]);
-              C[i / 2] = pk2(tb[a0 + 512], tb[a1 + 512]);
+              upk2(A[i / 2], tb[a0], tb[a1]);
+              upk2(B[i / 2], tb[a0 + 256], tb[a1 + 256]);
+              upk2(C[i / 2], tb[a0 + 512], tb[a1 + 512]);
             }
             __syncwarp();
-          }
-#pragma unroll 1
-          for (int c = k.c0; c < k.c1; ++c) {
-            if (!mbar_wait(tfull, tphase, abort_flag, p.wait_ns)) { ok = false; break; }
-            tphase ^= 1;
-            fence_after();
-            float g[FX_GROUPS][8];
-#pragma unroll
-            for (int grp = 0; grp < FX_GROUPS; ++grp) tmem_ld8(taddr + (uint32_t)(grp * FX_BN + cg * 8), g[grp]);
-            tmem_wait_ld();
-#pragma unroll
-            for (int grp = 0; grp < FX_GROUPS; ++grp) pin8(g[grp]);
-            fence_before();
-            __syncwarp();
-            if (lane < FX_GROUPS) mbar_arrive(gfree0 + 8 * lane);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              f2x e, f;
-              auto part = [&](int q) {
-                const f2x x = pk2(g[q][2 * i], g[q][2 * i + 1]);
-                return NEG ? x ^ 0x8000000080000000ull : x;
-              };
-              C[i] = add2(C[i], part(6));
-              C[i] = add2(C[i], part(5));
-#pragma unroll
-              for (int q = 4; q >= 1; --q) {
-                two_sum2(B[i], part(q), B[i], e);
-                C[i] = add2(C[i], e);
+#pragma unroll 4
+            for (int it = 0; it < 8; ++it) {
+              const int row = row0 + 4 * it + rl, at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
+              const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
+              if (interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row))) {
+                double *dst = base + (long long)row * ld + col;
+                double x = triple_to_f64(tb[at], tb[at + 256], tb[at + 512], sh);
+                if (off >> it & 1u) x = *dst + x;
+                *dst = x;
               }
-              two_sum2(A[i], part(0), A[i], e);
-              two_sum2(B[i], e, B[i], f);
-              C[i] = add2(C[i], f);
             }
+            __syncwarp();
           }
           if (!ok) break;
-          if (!live) continue;
-#pragma unroll
-          for (int i = 0; i < 8; i += 2) {
-            const int a0 = lane * FX_EPI_COLS + (i ^ (lane >> 2)), a1 = lane * FX_EPI_COLS + ((i + 1) ^ (lane >> 2));
-            upk2(A[i / 2], tb[a0], tb[a1]);
-            upk2(B[i / 2], tb[a0 + 256], tb[a1 + 256]);
-            upk2(C[i / 2], tb[a0 + 512], tb[a1 + 512]);
-          }
-          __syncwarp();
-#pragma unroll 4
-          for (int it = 0; it < 8; ++it) {
-            const int row = row0 + 4 * it + rl, at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
-            const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
-            if (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row)) {
-              double *dst = base + (long long)row * ld + col;
-              double v = triple_to_f64(tb[at], tb[at + 256], tb[at + 512], sh);
-              if (off >> it & 1u) v = *dst + v;
-              *dst = v;
-            }
-          }
-          __syncwarp();
           continue;
         }
         f2x fa[16], fb[16], fc[16];
@@ -689,17 +719,16 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           auto fold = [&](int g, float(&r)[32]) {
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-              f2x x = pk2(r[2 * i], r[2 * i + 1]);
-              if (NEG) x ^= 0x8000000080000000ull;
+              const f2x x = pk2(r[2 * i], r[2 * i + 1]);
               if (g >= 5) {
-                fc[i] = add2(fc[i], x);
+                fc[i] = NEG ? sub2(fc[i], x) : add2(fc[i], x);
               } else if (g >= 1) {
                 f2x e;
-                two_sum2(fb[i], x, fb[i], e);
+                fold2<NEG>(fb[i], x, fb[i], e);
                 fc[i] = add2(fc[i], e);
               } else {
                 f2x e, f;
-                two_sum2(fa[i], x, fa[i], e);
+                fold2<NEG>(fa[i], x, fa[i], e);
                 two_sum2(fb[i], e, fb[i], f);
                 fc[i] = add2(fc[i], f);
               }
@@ -792,6 +821,9 @@ struct FxOperand {
   int *counts;           // per row: entries of at least 2^-5 of the row's scale (null: not counted)
   int rexp_stride, tri, tri_off;
   int df;                // entries are FP32 pairs (hi, lo)
+  int vec;               // per batch entry of rexp_sub, row_exps and kexp; block_out has one each
+  const int *nblk;       // non-null: F64xBatch
+  int act, mb, kb, skip_zero;  // skip_zero: chunks of zeros only (tri = 1) are not written
   unsigned short *dst;
   long long plane, dst_stride;
 };
@@ -817,6 +849,13 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   const int c = blockIdx.x, r0 = ((int)blockIdx.y - (second ? p.blocks0 : 0)) * 8;
   const double *src = o.src + (long long)blockIdx.z * o.src_stride;
   const int kbeg = (c == 0) ? 0 : p.first + (c - 1) * FX_CHUNK;
+  if (o.nblk) {
+    const int blocks = __ldg(o.nblk + blockIdx.z);
+    if (blocks <= o.act || (o.mb >= 0 && r0 >= FX_CHUNK * (blocks - o.mb)) || (o.kb >= 0 && c >= blocks - o.kb) ||
+        (o.skip_zero && (c + 1) * FX_CHUNK <= r0))
+      return;
+  }
+  const size_t vec = (size_t)blockIdx.z * o.vec;
   const int klen = (c == 0) ? min(p.first, o.K) : min(FX_CHUNK, o.K - kbeg);
   const bool contig = o.ks == 1;
 #pragma unroll
@@ -827,7 +866,8 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     bool in = r < o.M && kk < klen;
     if (o.tri == 1) in = in && k >= r + o.tri_off;
     if (o.tri == 2) in = in && k <= r + o.tri_off;
-    const double *at = src + (long long)r * o.rs + (long long)k * o.ks;
+    const bool swap = o.tri == 3 && k > r;
+    const double *at = src + (long long)(swap ? k : r) * o.rs + (long long)(swap ? r : k) * o.ks;
     double v = 0.0;
     if (in && o.df) {
       const float2 q = *reinterpret_cast<const float2 *>(at);
@@ -846,7 +886,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     E = __ldg(o.rexp + (size_t)blockIdx.z * o.rexp_stride + (size_t)r * o.rexp_mul);
     if (p.codes) E = code_exponent(E);
     if (E < kNoExp) E = 0;  // no entry at all
-    if (o.rexp_sub) E -= __ldg(o.rexp_sub + r);
+    if (o.rexp_sub) E -= __ldg(o.rexp_sub + vec + r);
   }
   unsigned long long mant[4];
   int ex[4], emax = kNoExp, raw = kNoExp;
@@ -858,7 +898,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     int kx = 0;
     if (p.kexp) {
       const int k = kbeg + lane * 4 + i;
-      kx = (k < o.K) ? p.kexp_sign * __ldg(p.kexp + k) : 0;
+      kx = (k < o.K) ? p.kexp_sign * __ldg(p.kexp + vec + k) : 0;
     }
     neg |= (uint32_t)(u >> 63) << i;
     mant[i] = (u & ((1ull << 52) - 1)) | (1ull << 52);
@@ -887,7 +927,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   emax = __reduce_max_sync(0xffffffffu, emax);
   if (o.block_out) {
     raw = __reduce_max_sync(0xffffffffu, raw);
-    if (lane == 0 && raw > kNoExp && r < o.M) atomicMax(o.block_out, raw + __ldg(o.row_exps + r) - kBlockMargin);
+    if (lane == 0 && raw > kNoExp && r < o.M) atomicMax(o.block_out + blockIdx.z, raw + __ldg(o.row_exps + vec + r) - kBlockMargin);
   }
   int shift = 0;  // the row's own exponent, when it is found here
   if (o.rexp_out && r < o.M) {
@@ -1237,7 +1277,11 @@ __global__ void diag_exps_kernel(int n, const double *K, long long ldk, int *rex
   rexp[i] = (e > 0 && e < 2047) ? (e - 1022 + 1) >> 1 : 0;
 }
 // rexp[i]: exponent E, 2^E above the largest entry of row i of the lower triangle.  A warp per row.
-__global__ void __launch_bounds__(256) lower_row_exps_kernel(int n, const double *L, long long ldl, int *rexp) {
+__global__ void __launch_bounds__(256) lower_row_exps_kernel(int n, const double *L, long long ldl, int *rexp, const int *nblk, long long stride,
+                      int vec) {
+  if (nblk) n = FX_CHUNK * __ldg(nblk + blockIdx.z);
+  L += blockIdx.z * stride;
+  rexp += blockIdx.z * vec;
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;
   int m = 0;
@@ -1252,7 +1296,12 @@ __global__ void __launch_bounds__(256) lower_row_exps_kernel(int n, const double
 // cexp[c]: the same for column c of the rows scaled by 2^-rexp.  32 columns and
 // 64 rows per CTA; cexp holds large negative numbers on entry.
 __global__ void __launch_bounds__(256)
-lower_col_exps_kernel(int n, const double *L, long long ldl, const int *rexp, int *cexp) {
+lower_col_exps_kernel(int n, const double *L, long long ldl, const int *rexp, int *cexp, const int *nblk,
+                      long long stride, int vec) {
+  if (nblk) n = FX_CHUNK * __ldg(nblk + blockIdx.z);
+  L += blockIdx.z * stride;
+  rexp += blockIdx.z * vec;
+  cexp += blockIdx.z * vec;
   const int c = blockIdx.x * 32 + (threadIdx.x & 31), t0 = blockIdx.y * 64;
   if (c >= n || t0 + 63 < blockIdx.x * 32) return;
   int m = kNoExp;
@@ -1296,11 +1345,127 @@ cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, in
   cudaError_t e = cudaMemsetAsync(cexp, 0x80, (size_t)n * sizeof(int), s);
   if (e != cudaSuccess) return e;
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 4.0 * n * (n + 1.0), s,
-             launch_k(lower_row_exps_kernel, (unsigned)((n + 7) / 8), 256, 0, s, n, L, ldl, rexp));
+             launch_k(lower_row_exps_kernel, (unsigned)((n + 7) / 8), 256, 0, s, n, L, ldl, rexp, (const int *)nullptr, 0ll,
+                      0));
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 4.0 * n * (n + 1.0), s,
              launch_k(lower_col_exps_kernel, dim3((unsigned)((n + 31) / 32), (unsigned)((n + 63) / 64)), 256, 0, s, n, L,
-                      ldl, (const int *)rexp, cexp));
+                      ldl, (const int *)rexp, cexp, (const int *)nullptr, 0ll, 0));
   return cudaGetLastError();
+}
+cudaError_t f64x_lower_exps_batch(const F64xBatch &b, int n, const double *L, long long ldl, long long stride, int vec,
+                                  int *rexp, int *cexp, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(cexp, 0x80, (size_t)b.count * vec * sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  const double bytes = 4.0 * n * (n + 1.0) * b.count;
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, bytes, s,
+             launch_k(lower_row_exps_kernel, dim3((unsigned)((n + 7) / 8), 1, (unsigned)b.count), 256, 0, s, n, L, ldl,
+                      rexp, b.nblk, stride, vec));
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, bytes, s,
+             launch_k(lower_col_exps_kernel, dim3((unsigned)((n + 31) / 32), (unsigned)((n + 63) / 64), (unsigned)b.count),
+                      256, 0, s, n, L, ldl, (const int *)rexp, cexp, b.nblk, stride, vec));
+  return cudaGetLastError();
+}
+
+cudaError_t f64x_split_batch(const F64xBatch &b, const F64xBatchSplit &q, cudaStream_t s) {
+  if (b.count <= 0 || q.M <= 0 || q.K <= 0) return cudaSuccess;
+  if (q.M % FX_CHUNK || q.K % FX_CHUNK || (q.rexp_out && q.K != FX_CHUNK)) return cudaErrorInvalidValue;
+  static bool carve[2][64] = {};
+  const auto fx_split_kernel = q.wide ? f64x_split_kernel<kF64xWide, false> : f64x_split_kernel<kF64xSlices, false>;
+  if (cudaError_t e = carveout_max((const void *)fx_split_kernel, carve[q.wide]); e != cudaSuccess) return e;
+  FxSplit p = {};
+  FxOperand &o = p.op[0];
+  o.src = q.src;
+  o.rs = q.rs;
+  o.ks = q.ks;
+  o.src_stride = q.stride;
+  o.M = o.row_end = q.M;
+  o.K = q.K;
+  o.kpad = q.kpad;
+  o.rexp = q.rexp ? q.rexp : q.rexps;
+  o.rexp_mul = q.rexp ? 0 : 1;
+  o.rexp_sub = q.rexp_sub;
+  o.rexp_stride = q.rexp ? 1 : q.vec;
+  o.rexp_out = q.rexp_out;
+  o.block_out = q.block_out;
+  o.block_rows = q.block_out ? FX_CHUNK : 0;
+  o.row_exps = q.row_exps;
+  o.tri = q.tri;
+  o.vec = q.vec;
+  o.nblk = b.nblk;
+  o.act = b.act;
+  o.mb = b.mb;
+  o.kb = b.kb;
+  o.skip_zero = q.skip_zero ? 1 : 0;
+  o.dst = (unsigned short *)q.out + (long long)q.chunk0 * FX_CHUNK;
+  o.plane = (long long)b.count * q.rows * q.kpad;
+  o.dst_stride = (long long)q.rows * q.kpad;
+  p.first = FX_CHUNK;
+  p.kexp = q.kexp;
+  p.kexp_sign = q.kexp_minus ? -1 : 1;
+  p.blocks0 = q.M / 8;
+  const int S = q.wide ? kF64xWide : kF64xSlices;
+  if (q.block_out)
+    if (cudaError_t e = cudaMemsetAsync(q.block_out, 0x80, (size_t)b.count * sizeof(int), s); e != cudaSuccess) return e;
+  GPC_LAUNCH(GPC_TRACE_SPLIT, 0.0, (8.0 + 2.0 * S) * q.M * q.K * b.count, s,
+             launch_k(fx_split_kernel, dim3((unsigned)(q.K / FX_CHUNK), (unsigned)(q.M / 8), (unsigned)b.count), 256, 0,
+                      s, p));
+  return cudaGetLastError();
+}
+
+cudaError_t f64x_gemm_batch(const F64xBatch &b, const F64xBatchGemm &g, int *err, cudaStream_t s) {
+  if (b.count <= 0 || g.M <= 0 || g.N <= 0 || g.chunks <= 0) return cudaSuccess;
+  const int S = g.wide ? kF64xWide : kF64xSlices;
+  CUtensorMap ma, mb;
+  if (!make_map(&ma, g.A, g.a_kpad, b.count * g.a_rows, S, FX_BM) ||
+      !make_map(&mb, g.B, g.b_kpad, b.count * g.b_rows, S, FX_BN))
+    return cudaErrorInvalidValue;
+  FxParams p = {};
+  p.M = g.M;
+  p.N = g.N;
+  p.chunks = g.chunks;
+  p.qpc = FX_CHUNK / FX_BK;
+  p.a_row0 = g.a_row0;
+  p.b_row0 = g.b_row0;
+  p.a_k0 = g.a_k0;
+  p.b_k0 = g.b_k0;
+  p.a_rows = g.a_rows;
+  p.b_rows = g.b_rows;
+  p.lower = g.lower ? 1 : 0;
+  p.splits = 1;
+  p.tiles_m = (g.M + FX_BM - 1) / FX_BM;
+  p.tiles_n = (g.N + FX_BN - 1) / FX_BN;
+  p.per_batch = (int)count_tiles(p);
+  p.num_work = p.per_batch * b.count;
+  p.accumulate = g.wide ? 0 : 1;
+  p.ra = g.ra;
+  p.ra_mul = g.ra_sub ? 0 : 1;
+  p.ra_stride = g.ra_sub ? 1 : g.vec;
+  p.ra_sub = g.ra_sub;
+  p.sub_stride = g.vec;
+  p.rb = g.rb;
+  p.rb_stride = g.vec;
+  p.nblk = b.nblk;
+  p.act = b.act;
+  p.mb = b.mb;
+  p.nb = b.nb;
+  p.kb = b.kb;
+  p.C = g.C;
+  p.ldc = g.ldc;
+  p.sC = g.sC;
+  p.err = err;
+  p.gerr = error_word();
+  p.wait_ns = faults().wait_ns;
+  p.no_loads = faults().ozaki_no_loads;
+  p.sub = 1;
+  if (4 * p.num_work <= sm_count()) {
+    p.sub = 4;
+    p.num_work *= 4;
+  }
+  const int grid = std::min(p.num_work, sm_count());
+  const double mn = (g.lower ? 0.5 : 1.0) * g.M * (double)g.N * b.count;
+  const double flops = 2.0 * mn * g.chunks * FX_CHUNK * (S * (S + 1) / 2), bytes = 16.0 * mn;
+  return g.wide ? launch_product<kF64xWide, false, false>(ma, mb, p, grid, flops, bytes, s)
+                : launch_product<kF64xSlices, true, false>(ma, mb, p, grid, flops, bytes, s);
 }
 cudaError_t f64x_block_exp(int nb, const double *A, long long lda, const int *rexp, int *out, cudaStream_t s) {
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 8.0 * nb * nb, s, launch_k(block_exp_kernel, 1, 256, 0, s, nb, A, lda, rexp, out));

@@ -134,6 +134,12 @@ __device__ __forceinline__ void two_sum2(f2x a, f2x b, f2x &s, f2x &e) {
   const f2x bb = sub2(s, a);
   e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
+// s + e == a - b exactly.
+__device__ __forceinline__ void two_diff2(f2x a, f2x b, f2x &s, f2x &e) {
+  s = sub2(a, b);
+  const f2x bb = sub2(a, s);
+  e = sub2(sub2(a, add2(s, bb)), sub2(b, bb));
+}
 
 }  // namespace tc
 }  // namespace gpc
