@@ -1058,7 +1058,7 @@ __global__ void order_kernel(int batch, const int *n, int *order) {
 // 32 .. 128 1.04 and 0.72, 32 .. 512 26.6 and 4.8 (mixed 12.8 and 4.8).  With
 // more, small members fill the SMs: 400 of orders 32 .. 128 take 1.57 and 1.88,
 // 32 .. 200 3.10 and 3.12, 32 .. 300 7.2 and 5.0 (mixed 5.2 and 5.0), 32 .. 800
-// 93 and 22 (36 and 22); 512 of orders 64 .. 1024 200 and 45.
+// 93 and 22 (36 and 22); 512 of orders 64 .. 1024 200 and 43.
 bool in_steps(int batch, int nmax, bool mixed) {
   if (batch <= sm_count()) return nmax > 96;
   const double r = nmax / 512.0, alone_us = mixed ? 12.4e3 * std::pow(r, 2.2) : 26e3 * r * r * r;

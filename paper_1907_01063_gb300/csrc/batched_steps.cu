@@ -18,8 +18,8 @@
 // read it for the gradient and puts the factor there.  Members are taken in order
 // of size, largest first, in passes of as many as the workspace holds.
 //
-// 512 GPs of orders 64 .. 1024: 200 ms one CTA per GP, 45 ms here: 20 ms products
-// (195 launches; one 128-deep chunk per output tile, so their epilogues' instructions
+// 512 GPs of orders 64 .. 1024: 200 ms one CTA per GP, 43 ms here: 18 ms products
+// (195 launches; few 128-deep chunks per output tile, so their epilogues' instructions
 // bound them), 9 ms splits (3 TB/s), 5 ms covariance and 7 ms diagonal blocks (FP64
 // units), 2 ms gradient.  96 of orders 32 .. 512: 12.6 -> 3.8 ms.  Accuracy: the
 // likelihood's error against 64 bits is that of the kernel it replaces (5.9e-13).
@@ -425,31 +425,42 @@ cudaError_t batched_steps(int batch, const int *n, const long long *offK, const 
       g.sC = sC;
       return g;
     };
-    // ---- factorisation, right-looking
+    // ---- factorisation, left-looking: a block column takes all earlier ones' products
+    // at once, so that a tile's output is read and rounded once (right-looking, with one
+    // 128-deep chunk per visit, 512 GPs of orders 64 .. 1024 took 44.8 ms instead of 43.1).  The slices of L's block columns collect in the
+    // buffer of the adjoint's, rows scaled by the diagonal (mixed.cu).
+    TRY(f64x_diag_exps_batch(b, P, w.L, P, sL, P, w.rexp, s));
     for (int ib = 0; ib < nb; ++ib) {
       const int j = ib * SB, k = j + SB, M = P - k;
       double *D = w.L + (long long)j * P + j, *Di = w.inv + (size_t)ib * sb;
-      b.act = ib;
+      if (ib > 0) {
+        F64xBatchGemm g = {};
+        g.A = g.B = w.lt;
+        g.a_rows = g.b_rows = g.a_kpad = g.b_kpad = P;
+        g.a_row0 = g.b_row0 = j;
+        g.M = P - j;
+        g.N = SB;
+        g.chunks = ib;
+        g.lower = true;
+        g.ra = g.rb = w.rexp + j;
+        g.vec = P;
+        g.C = D;
+        g.ldc = P;
+        g.sC = sL;
+        TRY(product(ib, ib, -1, -1, g));
+      }
       TRY(diag_batch(b, D, P, sL, ib, Di, sinv, order + z0, info, s));
       if (M <= 0) continue;
       double *A21 = D + (long long)SB * P;
       TRY(split(ib + 1, -1, -1, rows_split(Di, SB, 1, sinv, SB, w.si, 2, true, w.iexp, SB)));
       TRY(split(ib + 1, ib + 1, -1, rows_split(A21, P, 1, sL, M, w.sx, 0, true, w.xexp, P)));
       TRY(product(ib + 1, ib + 1, -1, -1, wide_product(w.sx, P, w.xexp, w.si, w.iexp, M, false, A21, P, sL)));
-      TRY(split(ib + 1, ib + 1, -1, rows_split(A21, P, 1, sL, M, w.sc, 0, false, w.xexp, P)));
-      F64xBatchGemm g = {};
-      g.A = g.B = w.sc;
-      g.a_rows = g.b_rows = P;
-      g.a_kpad = g.b_kpad = SB;
-      g.M = g.N = M;
-      g.chunks = 1;
-      g.lower = true;
-      g.ra = g.rb = w.xexp;
-      g.vec = P;
-      g.C = A21 + SB;
-      g.ldc = P;
-      g.sC = sL;
-      TRY(product(ib + 1, ib + 1, ib + 1, -1, g));
+      F64xBatchSplit q = rows_split(A21, P, 1, sL, M, (unsigned short *)w.lt + (long long)k * P, 0, false, nullptr, P);
+      q.kpad = P;
+      q.chunk0 = ib;
+      q.rexps = w.rexp + k;
+      q.saturate = true;
+      TRY(split(ib + 1, ib + 1, -1, q));
     }
     // ---- solves, value and the upstream adjoint
     GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, mem, s,

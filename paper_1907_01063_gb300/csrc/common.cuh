@@ -416,6 +416,7 @@ struct F64xBatchSplit {
   const int *rexp_sub, *kexp;
   const int *rexps;               // ... or one per row
   bool kexp_minus;                // kexp enters with -1
+  bool saturate;                  // as in f64x_split
   int *block_out;                 // one per member
   bool skip_zero;                 // chunks left of the diagonal (tri = 1) are not written
   const int *row_exps;
@@ -432,6 +433,8 @@ struct F64xBatchGemm {
   long long ldc, sC;
 };
 cudaError_t f64x_gemm_batch(const F64xBatch &b, const F64xBatchGemm &g, int *err, cudaStream_t s);
+cudaError_t f64x_diag_exps_batch(const F64xBatch &b, int n, const double *K, long long ldk, long long stride, int vec,
+                                 int *rexp, cudaStream_t s);
 // rexp and cexp of f64x_lower_exps for every member (n rows and `vec` exponents at most).
 cudaError_t f64x_lower_exps_batch(const F64xBatch &b, int n, const double *L, long long ldl, long long stride, int vec,
                                   int *rexp, int *cexp, cudaStream_t s);

@@ -1,7 +1,7 @@
 // Diagonal-block kernels and elementwise helpers of the blocked factorisation.
 //
 // The small-block factorisation of Section 3.3 (potrf_la_kernel,
-// potrf_diag_kernel), the panel solve against a factored block
+// potrf_diag_kernel; potrf_batch_kernel for batches in lockstep), the panel solve against a factored block
 // (trsm_quad_kernel, trsm_rows_kernel) and the inverses of all diagonal blocks
 // (trtri_cols_kernel; the per-block inverses of Section 3.2).
 #include "common.cuh"

@@ -50,7 +50,7 @@
 // and 28 or 36 of 2 KiB of B per K = 16 step against 896 or 1152 cycles of MMA)
 // and the fold between chunks.  Measured: 4096^3 in 3.4 ms (S = 8, the product
 // launch 3.2 ms = 1546 BF16 TFLOP/s, 0.88 of the sustained rate) against 125 ms
-// for the FP64 kernel; 2000 x 1537 x 1025 and its reverse mode 1.02 against
+// for the FP64 kernel; 2000 x 1537 x 1025 and its reverse mode 0.96 against
 // 21.0 ms; largest error over sampled outputs 1.1e-17 sum |a||b| at 4096^3
 // against 3.2e-16.
 #include "common.cuh"
@@ -566,7 +566,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           // writes only one such group; with one chunk the groups take turns.  Folding
           // all 32 columns together needs some 5000 instructions per warp and 60 KB of
           // code, which pays only where a tile's chunks run through it many times.
-          // (One chunk, 9.2e3 accumulated tiles of a batch: 38 -> 29 us per tile and SM.)
+          // (One chunk, 9.2e3 accumulated tiles of a batch: 38 -> 24 us per tile and SM.)
           const int cg0 = p.sub == 4 ? w & 3 : 0, cg1 = p.sub == 4 ? cg0 + 1 : 4;
           double v[8];
           auto load = [&](int cg) {
@@ -1207,8 +1207,8 @@ cudaError_t f64x_split_blocks(int nblk, int first, const double *src, long long 
 
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
-                      double *partial, int *err, cudaStream_t s, int max_ctas, int kdepth, int max_items, const int *ra_sub,
-                      bool wide) {
+                      double *partial, int *err, cudaStream_t s, int max_ctas, int kdepth, int max_items,
+                      const int *ra_sub, bool wide) {
   if (M <= 0 || N <= 0 || chunks <= 0) return cudaSuccess;
   if (kdepth <= 0) kdepth = FX_CHUNK;
   if (kdepth > FX_CHUNK || kdepth % FX_BK || (wide && splits > 1)) return cudaErrorInvalidValue;
@@ -1269,7 +1269,11 @@ namespace {
 
 // e_i with K_ii < 4^e_i (|L_ij| <= sqrt(K_ii) < 2^e_i); 0 where K_ii is no
 // positive normal number (the factorisation fails there).
-__global__ void diag_exps_kernel(int n, const double *K, long long ldk, int *rexp) {
+__global__ void diag_exps_kernel(int n, const double *K, long long ldk, int *rexp, const int *nblk, long long stride,
+                                 int vec) {
+  if (nblk) n = FX_CHUNK * __ldg(nblk + blockIdx.z);
+  K += blockIdx.z * stride;
+  rexp += blockIdx.z * vec;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const unsigned long long u = (unsigned long long)__double_as_longlong(K[(long long)i * ldk + i]);
@@ -1338,7 +1342,8 @@ block_exp_kernel(int nb, const double *A, long long lda, const int *rexp, int *o
 
 cudaError_t f64x_diag_exps(int n, const double *K, long long ldk, int *rexp, cudaStream_t s) {
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 12.0 * n, s,
-             launch_k(diag_exps_kernel, (unsigned)((n + 255) / 256), 256, 0, s, n, K, ldk, rexp));
+             launch_k(diag_exps_kernel, (unsigned)((n + 255) / 256), 256, 0, s, n, K, ldk, rexp, (const int *)nullptr, 0ll,
+                      0));
   return cudaGetLastError();
 }
 cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, int *cexp, cudaStream_t s) {
@@ -1350,6 +1355,13 @@ cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, in
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 4.0 * n * (n + 1.0), s,
              launch_k(lower_col_exps_kernel, dim3((unsigned)((n + 31) / 32), (unsigned)((n + 63) / 64)), 256, 0, s, n, L,
                       ldl, (const int *)rexp, cexp, (const int *)nullptr, 0ll, 0));
+  return cudaGetLastError();
+}
+cudaError_t f64x_diag_exps_batch(const F64xBatch &b, int n, const double *K, long long ldk, long long stride, int vec,
+                                 int *rexp, cudaStream_t s) {
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 12.0 * n * b.count, s,
+             launch_k(diag_exps_kernel, dim3((unsigned)((n + 255) / 256), 1, (unsigned)b.count), 256, 0, s, n, K, ldk,
+                      rexp, b.nblk, stride, vec));
   return cudaGetLastError();
 }
 cudaError_t f64x_lower_exps_batch(const F64xBatch &b, int n, const double *L, long long ldl, long long stride, int vec,
@@ -1402,6 +1414,7 @@ cudaError_t f64x_split_batch(const F64xBatch &b, const F64xBatchSplit &q, cudaSt
   p.first = FX_CHUNK;
   p.kexp = q.kexp;
   p.kexp_sign = q.kexp_minus ? -1 : 1;
+  p.sat = q.saturate ? 1 : 0;
   p.blocks0 = q.M / 8;
   const int S = q.wide ? kF64xWide : kF64xSlices;
   if (q.block_out)

@@ -1,9 +1,8 @@
 // FP64 register-tiled GEMM on the FP64 tensor path (mma.sync m16n8k16 .f64).
 //
-// This is the workhorse of the FP64 blocked Cholesky (panel product with the
-// diagonal-block inverse, trailing update A22 -= L21 L21^T of Section 3.3) and
-// of the blocked adjoint sweep (the products of the reverse-mode procedure of
-// Section 3.3).  tcgen05 has no FP64 kind, so the FP64 tensor instruction on
+// Small products (the adjoint's symbolic step; the blocked Cholesky and adjoint of
+// Section 3.3 at small orders or without workspace for slices) and the output
+// blocks that a checked product on slices (f64x.cu) leaves to it.  tcgen05 has no FP64 kind, so the FP64 tensor instruction on
 // sm_103a is the warp-level DMMA; the m16n8k16 shape sustains the part's FP64
 // peak (about 1.05 TFLOP/s measured, the rate of plain DFMA at full occupancy)
 // with far fewer instructions and shared-memory operand reads than DFMA.

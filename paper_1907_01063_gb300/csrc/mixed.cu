@@ -5,8 +5,9 @@
 // same code on FP64 storage with the FP64-accurate products of f64x.cu (f64).
 //   forward: the trailing update A22 -= L21 L21^T;
 //   adjoint: Bbar -= Cbar R, Dbar -= Cbar^T C and Rbar -= [Dbar; Cbar]^T [R; B].
-// The diagonal-block factors, their inverses, the panel solves and the Dbar
-// symbolic step stay FP64.  Matrices that the split products update (the
+// The diagonal-block factors, their inverses, the factorisation's panel solves and
+// the Dbar symbolic step stay FP64; the adjoint's panels Cbar D^-1 are products with
+// the inverses at FP64 accuracy (f64x.cu).  Matrices that the split products update (the
 // trailing part of L, the not-yet-final part of Lbar) are held in
 // double-float storage (FP32 hi + lo in each 8-byte element); each block
 // column is read as FP64 when it becomes current (the diagonal factor and the
@@ -320,9 +321,8 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
   TRY(aux_for_device(&aux));
   // Within a step the Bbar update (rows below, columns left: the largest
   // product) runs on the auxiliary stream on all but tuning().mixed_adj_free_sms
-  // SMs (16 by default) while the
-  // caller's stream takes the rest of the Dbar chain (three small FP64
-  // products that fill only a few SMs) on the others; Rbar follows the chain
+  // SMs (16 by default; 8 to 32 differ by less than 2%) while the caller's stream
+  // takes the rest of the Dbar chain (three small FP64 products) on the others; Rbar follows the chain
   // and takes SMs as the Bbar update frees them, and the next step's Cbar,
   // which both updates write, waits for both.
   const int side = std::min(tuning().mixed_adj_free_sms, sm_count() / 2);
@@ -340,9 +340,10 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
       double *Cbar = A + (long long)k * lda + j;
       // Cbar <- Cbar D^{-1}, FP64 in and out on both paths: one product with the
       // block's inverse on eight slices (with seven the adjoint's error grows to
-      // twice that of a substitution).  (Two 64-wide substitutions with a
-      // product between them took 132 us at m = 8000 and 65 us at m = 500, this
-      // 40 and 22: the substitution is FP64 work, m 128^2 / 2 multiply-adds.)
+      // twice that of a substitution; with eight it is about half).  Over the sweep
+      // at n = 16384 the split takes 16 us and the product 37 us a step; two 64-wide
+      // substitutions, FP64 work of m 128^2 / 2 multiply-adds, took 52 us each in
+      // mid-sweep, and a split and a product between them.
       SliceBuf SX = slice_view(w.sx, m, 1);
       TRY(f64x_split(Cbar, lda, 1, m, nb, nb, SX, nullptr, nullptr, 0, false, s, 0, 0,
                      F64xRow{w.xexp, nullptr, nullptr, 0, 0, nullptr, df, true}));
