@@ -93,8 +93,8 @@ int gpc_version(void);
  * Workspace bytes that gpc_chol, gpc_chol_adjoint, gpc_gp_lml and
  * gpc_gp_lml_grad need for matrices of order n at `precision` with the
  * current tuning (gpc_set_tuning).  One workspace of this size serves any of
- * those calls with order <= n.  *bytes is a host pointer.
- * At precision GPC_FP64 and orders from 256 to 40960 this includes room for the
+ * those calls with order <= n, and one for GPC_MIXED those of GPC_FP64 as well.
+ * *bytes is a host pointer.  At orders from 256 to 40960 this includes room for the
  * BF16 slices on which the O(n^3) products run at FP64 accuracy
  * (gpc_workspace_size(16384) is 3.9 GB); every call also accepts the smaller
  * gpc_workspace_min_size and then uses the FP64 product kernels.

@@ -40,12 +40,13 @@ constexpr double kRefineTol = 1e-14;
 constexpr size_t kGemmWorkspace = size_t(256) << 20;  // gpc_gemm_workspace_size; 40 MB (split-K tiles) is accepted
 
 // FP64 calls run on slices where the workspace has room for them (gpc_workspace_size)
-// and on the FP64 kernels in the smaller workspace of gpc_workspace_min_size.
+// and on the FP64 kernels in the smaller workspace of gpc_workspace_min_size.  A
+// workspace for GPC_MIXED has that room too: callers share one between both precisions.
 size_t core_bytes(int n, int precision, bool slices) {
   size_t c = std::max(chol_workspace_bytes(n), adjoint_workspace_bytes(n));
   c = std::max(c, ltv_workspace_bytes(n));
   if (precision == GPC_MIXED) c = std::max(c, mixed_workspace_bytes(n));
-  else if (slices) c = std::max(c, mixed_workspace_bytes(n, true));
+  if (slices) c = std::max(c, mixed_workspace_bytes(n, true));
   return align_up(c, 256);
 }
 

@@ -140,6 +140,15 @@ def test_minimal_workspace_takes_the_fp64_kernels():
     assert rel(gp.gp_lml(dev(K), dev(y), ws=ws)["alpha"].cpu().numpy(), O.gp_lml(K, y)["alpha"]) <= 1e-11
 
 
+def test_a_mixed_workspace_serves_fp64_calls_on_slices():
+    n = 500
+    K, _ = problem(n, 3)
+    assert gp.workspace_size(n, "mixed") >= gp.workspace_size(n, "fp64")
+    own = gp.chol(dev(K))
+    shared = gp.chol(dev(K), ws=gp.workspace(n, "mixed"))
+    assert torch.equal(own, shared)  # the same route, so the same bits
+
+
 @pytest.mark.parametrize("spread", [0, 12, 40])
 @pytest.mark.parametrize("scale", [1.0, 2.0 ** -660, 2.0 ** 660])
 def test_diagonal_scaling_changes_nothing(spread, scale):
