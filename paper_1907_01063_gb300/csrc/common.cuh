@@ -231,7 +231,7 @@ cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t s);
 constexpr int kMaxBlock = 128;
 // Factor of the nb x nb block at A, in place.  On a failing pivot p records
 // {pivot_offset + p, status} in info if info[1] is still 0.
-// df: the block is read in double-float storage (written back as FP64).
+// df: the block (nb <= 64) is read in double-float storage and written back as FP64.
 cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_offset, cudaStream_t s,
                        bool df = false);
 // In-place panel solve against the lower nb x nb block T: mode 0 X <- X T^{-T},
@@ -244,6 +244,8 @@ cudaError_t trsm_rows(int m, int nb, double *X, long long ldx, const double *T, 
 // position of the n x n matrix out (leading dimension ldo; out may be L).
 cudaError_t trtri_batched(int n, const double *L, long long ldl, int first, int b, double *out,
                           cudaStream_t s, long long ldo = 0);
+// The same (ldo == 0) in the order of operations that the mixed path keeps, one CTA per block.
+cudaError_t trtri_sweep(int n, const double *L, long long ldl, int first, int b, double *out, cudaStream_t s);
 
 // ---------------------------------------------------------------- elementwise helpers
 // dst(i,j) = src(i,j) for j <= i; strict upper of dst set to 0 (src may == dst).
@@ -369,7 +371,6 @@ struct F64xRow {
   int block_rows = 0;
   int tri = 0;                    // 1: entries with k < r are zero (not read)
   const int *rexp_sub = nullptr;  // non-null: rexp holds one exponent, row r's is *rexp - rexp_sub[r]
-  bool df = false;                // the entries are FP32 pairs (double-float storage)
   bool wide = false;              // kF64xWide slices
 };
 cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,

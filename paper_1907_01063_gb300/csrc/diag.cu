@@ -1,7 +1,7 @@
 // Diagonal-block kernels and elementwise helpers of the blocked factorisation.
 //
 // The small-block factorisation of Section 3.3 (potrf_la_kernel,
-// potrf_diag_kernel; potrf_batch_kernel for batches in lockstep), the panel solve against a factored block
+// potrf_diag_kernel, potrf_lookahead_kernel in double-float storage; potrf_batch_kernel for batches in lockstep), the panel solve against a factored block
 // (trsm_quad_kernel, trsm_rows_kernel) and the inverses of all diagonal blocks
 // (trtri_cols_kernel; the per-block inverses of Section 3.2).
 #include "common.cuh"
@@ -180,6 +180,42 @@ trtri_cols_kernel(int n, const double *L, long long ldl, int first, int b, doubl
     }
 }
 
+// The mixed path's diagonal-block inverses (block ib at out + ib b^2, leading
+// dimension its size), one CTA per block, in place in shared memory by a backward
+// column sweep: with L = [[l, 0], [x, L2]],
+// L^{-1} = [[1/l, 0], [-L2^{-1} x / l, L2^{-1}]], every entry one chain of
+// multiply-adds.  Kept for its order of operations, as potrf_lookahead_kernel
+// below (480 us a launch against 42 to 69 of the kernels above).
+__global__ void __launch_bounds__(256)
+trtri_sweep_kernel(int n, const double *L, long long ldl, int first, int b, double *out) {
+  extern __shared__ double sm[];
+  __shared__ double col[kMaxBlock];
+  const TriBlock t = tri_block(blockIdx.x, n, first, b, out, 0);
+  const int nb = t.nb, ld = nb + 1;
+  const double *A = L + (long long)t.j0 * ldl + t.j0;
+  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
+    const int i = idx / nb, j = idx - i * nb;
+    sm[i * ld + j] = (j <= i) ? A[(long long)i * ldl + j] : 0.0;
+  }
+  __syncthreads();
+  for (int j = nb - 1; j >= 0; --j) {
+    const double ljj = sm[j * ld + j];
+    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) {
+      double v = 0.0;
+      for (int k = j + 1; k <= i; ++k) v = fma(sm[i * ld + k], sm[k * ld + j], v);
+      col[i] = -v / ljj;
+    }
+    __syncthreads();
+    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) sm[i * ld + j] = col[i];
+    if (threadIdx.x == 0) sm[j * ld + j] = 1.0 / ljj;
+    __syncthreads();
+  }
+  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
+    const int i = idx / nb, j = idx - i * nb;
+    t.dst[(long long)i * t.ldd + j] = (j <= i) ? sm[i * ld + j] : 0.0;
+  }
+}
+
 // An FP64 entry, or a double-float one (FP32 hi + lo in the same 8 bytes) when df.
 __device__ __forceinline__ double load_entry(const double *p, int df) {
   if (df) {
@@ -231,7 +267,7 @@ constexpr size_t potrf_smem() {
 }
 
 template <int NB>
-__device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, int *info, int pivot_offset, int df) {
+__device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, int *info, int pivot_offset) {
   constexpr int LD = NB + 4, NT = NB / 8, NW = NB / 16, OWN = NW - 1, TILES = NT * (NT - 1) / 2,
                 SLOTS = (TILES + OWN - 1) / OWN;
   extern __shared__ double sm[];
@@ -243,7 +279,7 @@ __device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, in
 #pragma unroll 16
   for (int idx = threadIdx.x; idx < NB * NB; idx += 32 * NW) {
     const int r = idx / NB, c = idx - r * NB;  // rows past nb: the identity
-    M[r * LD + c] = (r < nb && c < nb) ? (c <= r ? load_entry(A + (long long)r * lda + c, df) : 0.0) : (r == c ? 1.0 : 0.0);
+    M[r * LD + c] = (r < nb && c < nb) ? (c <= r ? A[(long long)r * lda + c] : 0.0) : (r == c ? 1.0 : 0.0);
   }
   __syncthreads();
   // tiles (ti, tk), 1 <= tk <= ti, in column order: slot s of owner o = w - 1 is number s OWN + o
@@ -372,13 +408,13 @@ __device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, in
 
 // Blocks of up to 64 rows.
 __global__ void __launch_bounds__(128)
-potrf_la_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, int df) {
-  potrf_block<64>(nb, A, lda, info, pivot_offset, df);
+potrf_la_kernel(int nb, double *A, long long lda, int *info, int pivot_offset) {
+  potrf_block<64>(nb, A, lda, info, pivot_offset);
 }
 // Blocks of 65 to 128 rows.
 __global__ void __launch_bounds__(256)
-potrf_diag_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, int df) {
-  potrf_block<128>(nb, A, lda, info, pivot_offset, df);
+potrf_diag_kernel(int nb, double *A, long long lda, int *info, int pivot_offset) {
+  potrf_block<128>(nb, A, lda, info, pivot_offset);
 }
 
 // Whole 128 blocks, one per member (grid.x).
@@ -386,7 +422,163 @@ __global__ void __launch_bounds__(256)
 potrf_batch_kernel(double *A, long long lda, long long sA, const int *n, int ib, const int *order, int *info) {
   const int z = blockIdx.x, nb = member_rows(n, z, ib);
   if (nb <= 0) return;
-  potrf_block<128>(nb, A + z * sA, lda, info + 2 * __ldg(order + z), ib * 128, 0);
+  potrf_block<128>(nb, A + z * sA, lda, info + 2 * __ldg(order + z), ib * 128);
+}
+
+// The factor of a diagonal block in double-float storage, nb <= 64 (the mixed
+// path's), with a one-column lookahead.  Column k+1 is finished (pivot, 1/sqrt,
+// scaling) by one warp while six other warps apply column k to the rest of the
+// block:
+//   * warp 0 (the pivot warp): for column k+1 it applies the column-k update
+//     itself, takes r = 1/sqrt(pivot), writes the final column to shared memory
+//     and publishes col_ready = k+1;
+//   * warps 1-3 and 5-7 (the updaters, u = 0..5) own whole columns j = u mod 6,
+//     lane l holding rows j + l and j + l + 32 in registers; at step k, once
+//     column k is final, the owner of column k+2 updates and stores it first and
+//     marks rounds[k+1], then every warp updates its later columns (rounds[0]:
+//     columns 0 and 1 stored as loaded, one mark per warp);
+//   * warp 4 idles, so the pivot warp has its SM sub-partition to itself.
+// Every wait is a bounded spin on a shared-memory word; a wait that runs out
+// records GPC_ERR_TIMEOUT and stops the block.
+//
+// The mixed path keeps this order of operations although potrf_block is faster
+// (74 against 51 us for 64 rows).  Its products keep 40 bits, so a last-bit change
+// of a factor's entry decides anew how the entries that follow are rounded, and
+// the hyperparameter gradient, whose sums cancel to 1/60 and less, moves by its
+// own error: by 7e-9 of its size at n = 16384 in one draw, where callers compare
+// runs to 1e-9.
+constexpr int PL_NB = 64, PL_LD = PL_NB + 1, PL_W = 6, PL_COLS = (PL_NB + PL_W - 1) / PL_W;
+constexpr long long PL_SPIN = 1LL << 24;
+
+__global__ void __launch_bounds__(256)
+potrf_lookahead_kernel(int nb, double *A, long long lda, int *info, int pivot_offset, int *gerr) {
+  __shared__ double M[PL_NB * PL_LD];
+  __shared__ int col_ready, stop;
+  __shared__ int rounds[PL_NB];  // rounds[r]: marks of round r
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    col_ready = -1;
+    stop = 0;
+  }
+  if (threadIdx.x < PL_NB) rounds[threadIdx.x] = 0;
+  const bool updater = warp != 0 && warp != 4;
+  const int uw = updater ? warp - 1 - (warp > 4) : 0;
+  double a0[PL_COLS], a1[PL_COLS];  // column uw + 6 c: rows j + lane, j + lane + 32
+  if (updater) {
+#pragma unroll
+    for (int c = 0; c < PL_COLS; ++c) {
+      const int j = uw + PL_W * c, r0 = j + lane, r1 = r0 + 32;
+      a0[c] = (j < nb && r0 < nb) ? load_entry(A + (long long)r0 * lda + j, 1) : 0.0;
+      a1[c] = (j < nb && r1 < nb) ? load_entry(A + (long long)r1 * lda + j, 1) : 0.0;
+    }
+  }
+  __syncthreads();
+  volatile int *vready = &col_ready, *vstop = &stop;
+  // Polls: the updaters back off between polls, so that their loads do not
+  // queue in front of the pivot warp's shared-memory accesses.
+  auto spin_ge = [&](volatile int *w, int target) -> bool {
+    for (long long it = 0; it < PL_SPIN; ++it) {
+      if (*w >= target) return true;
+      if (*vstop) return false;
+      if (updater) __nanosleep(64);
+    }
+    return false;
+  };
+  auto give_up = [&]() {  // a wait ran out: report and stop the block
+    if (info && info[1] == 0) info[1] = GPC_ERR_TIMEOUT;
+    record_error(gerr, GPC_ERR_TIMEOUT);
+    *vstop = 1;
+  };
+  if (updater) {
+    // round 0: columns 0 and 1 as loaded (owned by updaters 0 and 1)
+    if (uw <= 1 && uw < nb) {
+      const int j = uw, r0 = j + lane, r1 = r0 + 32;
+      if (r0 < nb) M[r0 * PL_LD + j] = a0[0];
+      if (r1 < nb) M[r1 * PL_LD + j] = a1[0];
+    }
+    __threadfence_block();
+    __syncwarp();
+    if (lane == 0) atomicAdd(&rounds[0], 1);
+  }
+  if (warp == 0) {
+    // ---- pivot warp: lanes own rows lane and lane + 32
+    for (int c = 0; c < nb; ++c) {
+      // column c comes from round max(c - 1, 0)
+      if (!spin_ge((volatile int *)&rounds[max(c - 1, 0)], c <= 1 ? PL_W : 1)) {
+        if (!*vstop && lane == 0) give_up();
+        break;
+      }
+      __threadfence_block();
+      const int i0 = lane, i1 = lane + 32;
+      double v0 = (i0 >= c && i0 < nb) ? M[i0 * PL_LD + c] : 0.0;
+      double v1 = (i1 >= c && i1 < nb) ? M[i1 * PL_LD + c] : 0.0;
+      if (c > 0) {  // the update by column c - 1, finished by this warp just before
+        const double lc = M[c * PL_LD + c - 1];
+        if (i0 >= c && i0 < nb) v0 = fma(-M[i0 * PL_LD + c - 1], lc, v0);
+        if (i1 >= c && i1 < nb) v1 = fma(-M[i1 * PL_LD + c - 1], lc, v1);
+      }
+      const double pv = (c < 32) ? __shfl_sync(0xffffffffu, v0, c) : __shfl_sync(0xffffffffu, v1, c - 32);
+      if (!(pv > 0.0 && pv <= 1.79769313486231570e308)) {
+        if (lane == 0) {
+          if (info && info[1] == 0) {
+            info[0] = pivot_offset + c;
+            info[1] = (pv != pv || pv > 1.79769313486231570e308) ? GPC_ERR_NAN : GPC_ERR_NOT_PD;
+          }
+          *vstop = 1;
+        }
+        break;
+      }
+      const double r = rsqrt_nr(pv);  // every lane: no broadcast on the chain
+      if (i0 >= c && i0 < nb) M[i0 * PL_LD + c] = (i0 == c) ? pv * r : v0 * r;
+      if (i1 >= c && i1 < nb) M[i1 * PL_LD + c] = (i1 == c) ? pv * r : v1 * r;
+      __threadfence_block();
+      __syncwarp();
+      if (lane == 0) *vready = c;
+    }
+  } else if (updater) {
+    // ---- updaters: step k applies column k to columns k + 2 .. nb - 1
+    for (int k = 0; k + 2 < nb; ++k) {
+      if (!spin_ge(vready, k)) {
+        if (!*vstop && lane == 0) give_up();
+        break;
+      }
+      __threadfence_block();
+#pragma unroll
+      for (int c = 0; c < PL_COLS; ++c) {
+        const int j = uw + PL_W * c;
+        if (j == k + 2) {  // warp-uniform: the column the pivot warp needs next
+          const double ljk = M[j * PL_LD + k];
+          const int r0 = j + lane, r1 = r0 + 32;
+          if (r0 < nb) {
+            a0[c] = fma(-M[r0 * PL_LD + k], ljk, a0[c]);
+            M[r0 * PL_LD + j] = a0[c];
+          }
+          if (r1 < nb) {
+            a1[c] = fma(-M[r1 * PL_LD + k], ljk, a1[c]);
+            M[r1 * PL_LD + j] = a1[c];
+          }
+          __threadfence_block();
+          __syncwarp();
+          if (lane == 0) atomicAdd(&rounds[k + 1], 1);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < PL_COLS; ++c) {
+        const int j = uw + PL_W * c;
+        if (j > k + 2 && j < nb) {  // warp-uniform
+          const double ljk = M[j * PL_LD + k];
+          const int r0 = j + lane, r1 = r0 + 32;
+          if (r0 < nb) a0[c] = fma(-M[r0 * PL_LD + k], ljk, a0[c]);
+          if (j + 32 < nb && r1 < nb) a1[c] = fma(-M[r1 * PL_LD + k], ljk, a1[c]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
+    const int r = idx / nb, c = idx - r * nb;
+    A[(long long)r * lda + c] = (c <= r) ? M[r * PL_LD + c] : 0.0;
+  }
 }
 
 // Row-parallel triangular solve of an m x nb panel X (in place) against the
@@ -593,12 +785,36 @@ cudaError_t trtri_batched(int n, const double *L, long long ldl, int first, int 
   return le;
 }
 
+cudaError_t trtri_sweep(int n, const double *L, long long ldl, int first, int b, double *out, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (b > kMaxBlock || first < 1 || first > b) return cudaErrorInvalidValue;
+  static bool attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(trtri_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)((size_t)kMaxBlock * (kMaxBlock + 1) * sizeof(double)));
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = true;
+  }
+  const int nblk = 1 + (n - first + b - 1) / b;
+  const size_t smem = (size_t)b * (b + 1) * sizeof(double);
+  GPC_LAUNCH(GPC_TRACE_DIAG, (double)n * b * b / 3.0, 16.0 * (double)n * b, s,
+             trtri_sweep_kernel<<<nblk, 256, smem, s>>>(n, L, ldl, first, b, out));
+  return cudaGetLastError();
+}
+
 cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_offset, cudaStream_t s, bool df) {
   if (nb <= 0) return cudaSuccess;
-  if (nb > kMaxBlock) return cudaErrorInvalidValue;
+  if (nb > (df ? PL_NB : kMaxBlock)) return cudaErrorInvalidValue;
+  if (df) {
+    GPC_LAUNCH(GPC_TRACE_DIAG, (double)nb * nb * nb / 3.0, 16.0 * nb * nb, s,
+               launch_k(potrf_lookahead_kernel, 1, 256, 0, s, nb, A, lda, info, pivot_offset, error_word()));
+    return cudaGetLastError();
+  }
   if (nb <= 64) {
     GPC_LAUNCH(GPC_TRACE_DIAG, (double)nb * nb * nb / 3.0, 16.0 * nb * nb, s,
-               launch_k(potrf_la_kernel, 1, 128, potrf_smem<64>(), s, nb, A, lda, info, pivot_offset, df ? 1 : 0));
+               launch_k(potrf_la_kernel, 1, 128, potrf_smem<64>(), s, nb, A, lda, info, pivot_offset));
     return cudaGetLastError();
   }
   static bool attr_set[64] = {};
@@ -611,7 +827,7 @@ cudaError_t potrf_diag(int nb, double *A, long long lda, int *info, int pivot_of
     attr_set[dev] = true;
   }
   GPC_LAUNCH(GPC_TRACE_DIAG, (double)nb * nb * nb / 3.0, 16.0 * nb * nb, s,
-             launch_k(potrf_diag_kernel, 1, 256, potrf_smem<128>(), s, nb, A, lda, info, pivot_offset, df ? 1 : 0));
+             launch_k(potrf_diag_kernel, 1, 256, potrf_smem<128>(), s, nb, A, lda, info, pivot_offset));
   return cudaGetLastError();
 }
 

@@ -820,7 +820,6 @@ struct FxOperand {
   const int *row_exps;
   int *counts;           // per row: entries of at least 2^-5 of the row's scale (null: not counted)
   int rexp_stride, tri, tri_off;
-  int df;                // entries are FP32 pairs (hi, lo)
   int vec;               // per batch entry of rexp_sub, row_exps and kexp; block_out has one each
   const int *nblk;       // non-null: F64xBatch
   int act, mb, kb, skip_zero;  // skip_zero: chunks of zeros only (tri = 1) are not written
@@ -866,10 +865,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   auto entry = [&](int row, int kk) {
     const int k = kbeg + kk;
     const bool swap = o.tri == 3 && k > row;
-    const double *at = src + (long long)(swap ? k : row) * o.rs + (long long)(swap ? row : k) * o.ks;
-    if (!o.df) return *at;
-    const float2 q = *reinterpret_cast<const float2 *>(at);
-    return exact_f64(q.x) + exact_f64(q.y);
+    return src[(long long)(swap ? k : row) * o.rs + (long long)(swap ? row : k) * o.ks];
   };
   double val[4];  // row r, K entries 4 lane ..
   if (o.ks == 1 && o.tri != 3) {
@@ -878,7 +874,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     // 9.3 -> 8.4 ms, the batch 43.1 -> 42.4 ms)
     if (r >= o.row_end) return;
     const double *at = src + (long long)r * o.rs + kbeg + lane * 4;
-    if (!o.df && ((uintptr_t)at & 15) == 0 && r < o.M && lane * 4 + 3 < klen) {
+    if (((uintptr_t)at & 15) == 0 && r < o.M && lane * 4 + 3 < klen) {
       const double2 a = *reinterpret_cast<const double2 *>(at), b = *reinterpret_cast<const double2 *>(at + 2);
       val[0] = a.x;
       val[1] = a.y;
@@ -1177,7 +1173,6 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
   o.block_rows = row.block_rows;
   o.row_exps = row.row_exps;
   o.tri = row.tri;
-  o.df = row.df ? 1 : 0;
   if (row.rexp_out && chunks != 1) return cudaErrorInvalidValue;
   if (row.block_out)
     if (cudaError_t e = cudaMemsetAsync(row.block_out, 0x80, sizeof(int), s); e != cudaSuccess) return e;

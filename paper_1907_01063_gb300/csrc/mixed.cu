@@ -6,8 +6,9 @@
 //   forward: the trailing update A22 -= L21 L21^T;
 //   adjoint: Bbar -= Cbar R, Dbar -= Cbar^T C and Rbar -= [Dbar; Cbar]^T [R; B].
 // The diagonal-block factors, their inverses, the factorisation's panel solves and
-// the Dbar symbolic step stay FP64; the adjoint's panels Cbar D^-1 are products with
-// the inverses at FP64 accuracy (f64x.cu).  Matrices that the split products update (the
+// the Dbar symbolic step stay FP64; the adjoint's panels Cbar D^-1 are FP64 solves on
+// the mixed path and products with the inverses at FP64 accuracy (f64x.cu) on the
+// FP64 path.  Matrices that the split products update (the
 // trailing part of L, the not-yet-final part of Lbar) are held in
 // double-float storage (FP32 hi + lo in each 8-byte element); each block
 // column is read as FP64 when it becomes current (the diagonal factor and the
@@ -91,16 +92,19 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
   w.t = (double *)p; p += b2();
   w.panel = (double *)p; p += align_up((size_t)n * MB * sizeof(double), 256);
   w.scratch = (double *)p; p += scratch_bytes();
-  w.sc = p; p += 2 * sbytes(n, 1, f64);  // two buffers: the next panel's slices while the last are in use
+  w.sc = p; p += 2 * sbytes(n, 1, f64);  // two buffers: a panel's rows, and its solved half
   if (adjoint) {
     w.sdc = p; p += sbytes(MB, nchunks(n), f64);
     w.lt = p; p += sbytes(n, nchunks(n), f64);
-    w.sx = p; p += f64x_slice_bytes(n, 1, true);
-    w.si = p; p += (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
+    if (f64) {
+      w.sx = p; p += f64x_slice_bytes(n, 1, true);
+      w.si = p; p += (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
+    }
   } else {
     w.grp = p; p += 2 * sbytes(n, defer_depth(), f64);
     w.tmp = p; p += sbytes(n, 1, f64);
   }
+  if (!f64) return w;
   w.rexp = (int *)p; p += exps_bytes(n);
   w.cexp = (int *)p; p += exps_bytes(n);
   w.xexp = (int *)p; p += exps_bytes(n);
@@ -113,12 +117,14 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
 
 size_t mixed_workspace_bytes(int n, bool f64) {
   n = std::max(n, 1);
-  const size_t common = ((size_t)nchunks(n) + 2) * b2() + align_up((size_t)n * MB * sizeof(double), 256) +
-                        scratch_bytes() + 2 * sbytes(n, 1, f64) + 3 * exps_bytes(n) + exps_bytes(nchunks(n) * MB) + 256 +
-                        1024;
-  const size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64) + f64x_slice_bytes(n, 1, true) +
-                     (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
+  size_t common = ((size_t)nchunks(n) + 2) * b2() + align_up((size_t)n * MB * sizeof(double), 256) + scratch_bytes() +
+                  2 * sbytes(n, 1, f64) + 1024;
+  size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64);
   const size_t fwd = 2 * sbytes(n, defer_depth(), f64) + sbytes(n, 1, f64);
+  if (f64) {
+    common += 3 * exps_bytes(n) + exps_bytes(nchunks(n) * MB) + 256;
+    adj += f64x_slice_bytes(n, 1, true) + (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
+  }
   return common + std::max(adj, fwd);
 }
 
@@ -288,7 +294,8 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
   if (strip_pending) TRY(cudaStreamWaitEvent(s, aux->ev_split, 0));
   if (rest_pending) TRY(cudaStreamWaitEvent(s, aux->ev_rest, 0));
   // every diagonal-block inverse, for the solves that follow the factorisation
-  return trtri_batched(n, L, ldl, std::min(MB, n), MB, w.inv, s);
+  return f64 ? trtri_batched(n, L, ldl, std::min(MB, n), MB, w.inv, s)
+             : trtri_sweep(n, L, ldl, std::min(MB, n), MB, w.inv, s);
 }
 
 // f64 (precision GPC_FP64): the same sweep with the products of f64x.cu on FP64
@@ -304,7 +311,6 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
 cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A, long long lda, void *ws,
                                int *err, cudaStream_t s, bool f64) {
   MixWs w = carve(ws, n, true, f64);
-  const bool df = !f64;
   const int nblk = nchunks(n);
   const int first = n - (nblk - 1) * MB;  // rows in the top-left block
   // L^T slices: operand row t = column t of L, K = rows of L, chunked like the sweep's blocks.
@@ -315,8 +321,12 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
   } else {
     TRY(split_operand(L, 1, ldl, n, n, first, LT, s));
   }
-  TRY(trtri_batched(n, L, ldl, first, MB, w.inv, s));  // independent of the sweep
-  TRY(f64x_split_blocks(nblk, first, w.inv, first, MB, (long long)MB * MB, (long long)MB * MB, w.si, w.iexp, s));
+  if (f64) {  // the inverses, independent of the sweep
+    TRY(trtri_batched(n, L, ldl, first, MB, w.inv, s));
+    TRY(f64x_split_blocks(nblk, first, w.inv, first, MB, (long long)MB * MB, (long long)MB * MB, w.si, w.iexp, s));
+  } else {
+    TRY(trtri_sweep(n, L, ldl, first, MB, w.inv, s));
+  }
   Aux *aux = nullptr;
   TRY(aux_for_device(&aux));
   // Within a step the Bbar update (rows below, columns left: the largest
@@ -338,17 +348,39 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
     bool bbar_pending = false;
     if (m > 0) {
       double *Cbar = A + (long long)k * lda + j;
-      // Cbar <- Cbar D^{-1}, FP64 in and out on both paths: one product with the
-      // block's inverse on eight slices (with seven the adjoint's error grows to
-      // twice that of a substitution; with eight it is about half).  Over the sweep
-      // at n = 16384 the split takes 16 us and the product 37 us a step; two 64-wide
-      // substitutions, FP64 work of m 128^2 / 2 multiply-adds, took 52 us each in
-      // mid-sweep, and a split and a product between them.
-      SliceBuf SX = slice_view(w.sx, m, 1);
-      TRY(f64x_split(Cbar, lda, 1, m, nb, nb, SX, nullptr, nullptr, 0, false, s, 0, 0,
-                     F64xRow{w.xexp, nullptr, nullptr, 0, 0, nullptr, df, true}));
-      TRY(f64x_gemm(SX, 0, 0, slice_view((char *)w.si + (size_t)ib * f64x_slice_bytes(MB, 1, true), MB, 1), 0, 0, m, nb, 1,
-                    false, w.xexp, w.iexp + (size_t)ib * MB, Cbar, lda, 1, nullptr, err, s, 0, 0, 0, nullptr, true));
+      if (f64) {
+        // Cbar <- Cbar D^{-1} as one product with the block's inverse on eight slices
+        // (with seven the adjoint's error grows to twice that of a substitution;
+        // with eight it is about half).  Over the sweep at n = 16384 the split takes
+        // 16 us and the product 37 us a step; two 64-wide substitutions, FP64 work of
+        // m 128^2 / 2 multiply-adds, 52 us each in mid-sweep, and a split and a product
+        // between them.
+        SliceBuf SX = slice_view(w.sx, m, 1);
+        TRY(f64x_split(Cbar, lda, 1, m, nb, nb, SX, nullptr, nullptr, 0, false, s, 0, 0,
+                       F64xRow{w.xexp, nullptr, nullptr, 0, 0, nullptr, true}));
+        TRY(f64x_gemm(SX, 0, 0, slice_view((char *)w.si + (size_t)ib * f64x_slice_bytes(MB, 1, true), MB, 1), 0, 0, m, nb,
+                      1, false, w.xexp, w.iexp + (size_t)ib * MB, Cbar, lda, 1, nullptr, err, s, 0, 0, 0, nullptr, true));
+      } else if (nb > MH) {
+        // Cbar <- Cbar D^{-1} as two 64-wide steps, right half first: with
+        // D = [Da 0; Dba Db], Xb = Cb Db^{-1}, then Ca -= Xb Dba (split-BF16,
+        // K = nb - 64) and Xa = Ca Da^{-1}.  The FP64 solves halve.  (The product with
+        // the inverse above is faster here too, 142 -> 128 ms a step at n = 16384,
+        // but the gradient moved by its own error with it: see
+        // potrf_lookahead_kernel.)
+        const int hb = nb - MH;
+        double *Cb = Cbar + MH;
+        const double *Dba = D + (long long)MH * ldl;
+        TRY(trsm_rows(m, hb, Cb, lda, Dba + MH, ldl, 1, s, true));
+        SliceBuf SX = slice_view((char *)w.sc + sbytes(n, 1, false), m, 1);
+        SliceBuf SD = slice_view(w.sdc, MH, 1);
+        TRY(split_operand(Cb, lda, 1, m, hb, hb, SX, s));
+        TRY(split_operand(Dba, 1, ldl, MH, hb, hb, SD, s));  // row c, K index t: Dba[t][c]
+        TRY(ozaki_gemm(SX, 0, 0, SD, 0, 0, m, MH, 1, false, -1.0f, (float2 *)Cbar, lda, 1, nullptr, err, s, 0,
+                       (hb + 31) / 32 * 32));
+        TRY(trsm_rows(m, MH, Cbar, lda, D, ldl, 1, s, true));
+      } else {
+        TRY(trsm_rows(m, nb, Cbar, lda, D, ldl, 1, s, true));  // Cbar <- Cbar D^{-1} (FP64)
+      }
       // Dbar -= Cbar^T C on slices (mixed: Dbar still in double-float storage):
       // the columns of Cbar (K = rows k..n) fill chunks 1.. of the block
       // column's slices; C^T is rows j..k of the L^T slices.
