@@ -25,6 +25,8 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <new>
+#include <vector>
 
 namespace gpc {
 namespace {
@@ -51,30 +53,116 @@ int defer_depth() { return std::max(1, std::min(tuning().mixed_defer, kMaxDefer)
 
 size_t b2() { return align_up((size_t)MB * MB * sizeof(double), 256); }
 
-// Per-device auxiliary stream and events for the factorisation's lookahead.
+// Auxiliary stream and events of one factorisation or adjoint.  A call leases a
+// set for as long as it enqueues: two host threads that shared one would record
+// each other's events between a record and its wait, and the background products
+// would start before their operands are written.  Sets stay with the caller's
+// stream that used them last, so that calls on different streams do not queue up
+// behind each other on a shared one, and one that a graph capture still holds goes
+// to callers in that capture only (any other call's work would be captured too).
 struct Aux {
   cudaStream_t st = nullptr;
   cudaEvent_t ev_split = nullptr, ev_rest = nullptr, ev_fork = nullptr;
+  cudaStream_t last = nullptr;  // the caller's stream of the last lease (compared only)
+  bool leased = false;
 };
+constexpr size_t kAuxKept = 8;  // sets kept per device; more exist only while that many calls enqueue at once
 std::mutex g_aux_mu;
-Aux g_aux[64];
+std::vector<Aux *> g_aux[64];
 
-cudaError_t aux_for_device(Aux **out) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> g(g_aux_mu);
-  Aux &a = g_aux[dev];
-  if (!a.st) {
-    if ((e = cudaStreamCreateWithFlags(&a.st, cudaStreamNonBlocking)) != cudaSuccess) return e;
-    if ((e = cudaEventCreateWithFlags(&a.ev_split, cudaEventDisableTiming)) != cudaSuccess) return e;
-    if ((e = cudaEventCreateWithFlags(&a.ev_rest, cudaEventDisableTiming)) != cudaSuccess) return e;
-    if ((e = cudaEventCreateWithFlags(&a.ev_fork, cudaEventDisableTiming)) != cudaSuccess) return e;
-  }
-  *out = &a;
-  return cudaSuccess;
+cudaError_t aux_create(Aux &a) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // creation is no part of any capture
+  const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+  cudaError_t e = cudaStreamCreateWithFlags(&a.st, cudaStreamNonBlocking);
+  for (cudaEvent_t *ev : {&a.ev_split, &a.ev_rest, &a.ev_fork})
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (swapped) cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
 }
+void aux_destroy(Aux *a) {
+  for (cudaEvent_t ev : {a->ev_split, a->ev_rest, a->ev_fork})
+    if (ev) cudaEventDestroy(ev);
+  if (a->st) cudaStreamDestroy(a->st);  // work in flight completes
+  delete a;
+}
+// 0: not capturing; otherwise the capture's id (all ones: an invalidated one).
+unsigned long long capture_id(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside a capture: the launches that follow report it
+    return 0;
+  }
+  return st == cudaStreamCaptureStatusNone ? 0 : (st == cudaStreamCaptureStatusActive ? id : ~0ull);
+}
+
+class AuxLease {
+ public:
+  explicit AuxLease(cudaStream_t s) : s_(s) {}
+  AuxLease(const AuxLease &) = delete;
+  AuxLease &operator=(const AuxLease &) = delete;
+  cudaError_t take(Aux **out) {
+    cudaError_t e = cudaGetDevice(&dev_);
+    if (e != cudaSuccess) return e;
+    if (dev_ < 0 || dev_ >= 64) return cudaErrorInvalidDevice;
+    const unsigned long long want = capture_id(s_);
+    std::lock_guard<std::mutex> g(g_aux_mu);
+    std::vector<Aux *> &pool = g_aux[dev_];
+    Aux *other = nullptr;
+    for (Aux *a : pool) {
+      if (a->leased) continue;
+      const unsigned long long held = capture_id(a->st);
+      if (held != 0 && held != want) continue;
+      if (a->last == s_) {
+        aux_ = a;
+        break;
+      }
+      if (!other) other = a;  // the one returned longest ago: returns go to the back
+    }
+    if (!aux_ && pool.size() >= kAuxKept) aux_ = other;
+    if (!aux_) {
+      Aux *a = new (std::nothrow) Aux;
+      if (!a) return cudaErrorMemoryAllocation;
+      if ((e = aux_create(*a)) != cudaSuccess) {
+        aux_destroy(a);
+        return e;
+      }
+      try {
+        pool.push_back(a);
+      } catch (...) {
+        aux_destroy(a);
+        return cudaErrorMemoryAllocation;
+      }
+      aux_ = a;
+    }
+    aux_->leased = true;
+    *out = aux_;
+    return cudaSuccess;
+  }
+  void joined() { joined_ = true; }
+  // Returned once the join is enqueued (after an error: joined here, so that the
+  // caller's stream still ends after everything that uses its buffers).
+  ~AuxLease() {
+    if (!aux_) return;
+    if (!joined_ && cudaEventRecord(aux_->ev_rest, aux_->st) == cudaSuccess) cudaStreamWaitEvent(s_, aux_->ev_rest, 0);
+    std::lock_guard<std::mutex> g(g_aux_mu);
+    std::vector<Aux *> &pool = g_aux[dev_];
+    pool.erase(std::find(pool.begin(), pool.end(), aux_));
+    if (pool.size() >= kAuxKept && capture_id(aux_->st) == 0) {
+      aux_destroy(aux_);
+      return;
+    }
+    aux_->leased = false;
+    aux_->last = s_;
+    pool.push_back(aux_);  // no allocation: one was just erased
+  }
+
+ private:
+  cudaStream_t s_;
+  int dev_ = 0;
+  Aux *aux_ = nullptr;
+  bool joined_ = false;
+};
 size_t scratch_bytes() { return std::max(gemm_f64_scratch_bytes(), kPartialCap); }
 int nchunks(int n) { return std::max(1, (n + MB - 1) / MB); }
 
@@ -173,8 +261,9 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
                : ozaki_gemm(A, ar, 0, B, br, 0, M, N, chunks, lower, -1.0f, (float2 *)C, ldl, 1, nullptr, e, st, ctas,
                             kdepth, items);
   };
+  AuxLease lease(s);
   Aux *aux = nullptr;
-  TRY(aux_for_device(&aux));
+  TRY(lease.take(&aux));
   const int D = defer_depth();
   const int nbc = nchunks(n);
   const int bg_ctas = std::max(1, sm_count() - std::max(0, std::min(tuning().mixed_free_sms, sm_count() / 2)));
@@ -293,6 +382,7 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
   while (rest_pending && slabs.next < slabs.count) TRY(launch_slab());
   if (strip_pending) TRY(cudaStreamWaitEvent(s, aux->ev_split, 0));
   if (rest_pending) TRY(cudaStreamWaitEvent(s, aux->ev_rest, 0));
+  lease.joined();
   // every diagonal-block inverse, for the solves that follow the factorisation
   return f64 ? trtri_batched(n, L, ldl, std::min(MB, n), MB, w.inv, s)
              : trtri_sweep(n, L, ldl, std::min(MB, n), MB, w.inv, s);
@@ -327,8 +417,9 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
   } else {
     TRY(trtri_sweep(n, L, ldl, first, MB, w.inv, s));
   }
+  AuxLease lease(s);
   Aux *aux = nullptr;
-  TRY(aux_for_device(&aux));
+  TRY(lease.take(&aux));
   // Within a step the Bbar update (rows below, columns left: the largest
   // product) runs on the auxiliary stream on all but tuning().mixed_adj_free_sms
   // SMs (16 by default; 8 to 32 differ by less than 2%) while the caller's stream
@@ -472,6 +563,7 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
       bbar_pending = false;
     }
   }
+  lease.joined();
   return cudaSuccess;
 }
 
