@@ -94,10 +94,13 @@ int gpc_version(void);
  * gpc_gp_lml_grad need for matrices of order n at `precision` with the
  * current tuning (gpc_set_tuning).  One workspace of this size serves any of
  * those calls with order <= n, and one for GPC_MIXED those of GPC_FP64 as well.
- * *bytes is a host pointer.  At orders from 256 to 40960 this includes room for the
+ * *bytes is a host pointer.  At orders from 321 to 40960 this includes room for the
  * BF16 slices on which the O(n^3) products run at FP64 accuracy
- * (gpc_workspace_size(16384) is 3.9 GB); every call also accepts the smaller
- * gpc_workspace_min_size and then uses the FP64 product kernels.
+ * (gpc_workspace_size(16384) is 3.9 GB).  Every call also accepts the smaller
+ * gpc_workspace_min_size: an FP64 call of those orders in a workspace that is
+ * smaller than its own gpc_workspace_size (one made for an order above 40960, say)
+ * runs on the FP64 product kernels, which are slower (257 ms against 5 s for a GP
+ * step of order 16384) and round differently.
  */
 int gpc_workspace_size(int n, int precision, size_t *bytes);
 int gpc_workspace_min_size(int n, int precision, size_t *bytes);

@@ -78,11 +78,13 @@ AdjWs carve_adj(void *ws, int n) {
 
 }  // namespace
 
-// Likelihood, adjoint and gradient in one pass (FP64 kernels / slices): 0.78 /
-// 0.81 ms at n = 200, 1.13 / 1.08 at 257, 2.50 / 2.10 at 513, 5.05 / 3.71 at 900,
-// 93 / 22.7 at 4096.  Above 40960 the slices of L^T (14 n^2 bytes) would take
+// Likelihood and adjoint in one pass, FP64 kernels / slices: 0.55 / 0.63 ms at
+// n = 160, 0.783 / 0.784 at 256, 0.95 / 1.00 at 257, 1.10 / 1.10 at 319, 1.03 / 1.07
+// at 320, 1.170 / 1.150 at 321, 1.23 / 1.18 at 384, 5.0 / 3.3 at 900, 93 / 19 at 4096:
+// slices are the slower side up to 320 (the same to 1% at 241 to 256) and the faster
+// one at every order above.  Above 40960 the slices of L^T (14 n^2 bytes) would take
 // more than 23 GB beside the caller's matrices.
-bool f64_on_slices(int n) { return (n >= 320 || n == 256) && n <= 40960; }
+bool f64_on_slices(int n) { return n > 320 && n <= 40960; }
 
 size_t chol_workspace_bytes(int n) {
   const size_t b = block_sz();

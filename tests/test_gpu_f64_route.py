@@ -1,0 +1,48 @@
+"""Which FP64 factorisations and adjoints run on BF16 slices: one threshold in the order, the same route in any
+workspace that is large enough."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1907_01063_gb300 as gp
+from oracle import oracle as O
+from paper_1907_01063_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+
+
+def kernels(fn):
+    torch.cuda.synchronize()
+    gp.trace_enable(True, timeline=True)
+    try:
+        out = fn()
+        torch.cuda.synchronize()
+    finally:
+        gp.trace_enable(False)
+    return out, [s["kernel"] for s in gp.trace_timeline()]
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("n,slices", [(255, False), (256, False), (257, False), (319, False), (320, False), (321, True),
+                                      (322, True), (383, True), (384, True)])
+def test_one_threshold(n, slices):
+    K = O.se_cov(W.gp_inputs(n, 3, n), 1.0, 1.0, 0.3, 1e-6)
+    Lo, Wt = O.chol(K), W.random_lower(n, n + 1)
+    for ws in (None, gp.workspace(700, "fp64"), gp.workspace(n, "mixed")):
+        L, names = kernels(lambda: gp.chol(dev(K), ws=ws))
+        assert any("f64x_gemm" in k for k in names) == slices
+        G, names = kernels(lambda: gp.chol_adjoint(dev(Lo), dev(Wt), ws=ws))
+        assert any("f64x_gemm" in k for k in names) == slices
+        # condition about 1e4 times the unit roundoff, as for the FP64 kernels
+        assert rel(L.cpu().numpy(), Lo) <= 1e-12 and rel(G.cpu().numpy(), O.chol_adjoint(Lo, Wt)) <= 1e-12
+        if ws is None:
+            first = L, G
+        else:
+            assert torch.equal(L, first[0]) and torch.equal(G, first[1])
