@@ -124,12 +124,13 @@ int gpc_workspace_min_size(int n, int precision, size_t *bytes);
  * FP64 chain (0..32, default 2); work items per CTA of a background product
  * (0 = one persistent CTA per SM, else 1..1024, so CTAs retire and the
  * chain's kernels get SMs); and whether the chain's launches take the
- * device's greatest stream priority (0 or 1, default 1). */
+ * device's greatest stream priority (0 or 1, default 1).  FP64 calls on slices
+ * always merge six block columns; the other three apply to them too. */
 #define GPC_TUNE_MIXED_DEFER 4
 #define GPC_TUNE_MIXED_FREE_SMS 5
 #define GPC_TUNE_MIXED_CTA_ITEMS 6
 #define GPC_TUNE_MIXED_PRIORITY 7
-/* Mixed adjoint: SMs its background products leave to the chain (0..64, default 16). */
+/* Adjoint on slices (both precisions): SMs its background products leave to the chain (0..64, default 16). */
 #define GPC_TUNE_MIXED_ADJ_FREE_SMS 8
 /* FP64 products (GEMM, factorisation and adjoint pieces): a single product
  * whose M and N are both at most this value takes 32 x 32 output tiles

@@ -49,7 +49,11 @@ struct MixWs {
   int *rexp, *cexp, *xexp, *iexp, *bexp;  // scale exponents: rows of L, its columns, panel rows, inverses, block column
 };
 constexpr int kMaxDefer = 8;
-int defer_depth() { return std::max(1, std::min(tuning().mixed_defer, kMaxDefer)); }
+// Block columns per deferred update.  The knob belongs to the mixed path: the FP64
+// path's workspace, and whether a call fits into one that was made before, must not
+// change with it.  Six is the tuner's choice at n = 16384.
+constexpr int kF64Defer = 6;
+int defer_depth(bool f64) { return f64 ? kF64Defer : std::max(1, std::min(tuning().mixed_defer, kMaxDefer)); }
 
 size_t b2() { return align_up((size_t)MB * MB * sizeof(double), 256); }
 
@@ -189,7 +193,7 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
       w.si = p; p += (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
     }
   } else {
-    w.grp = p; p += 2 * sbytes(n, defer_depth(), f64);
+    w.grp = p; p += 2 * sbytes(n, defer_depth(f64), f64);
     w.tmp = p; p += sbytes(n, 1, f64);
   }
   if (!f64) return w;
@@ -208,7 +212,7 @@ size_t mixed_workspace_bytes(int n, bool f64) {
   size_t common = ((size_t)nchunks(n) + 2) * b2() + align_up((size_t)n * MB * sizeof(double), 256) + scratch_bytes() +
                   2 * sbytes(n, 1, f64) + 1024;
   size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64);
-  const size_t fwd = 2 * sbytes(n, defer_depth(), f64) + sbytes(n, 1, f64);
+  const size_t fwd = 2 * sbytes(n, defer_depth(f64), f64) + sbytes(n, 1, f64);
   if (f64) {
     common += 3 * exps_bytes(n) + exps_bytes(nchunks(n) * MB) + 256;
     adj += f64x_slice_bytes(n, 1, true) + (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
@@ -264,7 +268,7 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
   AuxLease lease(s);
   Aux *aux = nullptr;
   TRY(lease.take(&aux));
-  const int D = defer_depth();
+  const int D = defer_depth(f64);
   const int nbc = nchunks(n);
   const int bg_ctas = std::max(1, sm_count() - std::max(0, std::min(tuning().mixed_free_sms, sm_count() / 2)));
   const int bg_items = std::max(0, tuning().mixed_cta_items);

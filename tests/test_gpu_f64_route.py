@@ -46,3 +46,18 @@ def test_one_threshold(n, slices):
             first = L, G
         else:
             assert torch.equal(L, first[0]) and torch.equal(G, first[1])
+
+
+@pytest.mark.parametrize("depth", [1, 8])
+def test_the_mixed_depth_knob_leaves_fp64_calls_alone(depth):
+    n = 900
+    K = dev(O.se_cov(W.gp_inputs(n, 3, 7), 1.0, 1.0, 0.3, 1e-6))
+    ws = gp.workspace(n, "fp64")
+    want, _ = kernels(lambda: gp.chol(K, ws=ws))
+    old = gp.get_tuning(gp.GPC_TUNE_MIXED_DEFER)
+    try:
+        gp.set_tuning(gp.GPC_TUNE_MIXED_DEFER, depth)
+        L, names = kernels(lambda: gp.chol(K, ws=ws))
+    finally:
+        gp.set_tuning(gp.GPC_TUNE_MIXED_DEFER, old)
+    assert any("f64x_gemm" in k for k in names) and torch.equal(L, want)
