@@ -363,7 +363,7 @@ constexpr float kF64xTheta = 0x1.7p-10f;
 size_t f64x_slice_bytes(int rows, int kchunks, bool wide = false);
 // The slices of split_operand, kF64xSlices of them, of the entries scaled by
 // 2^(kexp_sign kexp[k] - rexp[r]) (either may be null).  saturate: scaled
-// entries above 2^30 become 2^30, otherwise (and for NaN) NaN.
+// entries above 2^30 become 2^30, otherwise those from 2^100 on NaN; NaN stays NaN.
 struct F64xRow {
   int *rexp_out = nullptr;        // non-null (K within one chunk): rows scaled by their own largest entry, exponents here
   int *block_out = nullptr;       // non-null: the scale of all entries together, each with row_exps[r] added to its
@@ -372,6 +372,8 @@ struct F64xRow {
   int tri = 0;                    // 1: entries with k < r are zero (not read)
   const int *rexp_sub = nullptr;  // non-null: rexp holds one exponent, row r's is *rexp - rexp_sub[r]
   bool wide = false;              // kF64xWide slices
+  int *over_out = nullptr;        // with rexp_sub: entries of 2^100 and more raise this to the exponent they need
+  const int *alt = nullptr;       // with rexp_sub: such an exponent: split again with it, or nothing where *rexp covers it
 };
 cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,
                        const int *rexp, const int *kexp, int kexp_sign, bool saturate, cudaStream_t s,
@@ -382,12 +384,12 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
 cudaError_t f64x_diag_exps(int n, const double *K, long long ldk, int *rexp, cudaStream_t s);
 cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, int *cexp, cudaStream_t s);
 cudaError_t f64x_block_exp(int nb, const double *A, long long lda, const int *rexp, int *out, cudaStream_t s);
-// C (FP64) -= 2^(ra_i + rb_j) A B^T (with ra_sub: 2^(*ra - ra_sub_i + rb_j)),
+// C (FP64) -= 2^(ra_i + rb_j) A B^T (with ra_sub: 2^(max(*ra, *ra_alt) - ra_sub_i + rb_j)),
 // or with `wide` C = that product on kF64xWide slices; the other arguments as for ozaki_gemm.
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
                       double *partial, int *err, cudaStream_t s, int max_ctas = 0, int kdepth = 0, int max_items = 0,
-                      const int *ra_sub = nullptr, bool wide = false);
+                      const int *ra_sub = nullptr, bool wide = false, const int *ra_alt = nullptr);
 // Slices of the transposes of lower-triangular diagonal blocks (the first of order `first` at src with leading
 // dimension ld0, the others of order 128, `stride` apart from src + off1, with ld): operand row c = column c, scaled
 // by its own largest entry; block ib's kF64xWide slices at out + ib f64x_slice_bytes(128, 1, true), its scale

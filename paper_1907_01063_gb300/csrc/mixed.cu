@@ -47,6 +47,7 @@ struct MixWs {
   void *grp, *tmp;                        // factorisation: two group buffers, per-step temporaries
   void *sx, *si;                          // adjoint, eight slices: panel rows, diagonal-block inverses
   int *rexp, *cexp, *xexp, *iexp, *bexp;  // scale exponents: rows of L, its columns, panel rows, inverses, block column
+  int *oexp;                              // per block column: the exponent its finished block needs, if above bexp
 };
 constexpr int kMaxDefer = 8;
 // Block columns per deferred update.  The knob belongs to the mixed path: the FP64
@@ -201,7 +202,8 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
   w.cexp = (int *)p; p += exps_bytes(n);
   w.xexp = (int *)p; p += exps_bytes(n);
   w.iexp = (int *)p; p += exps_bytes(nchunks(n) * MB);
-  w.bexp = (int *)p;
+  w.bexp = (int *)p; p += 256;
+  w.oexp = (int *)p;
   return w;
 }
 
@@ -214,7 +216,7 @@ size_t mixed_workspace_bytes(int n, bool f64) {
   size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64);
   const size_t fwd = 2 * sbytes(n, defer_depth(f64), f64) + sbytes(n, 1, f64);
   if (f64) {
-    common += 3 * exps_bytes(n) + exps_bytes(nchunks(n) * MB) + 256;
+    common += 3 * exps_bytes(n) + exps_bytes(nchunks(n) * MB) + 256 + exps_bytes(nchunks(n));
     adj += f64x_slice_bytes(n, 1, true) + (size_t)nchunks(n) * f64x_slice_bytes(MB, 1, true);
   }
   return common + std::max(adj, fwd);
@@ -401,7 +403,10 @@ cudaError_t chol_mixed(int n, double *L, long long ldl, void *ws, int *info, cud
 // L' (cexp), panel rows of the adjoint (xexp, found by the split itself) and, for
 // its columns c, the block column's largest entry in equilibrated units less s_c
 // (bexp; each chunk of 128 keeps its own exponent, so this one only has to keep
-// FP32's range).
+// FP32's range).  The finished diagonal block D^-T sym(tril(D^T Dbar)) D^-1 may grow
+// past that range, by the square of the equilibrated block's inverse: its split then
+// reports the exponent it needs (oexp) and the block column is split again, in a
+// launch that otherwise ends at once.
 cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A, long long lda, void *ws,
                                int *err, cudaStream_t s, bool f64) {
   MixWs w = carve(ws, n, true, f64);
@@ -411,6 +416,7 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
   SliceBuf LT = slice_view(w.lt, n, nblk);
   if (f64) {
     TRY(f64x_lower_exps(n, L, ldl, w.rexp, w.cexp, s));
+    TRY(cudaMemsetAsync(w.oexp, 0x80, exps_bytes(nblk), s));
     TRY(f64x_split(L, 1, ldl, n, n, first, LT, w.cexp, w.rexp, -1, false, s, 0, 0, F64xRow{nullptr, nullptr, nullptr, 0, 1, nullptr}));
   } else {
     TRY(split_operand(L, 1, ldl, n, n, first, LT, s));
@@ -546,17 +552,23 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
       TRY(gemm_f64(d, w.scratch, s));
     }
     if (j > 0) {  // Rbar -= [Dbar; Cbar]^T [R; B] on slices (Rbar in double-float storage)
-      if (f64)  // chunk 0: the finished Dbar
-        TRY(f64x_split(Dbar, 1, lda, nb, nb, nb, SDC, w.bexp, w.rexp + j, 1, false, s, 0, 0,
-                       F64xRow{nullptr, nullptr, nullptr, 0, 0, w.rexp + j}));
-      else
+      if (f64) {  // chunk 0: the finished Dbar
+        F64xRow row;
+        row.rexp_sub = w.rexp + j;
+        row.over_out = w.oexp + ib;
+        TRY(f64x_split(Dbar, 1, lda, nb, nb, nb, SDC, w.bexp, w.rexp + j, 1, false, s, 0, 0, row));
+        row.over_out = nullptr;
+        row.alt = w.oexp + ib;
+        TRY(f64x_split(Dbar, 1, lda, nb, m + nb, nb, SDC, w.bexp, w.rexp + j, 1, false, s, 0, 0, row));
+      } else {
         TRY(split_operand(Dbar, 1, lda, nb, nb, nb, SDC, s, 0));
+      }
       const int tiles = (j + 63) / 64;
       int splits = std::max(1, std::min(chunks, (2 * sm_count() + tiles - 1) / tiles));
       while (splits > 1 && ozaki_partial_bytes(nb, j, splits) > kPartialCap) --splits;
       if (f64)
         TRY(f64x_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, w.bexp, w.cexp, A + (long long)j * lda, lda,
-                      splits, w.scratch, err, s, 0, 0, 0, w.rexp + j));
+                      splits, w.scratch, err, s, 0, 0, 0, w.rexp + j, false, w.oexp + ib));
       else
         TRY(ozaki_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, -1.0f, (float2 *)(A + (long long)j * lda),
                        lda, splits, (float2 *)w.scratch, err, s));
