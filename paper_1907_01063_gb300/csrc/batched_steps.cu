@@ -54,9 +54,10 @@ __device__ __forceinline__ int member_order(const Member &m, int gi) {
   return n < 1 || n > m.nmax ? 0 : n;  // sizes travel in device memory
 }
 
-// Blocks of every member of the pass (0: an order out of range), and its info.
-__global__ void steps_init_kernel(Member m, int count, int *nblk, int *nrow) {
+// Blocks of every member of the pass (0: an order out of range), and its info; err: no product has given up yet.
+__global__ void steps_init_kernel(Member m, int count, int *nblk, int *nrow, int *err) {
   const int z = blockIdx.x * blockDim.x + threadIdx.x;
+  if (z == 0) *err = GPC_OK;
   if (z >= count) return;
   const int gi = m.order[m.z0 + z], n = m.n[gi];
   const bool bad = n < 1 || n > m.nmax;
@@ -274,7 +275,10 @@ steps_grad_kernel(Member m, const double *Lw, const double *Kb, long long sL, do
   }
 }
 
-__global__ void __launch_bounds__(96) steps_grad_sum_kernel(Member m, const double *part, double *grad3) {
+// The gradient from the sums.  A product whose bounded wait gave up (err) served
+// every member of the pass: those still fine take its status, and NaN results.
+__global__ void __launch_bounds__(96)
+steps_grad_sum_kernel(Member m, const double *part, double *value, double *grad3, const int *err) {
   __shared__ double tot[3];
   const int gi = member_index(m), n = member_order(m, gi), w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (n == 0) return;
@@ -285,8 +289,12 @@ __global__ void __launch_bounds__(96) steps_grad_sum_kernel(Member m, const doub
   __syncthreads();
   if (threadIdx.x == 0) {
     const double al = m.hyp[3 * gi], rho = m.hyp[3 * gi + 1], sig = m.hyp[3 * gi + 2];
-    const bool bad = m.info[2 * gi + 1] != GPC_OK;
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
+    if (*err != GPC_OK && m.info[2 * gi + 1] == GPC_OK) {
+      m.info[2 * gi + 1] = *err;
+      value[gi] = nan;
+    }
+    const bool bad = m.info[2 * gi + 1] != GPC_OK;
     grad3[3 * gi] = bad ? nan : 2.0 * (tot[0] + tot[2] * (al * al)) / al;
     grad3[3 * gi + 1] = bad ? nan : tot[1] / (rho * rho * rho);
     grad3[3 * gi + 2] = bad ? nan : 2.0 * sig * tot[2];
@@ -297,7 +305,7 @@ __global__ void __launch_bounds__(96) steps_grad_sum_kernel(Member m, const doub
 struct StepWs {
   double *L, *Kb, *inv, *m, *t, *z, *a, *part;
   void *lt, *sc, *sdc, *sx, *si, *sy;
-  int *rexp, *cexp, *xexp, *iexp, *yexp, *bexp, *nblk, *n;
+  int *rexp, *cexp, *xexp, *iexp, *yexp, *bexp, *nblk, *n, *err;
   size_t bytes;
 };
 StepWs carve(void *ws, int count, int nmax) {
@@ -330,7 +338,8 @@ StepWs carve(void *ws, int count, int nmax) {
   w.yexp = (int *)take(Z * P * 4);
   w.bexp = (int *)take(Z * 4);
   w.nblk = (int *)take(Z * 4);
-  w.n = (int *)take(Z * 4);
+  w.n = (int *)take((Z + 1) * 4);
+  w.err = w.n + Z;
   w.bytes = p;
   return w;
 }
@@ -365,7 +374,7 @@ cudaError_t batched_steps(int batch, const int *n, const long long *offK, const 
     const dim3 rows(P / 8, 1, Z), one(1, 1, Z);
     const double mem = 8.0 * Z * P * (P + 1.0);
     GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 8.0 * Z, s,
-               launch_k(steps_init_kernel, (unsigned)((Z + 255) / 256), 256, 0, s, m, Z, w.nblk, w.n));
+               launch_k(steps_init_kernel, (unsigned)((Z + 255) / 256), 256, 0, s, m, Z, w.nblk, w.n, w.err));
     GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, mem, s, launch_k(steps_cov_kernel, rows, 256, 0, s, m, w.L, sL));
     F64xBatch b;
     b.count = Z;
@@ -382,7 +391,7 @@ cudaError_t batched_steps(int batch, const int *n, const long long *offK, const 
       b.mb = mb;
       b.nb = nb_;
       b.kb = kb;
-      return f64x_gemm_batch(b, g, nullptr, s);
+      return f64x_gemm_batch(b, g, w.err, s);
     };
     // Operand of whole 128 x 128 blocks or panels with each row's own scale
     auto rows_split = [&](const double *src, long long rs, long long ks, long long stride, int M, void *out, int tri,
@@ -598,7 +607,8 @@ cudaError_t batched_steps(int batch, const int *n, const long long *offK, const 
     GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 2.0 * mem, s,
                launch_k(steps_grad_kernel, rows, 256, 0, s, m, (const double *)w.L, (const double *)w.Kb, sL, w.part));
     GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 0.0, s,
-               launch_k(steps_grad_sum_kernel, one, 96, 0, s, m, (const double *)w.part, grad3));
+               launch_k(steps_grad_sum_kernel, one, 96, 0, s, m, (const double *)w.part, value, grad3,
+                        (const int *)w.err));
   }
   return cudaGetLastError();
 }

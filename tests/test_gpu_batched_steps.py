@@ -79,3 +79,24 @@ def test_failures_and_refused_orders_stay_with_their_member():
     _, _, info = gp.batched_gp_lml_grad(b, X, y, torch.as_tensor(hyps))
     assert info.cpu().tolist()[0] == [-1, gp.GPC_OK]
     assert [info.cpu().tolist()[i] for i in (1, 3)] == [[-1, gp.GPC_ERR_INVALID_ARG]] * 2
+
+
+def test_a_product_that_gives_up_is_reported_per_member():
+    sizes = [300, 140, 200]
+    Xs, ys, hyps = make_batch(sizes, seed=6)
+    Xs[2][150] = np.nan
+    gp.get_error(clear=True)
+    try:
+        gp.set_test_fault(gp.GPC_TEST_WAIT_NS, 1_000_000)
+        gp.set_test_fault(gp.GPC_TEST_OZAKI_NO_LOADS, 1)
+        _, v, g, info = run_batch(sizes, Xs, ys, hyps)
+    finally:
+        gp.set_test_fault(gp.GPC_TEST_WAIT_NS, 0)
+        gp.set_test_fault(gp.GPC_TEST_OZAKI_NO_LOADS, 0)
+    assert gp.get_error(clear=True) == gp.GPC_ERR_TIMEOUT
+    assert info[0].tolist() == [-1, gp.GPC_ERR_TIMEOUT] and info[1].tolist() == [-1, gp.GPC_ERR_TIMEOUT]
+    assert info[2, 1] in (gp.GPC_ERR_NAN, gp.GPC_ERR_TIMEOUT)  # the product may be what should have met the NaN
+    assert np.all(np.isnan(v)) and np.all(np.isnan(g))
+    b, v, g, info = run_batch(sizes, Xs, ys, hyps)
+    check(sizes, Xs, ys, hyps, b, v, g, info, (0, 1))
+    assert info[2].tolist() == [150, gp.GPC_ERR_NAN] and gp.get_error() == gp.GPC_OK
