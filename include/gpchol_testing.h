@@ -38,6 +38,8 @@ int gpc_test_ozaki_gemm(int M, int N, int K, const double *A, const double *B, d
  * the plain division and square root.
  */
 int gpc_test_recip_rsqrt(int n, const double *x, double *out, gpc_stream_t stream);
+/* out[i]: the reciprocal the FP64 diagonal-block factor takes of a pivot x_i (x_i and 1/x_i normal). */
+int gpc_test_recip_cubic(int n, const double *x, double *out, gpc_stream_t stream);
 
 /*
  * The FP64 -> double-float conversion of the mixed path (the split of every

@@ -142,7 +142,8 @@ __device__ __forceinline__ void record_error(int *word, int status) {
 // within 2 ulp of the correctly rounded value, checked against CUDA's 1.0 / x
 // and rsqrt over the normal range by gpc_test_recip_rsqrt's test; recip_nr
 // needs 1/x normal too, x < 2^1022, which holds for any pivot of a matrix whose
-// entries are below 2^511).  FP64 instructions are scarce on this part, so this
+// entries are below 2^511; the batched kernel's, the single matrix's has its own,
+// recip_cubic in diag.cu).  FP64 instructions are scarce on this part, so this
 // short dependent chain is what the diagonal factorisation's serial part waits on.
 __device__ __forceinline__ double recip_nr(double x) {
   if (!(x >= 2.2250738585072014e-308)) return 1.0 / x;
@@ -261,6 +262,8 @@ cudaError_t lower_to_symmetric_half(int n, double *A, long long lda, cudaStream_
 cudaError_t reset_info(int *info, cudaStream_t s);
 // Test hook: out[4 i ..] = {recip_nr(x_i), 1.0 / x_i, rsqrt_nr(x_i), rsqrt(x_i)}.
 cudaError_t recip_rsqrt_probe(int n, const double *x, double *out, cudaStream_t s);
+// out[i] = the reciprocal that the diagonal-block factor takes of a pivot x_i.
+cudaError_t recip_cubic_probe(int n, const double *x, double *out, cudaStream_t s);
 
 // ---------------------------------------------------------------- drivers
 // Fused GLM likelihood and gradient (glm.cu).

@@ -247,17 +247,19 @@ __device__ __forceinline__ double load_entry(const double *p, int df) {
 // GPC_ERR_NAN for NaN/Inf) and the rest of the block is written back unfinished.
 // Measured: 64 rows 74 -> 51 us against a column-by-column lookahead with one
 // pivot warp (square roots and two row halves on the chain), 128 rows 250 -> 170.
-// 1/x to about 2 ulp: the hardware seed and one third-order step y (1 + e + e^2).
+// 1/x within 2 ulp for x and 1/x normal: the hardware seed and one third-order
+// Householder step for the reciprocal, y (1 + e + e^2) with e = 1 - x y (pinned
+// beside the other refinements by gpc_test_recip_cubic's test).
 __device__ __forceinline__ double recip_cubic(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
-// Positive, finite and normal, by the high word (a comparison of FP64 values
-// would take the FP64 pipe).
-__device__ __forceinline__ bool normal_positive(double x) {
-  return (unsigned)(__double2hiint(x) - 0x00100000) < 0x7FE00000u;
+// Positive and normal with a normal reciprocal (x < 2^1022), by the high word (a
+// comparison of FP64 values would take the FP64 pipe).
+__device__ __forceinline__ bool plain_pivot(double x) {
+  return (unsigned)(__double2hiint(x) - 0x00100000) < 0x7FC00000u;
 }
 
 constexpr int kPotrfW = 12;  // row of W: 8 entries, padded against bank conflicts
@@ -273,9 +275,17 @@ __device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, in
   extern __shared__ double sm[];
   double *M = sm, *W = sm + NB * LD, *Wd = W + NB * kPotrfW, *pinv_s = Wd + 8 * 9;
   __shared__ int fail;  // failing column, or NB
+  // Pivots beyond plain_pivot: 1/d is pinv sc sc, sc a power of two applied in two
+  // steps, since 1/d itself would overflow (denormal pivots) or lose its digits.
+  __shared__ double sc_s[NB];
+  __shared__ int scaled;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tr = lane >> 2, tc = lane & 3;  // row and column pair of an 8 x 8 tile
-  if (threadIdx.x == 0) fail = NB;
+  if (threadIdx.x == 0) {
+    fail = NB;
+    scaled = 0;
+  }
+  if (threadIdx.x < NB) sc_s[threadIdx.x] = 1.0;
 #pragma unroll 16
   for (int idx = threadIdx.x; idx < NB * NB; idx += 32 * NW) {
     const int r = idx / NB, c = idx - r * NB;  // rows past nb: the identity
@@ -323,7 +333,7 @@ __device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, in
       for (int j = 0; j < 8; ++j) {
         const double aj = j < 4 ? a0 : a1;
         const double d = __shfl_sync(0xffffffffu, aj, j * 4 + (j & 3));
-        const bool fine = normal_positive(d);
+        const bool fine = plain_pivot(d);
         if (ok && !fine && !(d > 0.0 && d <= 1.79769313486231570e308)) {
           ok = false;
           if (lane == 0) {
@@ -338,7 +348,19 @@ __device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, in
         const double aij = __shfl_sync(0xffffffffu, aj, (lane & ~3) | (j & 3));
         const double k0 = __shfl_sync(0xffffffffu, aj, q * 4 + (j & 3));
         const double k1 = __shfl_sync(0xffffffffu, aj, (q + 4) * 4 + (j & 3));
-        const double pinv = fine ? recip_cubic(d) : 1.0 / d, t = aij * pinv;
+        double pinv, t;
+        if (fine) {
+          pinv = recip_cubic(d);
+          t = aij * pinv;
+        } else {
+          const double sc = d < 1.0 ? 0x1p270 : 0x1p-270;
+          pinv = 1.0 / (d * sc * sc);
+          t = aij * sc * pinv * sc;
+          if (lane == 0) {
+            sc_s[8 * p + j] = sc;
+            scaled = 1;
+          }
+        }
         if (j < 3 && q > j) a0 = fma(-t, k0, a0);
         if (j < 7 && q + 4 > j) a1 = fma(-t, k1, a1);
         if (q == (j & 3)) Wd[i * 9 + j] = t;
@@ -378,7 +400,8 @@ __device__ __forceinline__ void potrf_block(int nb, double *A, long long lda, in
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           xr[2 * u] = x[u];
-          W[row * kPotrfW + 2 * u + h] = x[u] * pinv_s[8 * p + 2 * u + h];
+          const int c = 8 * p + 2 * u + h;
+          W[row * kPotrfW + 2 * u + h] = scaled ? x[u] * sc_s[c] * pinv_s[c] * sc_s[c] : x[u] * pinv_s[c];
         }
       }
     }
@@ -733,6 +756,12 @@ __global__ void reset_info_kernel(int *info) {
   info[1] = GPC_OK;
 }
 
+// Test hook: the pivots' reciprocals.
+__global__ void recip_cubic_probe_kernel(int n, const double *x, double *out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = recip_cubic(x[i]);
+}
+
 unsigned blocks_for(long long total, int threads) { return (unsigned)((total + threads - 1) / threads); }
 
 // Test hook: the refined reciprocals next to CUDA's own 1.0 / x and rsqrt(x).
@@ -959,6 +988,12 @@ cudaError_t lower_to_symmetric_half(int n, double *A, long long lda, cudaStream_
 cudaError_t recip_rsqrt_probe(int n, const double *x, double *out, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 40.0 * n, s, recip_rsqrt_probe_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, x, out));
+  return cudaGetLastError();
+}
+
+cudaError_t recip_cubic_probe(int n, const double *x, double *out, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 16.0 * n, s, recip_cubic_probe_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, x, out));
   return cudaGetLastError();
 }
 

@@ -70,6 +70,13 @@ extern "C" int gpc_test_recip_rsqrt(int n, const double *x, double *out, gpc_str
   return recip_rsqrt_probe(n, x, out, stream) == cudaSuccess ? GPC_OK : GPC_ERR_CUDA;
 }
 
+extern "C" int gpc_test_recip_cubic(int n, const double *x, double *out, gpc_stream_t stream) {
+  if (n < 0) return GPC_ERR_INVALID_ARG;
+  if (n == 0) return GPC_OK;
+  if (!x || !out) return GPC_ERR_INVALID_ARG;
+  return recip_cubic_probe(n, x, out, stream) == cudaSuccess ? GPC_OK : GPC_ERR_CUDA;
+}
+
 extern "C" int gpc_test_split_f64(int n, const double *x, float *hilo, double *back, gpc_stream_t stream) {
   if (n < 0) return GPC_ERR_INVALID_ARG;
   if (n == 0) return GPC_OK;
