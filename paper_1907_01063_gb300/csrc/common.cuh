@@ -375,7 +375,7 @@ struct F64xRow {
   int tri = 0;                    // 1: entries with k < r are zero (not read)
   const int *rexp_sub = nullptr;  // non-null: rexp holds one exponent, row r's is *rexp - rexp_sub[r]
   bool wide = false;              // kF64xWide slices
-  int *over_out = nullptr;        // with rexp_sub: entries of 2^100 and more raise this to the exponent they need
+  int *over_out = nullptr;        // with rexp_sub: raised to *rexp, or to the exponent that entries of 2^100 and more need
   const int *alt = nullptr;       // with rexp_sub: such an exponent: split again with it, or nothing where *rexp covers it
 };
 cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int K, int first, const SliceBuf &out,
@@ -387,12 +387,12 @@ cudaError_t f64x_split(const double *src, long long rs, long long ks, int M, int
 cudaError_t f64x_diag_exps(int n, const double *K, long long ldk, int *rexp, cudaStream_t s);
 cudaError_t f64x_lower_exps(int n, const double *L, long long ldl, int *rexp, int *cexp, cudaStream_t s);
 cudaError_t f64x_block_exp(int nb, const double *A, long long lda, const int *rexp, int *out, cudaStream_t s);
-// C (FP64) -= 2^(ra_i + rb_j) A B^T (with ra_sub: 2^(max(*ra, *ra_alt) - ra_sub_i + rb_j)),
+// C (FP64) -= 2^(ra_i + rb_j) A B^T (with ra_sub: 2^(*ra - ra_sub_i + rb_j)),
 // or with `wide` C = that product on kF64xWide slices; the other arguments as for ozaki_gemm.
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
                       double *partial, int *err, cudaStream_t s, int max_ctas = 0, int kdepth = 0, int max_items = 0,
-                      const int *ra_sub = nullptr, bool wide = false, const int *ra_alt = nullptr);
+                      const int *ra_sub = nullptr, bool wide = false);
 // Slices of the transposes of lower-triangular diagonal blocks (the first of order `first` at src with leading
 // dimension ld0, the others of order 128, `stride` apart from src + off1, with ld): operand row c = column c, scaled
 // by its own largest entry; block ib's kF64xWide slices at out + ib f64x_slice_bytes(128, 1, true), its scale

@@ -102,7 +102,6 @@ struct FxParams {
   const int *ra, *rb;              // scale exponents of the output's rows and columns (null: 0), ...
   int ra_mul;                      // 0: one exponent for all rows, less ra_sub[row]
   const int *ra_sub;
-  const int *ra_alt;               // non-null: that exponent is *ra_alt where this is larger
   int sub_stride;
   int ra_codes, rb_codes;          // ... or row_codes_kernel codes
   const int *nblk;                 // non-null: F64xBatch
@@ -557,12 +556,9 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             row0 + 32 <= p.M && colh + 32 <= p.N && (!p.lower || colh + 31 + p.lower_off <= row0);
         const bool live = !p.flags || row0 >= p.M || colh >= p.N ||
                           p.flags[(size_t)k.b * p.flag_stride + (size_t)(4 * k.tm + q) * p.flag_ld + 2 * k.tn + half];
-        int ea = 0;
-        if (row0 + lane < p.M) {
-          ea = row_exp(p.ra, p.ra_codes, k.b * p.ra_stride + (row0 + lane) * p.ra_mul);
-          if (p.ra_alt && __ldg(p.ra_alt) > __ldg(p.ra)) ea = __ldg(p.ra_alt);
-          if (p.ra_sub) ea -= __ldg(p.ra_sub + k.b * p.sub_stride + row0 + lane);
-        }
+        const int ea = row0 + lane < p.M ? row_exp(p.ra, p.ra_codes, k.b * p.ra_stride + (row0 + lane) * p.ra_mul) -
+                                              (p.ra_sub ? __ldg(p.ra_sub + k.b * p.sub_stride + row0 + lane) : 0)
+                                        : 0;
         const int ebl = colh + lane < p.N ? row_exp(p.rb, p.rb_codes, k.b * p.rb_stride + colh + lane) : 0;
         if (p.sub == 4 || p.chunks == 1) {
           // 8 columns of each warp's 32 at a time.  With few tiles (sub: the
@@ -822,10 +818,10 @@ struct FxOperand {
   int *block_out;        // non-null: largest exponent of all entries, each plus row_exps[r] and, in the rows from
   int block_rows;        // block_rows on, the entry's kexp; less kBlockMargin
   const int *row_exps;
-  int *over_out;         // non-null (rexp_mul 0): where entries of 2^100 and more were met, the common exponent that
-                         // would put the largest 2^kBlockMargin above the scale
-  const int *alt;        // non-null: such an exponent; the launch does nothing unless it is above *rexp, and splits
-                         // everything again with it otherwise
+  int *over_out;         // non-null (seven slices, rexp_mul 0): takes *rexp, or where entries of 2^100 and more were met
+                         // the common exponent that puts the largest 2^kBlockMargin above the scale
+  const int *alt;        // non-null (the same): such an exponent; the launch does nothing unless it is above *rexp, and
+                         // splits everything again with it otherwise
   int *counts;           // per row: entries of at least 2^-5 of the row's scale (null: not counted)
   int rexp_stride, tri, tri_off;
   int vec;               // per batch entry of rexp_sub, row_exps and kexp; block_out has one each
@@ -864,7 +860,8 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
         (o.skip_zero && (c + 1) * FX_CHUNK <= r0))
       return;
   }
-  if (o.alt && __ldg(o.alt) <= __ldg(o.rexp)) return;
+  constexpr bool RESCALES = S == kF64xSlices && !ABS;  // has over_out and alt
+  if (RESCALES && o.alt && __ldg(o.alt) <= __ldg(o.rexp)) return;
   const size_t vec = (size_t)blockIdx.z * o.vec;
   const int klen = (c == 0) ? min(p.first, o.K) : min(FX_CHUNK, o.K - kbeg);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -912,10 +909,10 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
   }
   int E = 0, common = 0;
   if (o.rexp && r < o.M) {
-    E = __ldg(o.alt ? o.alt : o.rexp + (size_t)blockIdx.z * o.rexp_stride + (size_t)r * o.rexp_mul);
+    E = __ldg(RESCALES && o.alt ? o.alt : o.rexp + (size_t)blockIdx.z * o.rexp_stride + (size_t)r * o.rexp_mul);
+    common = E;
     if (p.codes) E = code_exponent(E);
     if (E < kNoExp) E = 0;  // no entry at all
-    common = E;
     if (o.rexp_sub) E -= __ldg(o.rexp_sub + vec + r);
   }
   unsigned long long mant[4];
@@ -938,7 +935,7 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
       ex[i] = kNoExp;
     } else if (e == 2047 || (ex[i] >= 30 && !o.rexp_out)) {
       const bool isnan = e == 2047 && (u << 12) != 0;
-      if (e != 2047 && ex[i] >= 100) over = max(over, ex[i]);
+      if (RESCALES && e != 2047 && ex[i] >= 100) over = max(over, ex[i]);
       if (isnan || (!p.sat && (e == 2047 || ex[i] >= 100))) nan |= 1u << i;
       if (p.sat || nan >> i & 1u) {
         mant[i] = 1ull << 52;
@@ -956,9 +953,10 @@ __global__ void __launch_bounds__(256) f64x_split_kernel(const __grid_constant__
     if (lane == 0 && n > 0) atomicAdd(o.counts + (size_t)blockIdx.z * o.rexp_stride + r, n);
   }
   emax = __reduce_max_sync(0xffffffffu, emax);
-  if (o.over_out) {
+  if (RESCALES && o.over_out) {
     over = __reduce_max_sync(0xffffffffu, over);
-    if (lane == 0 && over > kNoExp) atomicMax(o.over_out, common + over + 1 - kBlockMargin);
+    if (over > kNoExp) common = (common < kNoExp ? 0 : common) + over + 1 - kBlockMargin;
+    if (lane == 0 && r < o.M) atomicMax(o.over_out, common);
   }
   if (o.block_out) {
     raw = __reduce_max_sync(0xffffffffu, raw);
@@ -1244,7 +1242,7 @@ cudaError_t f64x_split_blocks(int nblk, int first, const double *src, long long 
 cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B, int b_row0, int b_k0, int M, int N,
                       int chunks, bool lower, const int *ra, const int *rb, double *C, long long ldc, int splits,
                       double *partial, int *err, cudaStream_t s, int max_ctas, int kdepth, int max_items,
-                      const int *ra_sub, bool wide, const int *ra_alt) {
+                      const int *ra_sub, bool wide) {
   if (M <= 0 || N <= 0 || chunks <= 0) return cudaSuccess;
   if (kdepth <= 0) kdepth = FX_CHUNK;
   if (kdepth > FX_CHUNK || kdepth % FX_BK || (wide && splits > 1)) return cudaErrorInvalidValue;
@@ -1271,7 +1269,6 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
   p.ra = ra;
   p.ra_mul = ra_sub ? 0 : 1;
   p.ra_sub = ra_sub;
-  p.ra_alt = ra_alt;
   p.rb = rb;
   p.C = C;
   p.ldc = ldc;

@@ -47,7 +47,7 @@ struct MixWs {
   void *grp, *tmp;                        // factorisation: two group buffers, per-step temporaries
   void *sx, *si;                          // adjoint, eight slices: panel rows, diagonal-block inverses
   int *rexp, *cexp, *xexp, *iexp, *bexp;  // scale exponents: rows of L, its columns, panel rows, inverses, block column
-  int *oexp;                              // per block column: the exponent its finished block needs, if above bexp
+  int *oexp;                              // per block column: bexp, or what its finished block needs
 };
 constexpr int kMaxDefer = 8;
 // Block columns per deferred update.  The knob belongs to the mixed path: the FP64
@@ -567,8 +567,8 @@ cudaError_t chol_adjoint_mixed(int n, const double *L, long long ldl, double *A,
       int splits = std::max(1, std::min(chunks, (2 * sm_count() + tiles - 1) / tiles));
       while (splits > 1 && ozaki_partial_bytes(nb, j, splits) > kPartialCap) --splits;
       if (f64)
-        TRY(f64x_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, w.bexp, w.cexp, A + (long long)j * lda, lda,
-                      splits, w.scratch, err, s, 0, 0, 0, w.rexp + j, false, w.oexp + ib));
+        TRY(f64x_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, w.oexp + ib, w.cexp, A + (long long)j * lda, lda,
+                      splits, w.scratch, err, s, 0, 0, 0, w.rexp + j));
       else
         TRY(ozaki_gemm(SDC, 0, 0, LT, 0, ib * MB, nb, j, chunks, false, -1.0f, (float2 *)(A + (long long)j * lda),
                        lda, splits, (float2 *)w.scratch, err, s));
