@@ -252,8 +252,15 @@ int gpc_chol_adjoint(int n, const double *L, int ldl, const double *Lbar, int ld
     e = to_df_lower(n, Lbar, ldlb, Kbar, ldkb, stream);
     if (e == cudaSuccess) e = chol_adjoint_mixed(n, L, ldl, Kbar, ldkb, w.core, w.flags, stream);
   } else {
-    e = copy_lower(n, Lbar, ldlb, Kbar, ldkb, stream);
+    // The slices count denormals as zeros; the adjoint is linear in Lbar, so one that lies
+    // near them is taken 2^kTinyShift up and its result down again (two launches that
+    // otherwise end at once).
+    constexpr int kTinyShift = 600;
+    int *emax = w.slices ? (int *)w.vec : nullptr;
+    e = copy_lower(n, Lbar, ldlb, Kbar, ldkb, stream, emax);
+    if (e == cudaSuccess && emax) e = rescale_tiny(n, Kbar, ldkb, kTinyShift, emax, stream);
     if (e == cudaSuccess) e = chol_adjoint_fp64(n, L, ldl, Kbar, ldkb, w.core, w.flags, stream, w.slices);
+    if (e == cudaSuccess && emax) e = rescale_tiny(n, Kbar, ldkb, -kTinyShift, emax, stream);
   }
   if (e == cudaSuccess && symmetric_out) e = lower_to_symmetric_half(n, Kbar, ldkb, stream);
   return status_of(e);

@@ -250,8 +250,11 @@ cudaError_t trtri_sweep(int n, const double *L, long long ldl, int first, int b,
 
 // ---------------------------------------------------------------- elementwise helpers
 // dst(i,j) = src(i,j) for j <= i; strict upper of dst set to 0 (src may == dst).
+// emax (may be null): takes the lower triangle's largest biased exponent.
 cudaError_t copy_lower(int n, const double *src, long long lds, double *dst, long long ldd,
-                       cudaStream_t s);
+                       cudaStream_t s, int *emax = nullptr);
+// The lower triangle times 2^shift where *emax, from copy_lower, says that all of it is below 2^-900.
+cudaError_t rescale_tiny(int n, double *A, long long lda, int shift, const int *emax, cudaStream_t s);
 // dst (m x c) = src (m x c).
 cudaError_t copy_rect(int m, int c, const double *src, long long lds, double *dst,
                       long long ldd, cudaStream_t s);

@@ -6,6 +6,8 @@
 // (trtri_cols_kernel; the per-block inverses of Section 3.2).
 #include "common.cuh"
 
+#include <algorithm>
+
 namespace gpc {
 namespace {
 
@@ -716,12 +718,34 @@ trsm_quad_kernel(int m, double *X, long long ldx, const double *T, long long ldt
   }
 }
 
-__global__ void copy_lower_kernel(int n, const double *src, long long lds, double *dst,
-                                  long long ldd) {
+// emax (null, or zero on entry): the largest biased exponent of the lower triangle.
+__global__ void __launch_bounds__(256)
+copy_lower_kernel(int n, const double *src, long long lds, double *dst, long long ldd, int *emax) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)n * n) return;
-  const int i = (int)(idx / n), j = (int)(idx - (long long)i * n);
-  dst[(long long)i * ldd + j] = (j <= i) ? src[(long long)i * lds + j] : 0.0;
+  double v = 0.0;
+  if (idx < (long long)n * n) {
+    const int i = (int)(idx / n), j = (int)(idx - (long long)i * n);
+    if (j <= i) v = src[(long long)i * lds + j];
+    dst[(long long)i * ldd + j] = v;
+  }
+  if (!emax) return;
+  __shared__ int es[8];  // one look at *emax per CTA: one per warp cost 0.2 ms at n = 6007
+  const int e = __reduce_max_sync(0xffffffffu, (__double2hiint(v) >> 20) & 0x7FF);
+  if ((threadIdx.x & 31) == 0) es[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  int m = es[0];
+  for (int w = 1; w < 8; ++w) m = max(m, es[w]);
+  if (m > *(volatile int *)emax) atomicMax(emax, m);
+}
+
+// The lower triangle times 2^shift where *emax is below kTinyExponent; otherwise nothing.
+constexpr int kTinyExponent = 123;  // 2^-900
+__global__ void __launch_bounds__(256)
+rescale_tiny_kernel(int n, double *A, long long lda, int shift, const int *emax) {
+  if (*emax >= kTinyExponent) return;
+  for (int i = blockIdx.x; i < n; i += gridDim.x)
+    for (int j = threadIdx.x; j <= i; j += 256) A[(long long)i * lda + j] = scalbn(A[(long long)i * lda + j], shift);
 }
 
 __global__ void copy_rect_kernel(int m, int c, const double *src, long long lds, double *dst,
@@ -955,11 +979,19 @@ cudaError_t trsm_rows(int m, int nb, double *X, long long ldx, const double *T, 
   return cudaGetLastError();
 }
 
-cudaError_t copy_lower(int n, const double *src, long long lds, double *dst, long long ldd,
-                       cudaStream_t s) {
+cudaError_t copy_lower(int n, const double *src, long long lds, double *dst, long long ldd, cudaStream_t s, int *emax) {
   if (n <= 0) return cudaSuccess;
+  if (emax)
+    if (cudaError_t e = cudaMemsetAsync(emax, 0, sizeof(int), s); e != cudaSuccess) return e;
   GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 8.0 * (double)n * n * 1.5, s,
-             copy_lower_kernel<<<blocks_for((long long)n * n, 256), 256, 0, s>>>(n, src, lds, dst, ldd));
+             copy_lower_kernel<<<blocks_for((long long)n * n, 256), 256, 0, s>>>(n, src, lds, dst, ldd, emax));
+  return cudaGetLastError();
+}
+
+cudaError_t rescale_tiny(int n, double *A, long long lda, int shift, const int *emax, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  GPC_LAUNCH(GPC_TRACE_ELEM, 0.0, 0.0, s,
+             rescale_tiny_kernel<<<std::min(n, 4 * sm_count()), 256, 0, s>>>(n, A, lda, shift, emax));
   return cudaGetLastError();
 }
 

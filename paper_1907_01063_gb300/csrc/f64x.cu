@@ -1302,7 +1302,7 @@ cudaError_t f64x_gemm(const SliceBuf &A, int a_row0, int a_k0, const SliceBuf &B
 namespace {
 
 // e_i with K_ii < 4^e_i (|L_ij| <= sqrt(K_ii) < 2^e_i); 0 where K_ii is no
-// positive normal number (the factorisation fails there).
+// positive number (the factorisation fails there).  The factor of denormals is normal.
 __global__ void diag_exps_kernel(int n, const double *K, long long ldk, int *rexp, const int *nblk, long long stride,
                                  int vec) {
   if (nblk) n = FX_CHUNK * __ldg(nblk + blockIdx.z);
@@ -1311,8 +1311,9 @@ __global__ void diag_exps_kernel(int n, const double *K, long long ldk, int *rex
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const unsigned long long u = (unsigned long long)__double_as_longlong(K[(long long)i * ldk + i]);
-  const int e = (int)(u >> 52);  // the sign bit too: negative entries are above 2047
-  rexp[i] = (e > 0 && e < 2047) ? (e - 1022 + 1) >> 1 : 0;
+  const int b = (int)(u >> 52);                              // the sign bit too: negative entries are above 2047
+  const int e = b > 0 ? b : 12 - __clzll((long long)u);      // goes on below 1 for denormals
+  rexp[i] = (u != 0 && b < 2047) ? (e - 1022 + 1) >> 1 : 0;
 }
 // rexp[i]: exponent E, 2^E above the largest entry of row i of the lower triangle.  A warp per row.
 __global__ void __launch_bounds__(256) lower_row_exps_kernel(int n, const double *L, long long ldl, int *rexp, const int *nblk, long long stride,
