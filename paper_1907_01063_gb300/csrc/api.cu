@@ -70,7 +70,9 @@ ApiWs carve(void *ws, size_t ws_bytes, int n, int precision) {
   ApiWs w;
   w.slices = precision == GPC_FP64 && f64_on_slices(n) && ws_bytes >= full_bytes(n, precision);
   char *p = (char *)ws;
-  w.core = p;
+  // The copies of slices want 16-byte aligned buffers, the FP64 kernels only doubles: a
+  // caller's workspace may start anywhere those can (mixed_workspace_bytes has 1 KB to spare).
+  w.core = w.slices ? (void *)align_up((size_t)p, 256) : p;
   p += core_bytes(n, precision, w.slices);
   w.vec = (double *)p;
   p += align_up(4 * (size_t)std::max(n, 1) * sizeof(double), 256);

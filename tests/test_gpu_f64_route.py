@@ -61,3 +61,32 @@ def test_the_mixed_depth_knob_leaves_fp64_calls_alone(depth):
     finally:
         gp.set_tuning(gp.GPC_TUNE_MIXED_DEFER, old)
     assert any("f64x_gemm" in k for k in names) and torch.equal(L, want)
+
+
+@pytest.mark.parametrize("offset", [8, 16, 40, 248])
+def test_a_workspace_may_start_at_any_double(offset):
+    n = 500
+    K = dev(O.se_cov(W.gp_inputs(n, 3, 8), 1.0, 1.0, 0.3, 1e-6))
+    Wt, y = dev(W.random_lower(n, 9)), dev(W.gp_inputs(n, 1, 10)[:, 0])
+    size = gp.workspace_size(n, "fp64")
+    ws = torch.empty(size + offset, dtype=torch.uint8, device="cuda")[offset:]
+
+    def step(ws):
+        L = gp.chol(K, ws=ws)
+        r = gp.gp_lml(K, y, ws=ws)
+        return L, gp.chol_adjoint(L, Wt, ws=ws), r["alpha"], gp.gp_lml_grad(r["L"], r["alpha"], ws=ws)
+
+    got, names = kernels(lambda: step(ws))
+    assert any("f64x_gemm" in k for k in names)
+    assert all(torch.equal(a, b) for a, b in zip(got, step(None)))
+
+
+def test_matrices_may_start_at_any_double_with_odd_leading_dimensions():
+    n, ld = 450, 463
+    Kh, Wt = O.se_cov(W.gp_inputs(n, 3, 8), 1.0, 1.0, 0.3, 1e-6), W.random_lower(n, 9)
+    Kp, Wp, Lp, Gp = (torch.zeros(n * ld + 1, dtype=torch.float64, device="cuda")[1:].view(n, ld)[:, :n] for _ in range(4))
+    Kp.copy_(dev(Kh))
+    Wp.copy_(dev(Wt))
+    L = gp.chol(Kp, out=Lp)
+    G = gp.chol_adjoint(L, Wp, out=Gp)
+    assert torch.equal(L, gp.chol(dev(Kh))) and torch.equal(G, gp.chol_adjoint(L.contiguous(), dev(Wt)))
