@@ -1547,7 +1547,9 @@ bool choose_panels(const Gemm &g, size_t bytes, Panels &out) {
   for (;;) {
     int kp = kall;
     while (kp > 128 && panel_bytes(mp, np, kp, g.batch) > bytes) kp = (kp / 2 + 127) / 128 * 128;
-    const bool fits = panel_bytes(mp, np, kp, g.batch) <= bytes;
+    // one grid row per 8 operand rows of the split, 65535 at most, however large the workspace
+    const bool fits = panel_bytes(mp, np, kp, g.batch) <= bytes &&
+                      align_up((size_t)mp, 128) + align_up((size_t)np, 128) <= 8 * 65535;
     if (fits && kp >= std::min(kall, 512)) {
       out = {mp, np, kp};
       return true;

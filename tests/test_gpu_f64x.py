@@ -204,3 +204,11 @@ def test_nan_in_the_adjoint_spreads():
     G = gp.chol_adjoint(dev(L), dev(Wt)).cpu().numpy()
     ref = O.chol_adjoint(L, Wt)
     assert np.isnan(G[350, 100]) and np.isnan(ref[350, 100])
+
+
+@pytest.mark.parametrize("m,n", [(530000, 64), (64, 530000)])
+def test_a_large_workspace_does_not_make_panels_too_long(m, n):
+    # more operand rows than one launch of the split covers, in a workspace that holds them all
+    r = np.random.default_rng(m)
+    A, B = r.standard_normal((m, 64)), r.standard_normal((64, n))
+    check(run(A, B, torch.empty(3 << 30, dtype=torch.uint8, device="cuda")), A, B)
