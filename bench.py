@@ -560,9 +560,9 @@ def main():
     tuned = {}
     if not args.no_autotune:
         from paper_1907_01063_gb300 import autotune
-        # FP64 schedule (block size, split-K minimum, small-product tile limit),
-        # timed on chol + adjoint at the workload's order capped at 8192 (one
-        # FP64 pass at 16384 takes seconds); the choice is applied
+        # FP64 schedule: block size and split-K minimum of the FP64 product kernels
+        # at the largest order that always runs on them, small-product tile limit at
+        # the workload's order capped at 8192; the choice is applied
         rec64 = autotune.tune_fp64(min(n, 8192))
         tuned["fp64_block"] = rec64["best"]["fp64_block"]
         tuned["fp64_schedule"] = dict(rec64["best"], timed_at_n=rec64["n"])

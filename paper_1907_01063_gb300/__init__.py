@@ -243,6 +243,14 @@ def workspace_size(n: int, precision="fp64") -> int:
     return b.value
 
 
+def workspace_min_size(n: int, precision="fp64") -> int:
+    """The smallest workspace a call of order n accepts: FP64 calls run on the FP64 product kernels in it."""
+    b = ctypes.c_size_t()
+    _check(capi.gpc_workspace_min_size(int(n), precision_code(precision), ctypes.byref(b)),
+           "gpc_workspace_min_size")
+    return b.value
+
+
 def workspace(n: int, precision="fp64", device=None) -> torch.Tensor:
     """A byte tensor large enough for any call at order <= n."""
     return torch.empty(workspace_size(n, precision), dtype=torch.uint8,
@@ -265,10 +273,9 @@ def check_info(info: torch.Tensor, what: str = "factorisation"):
 def _ws_for(n: int, precision, ws: torch.Tensor | None, device) -> torch.Tensor:
     if ws is None:
         return torch.empty(workspace_size(n, precision), dtype=torch.uint8, device=device)
-    b = ctypes.c_size_t()
-    _check(capi.gpc_workspace_min_size(int(n), precision_code(precision), ctypes.byref(b)), "gpc_workspace_min_size")
-    if ws.numel() * ws.element_size() < b.value or not ws.is_cuda:
-        raise ValueError(f"workspace too small: need {b.value} bytes")
+    need = workspace_min_size(n, precision)
+    if ws.numel() * ws.element_size() < need or not ws.is_cuda:
+        raise ValueError(f"workspace too small: need {need} bytes")
     return ws
 
 

@@ -9,21 +9,24 @@ Offline (``tune_*``: dedicated timing runs, cached) and online
 (``OnlineTuner``: the caller's own repeated calls are the timing runs).
 
 Knobs:
-  * batch_block: block size inside the batched per-GP pass (32 or 64), timed
-    on a batch of GPs with the caller's size mix, separately per precision.
-  * fp64_block: block size of the FP64 blocked factorisation and adjoint
-    (64, 96 or 128), timed on chol + adjoint at a stand-in order.
+  * batch_block: block size inside the persistent launch of a batch (32 or 64),
+    timed on a batch of GPs with the caller's size mix, separately per precision;
+    left alone for batches that run in lockstep, which do not read it.
+  * fp64_block: block size of the blocked factorisation and adjoint on the FP64
+    product kernels (64, 96 or 128), timed on chol + adjoint in the minimal
+    workspace, where every order runs on them.
   * the mixed schedule (tune_mixed): the update depth D -- the tcgen05
     trailing and background products take K = 128 D per read-modify-write of
     their double-float output tiles (D in 1, 2, 4, 6, 8) -- and the SMs the
     background products leave to the FP64 chain in the factorisation (2, 4,
     8) and in the adjoint (8, 16, 24); the slice chunk (the K tile of one
     exponent group) stays 128.
-  * the FP64 schedule (tune_fp64): the block size above together with the
-    minimum K per split of the split-K products (the K tile of a partial
-    product: 32, 64, 128) and the output tile of the FP64 products (single
-    products up to a size limit take 32 x 32 tiles, the rest 64 x 64; the
-    limit is searched over 256, 0 (always 64 x 64), 128 and 512).
+  * the FP64 schedule (tune_fp64): the block size above and the minimum K per
+    split of the split-K products (32, 64, 128), timed on the FP64 product kernels
+    at the largest order that always runs on them (320; above, FP64 calls run on
+    slices), and the output tile of the FP64 products (single products up to a size
+    limit take 32 x 32 tiles, the rest 64 x 64; the limit is searched over 256, 0
+    (always 64 x 64), 128 and 512), timed at the caller's order.
 Schedules with several knobs are searched coordinate by coordinate
 (coordinate_search): each knob in turn over its candidates with the others
 held at their best so far.  Cache keys carry the device, the precision and the
@@ -87,7 +90,14 @@ def _time(fn, reps: int = 2) -> float:
 
 
 def tune_batch_block(batch: "gp.Batch", X, y, hyp, force: bool = False) -> dict:
-    """Pick the batched block size for this batch's size mix and precision; applies it."""
+    """Pick the batched block size for this batch's size mix and precision; applies it.
+
+    A batch that runs in lockstep (more than the two launches of the persistent
+    way) does not read the knob: it stays as it is, and nothing is stored."""
+    before = gp.launch_count()
+    gp.batched_gp_lml_grad(batch, X, y, hyp)
+    if gp.launch_count() - before > 2:
+        return {"best": gp.get_tuning(gp.GPC_TUNE_BATCH_BLOCK), "ms": {}, "lockstep": True}
     key = f"{_device_key()}/batch/{batch.precision}/{batch.batch}x{batch.nmax}/sum{batch.total_rows}"
     db = _load()
     if key in db and not force:
@@ -105,27 +115,33 @@ def tune_batch_block(batch: "gp.Batch", X, y, hyp, force: bool = False) -> dict:
     return rec
 
 
-def tune_fp64_block(n: int = 4096, force: bool = False) -> dict:
-    """Pick the FP64 factorisation block size (timed on chol + adjoint at order n); applies it."""
-    key = f"{_device_key()}/fp64_block/{n}"
-    db = _load()
-    if key in db and not force:
-        gp.set_tuning(gp.GPC_TUNE_BLOCK, db[key]["best"])
-        return db[key]
+def _kernels_pass(n: int):
+    """chol + adjoint of order n on the FP64 product kernels (minimal workspace), as a function to time."""
     L0 = W.known_factor(n, seed=0)
     Ld = torch.as_tensor(L0, device="cuda")
     K = Ld @ Ld.T
     Lbar = torch.as_tensor(W.random_lower(n, seed=1), device="cuda")
+    L, Kbar = torch.empty_like(K), torch.empty_like(K)
+
+    def run():  # the size depends on the knobs
+        ws = torch.empty(gp.workspace_min_size(n, "fp64"), dtype=torch.uint8, device="cuda")
+        gp.chol(K, out=L, ws=ws, check=False)
+        gp.chol_adjoint(L, Lbar, out=Kbar, ws=ws)
+
+    return run
+
+
+def tune_fp64_block(n: int = 4096, force: bool = False) -> dict:
+    """Pick the block size of the FP64 product kernels (timed on chol + adjoint at order n); applies it."""
+    key = f"{_device_key()}/fp64_kernels_block/{n}"
+    db = _load()
+    if key in db and not force:
+        gp.set_tuning(gp.GPC_TUNE_BLOCK, db[key]["best"])
+        return db[key]
+    run = _kernels_pass(n)
     times = {}
     for b in (64, 96, 128):
         gp.set_tuning(gp.GPC_TUNE_BLOCK, b)
-        ws = gp.workspace(n, "fp64")
-        L = torch.empty_like(K)
-
-        def run():
-            gp.chol(K, out=L, ws=ws, check=False)
-            gp.chol_adjoint(L, Lbar, ws=ws)
-
         times[b] = _time(run, reps=1 if n >= 8192 else 2)  # one FP64 pass at n = 16384 is seconds
     best = min(times, key=times.get)
     gp.set_tuning(gp.GPC_TUNE_BLOCK, best)
@@ -172,8 +188,9 @@ def coordinate_search(knobs, measure, start=None) -> dict:
 
 _MIXED_KNOBS = [("mixed_defer", (6, 1, 2, 4, 8)), ("mixed_free_sms", (2, 4, 8)),
                 ("mixed_adj_free_sms", (16, 8, 24))]
-_FP64_KNOBS = [("fp64_block", (128, 64, 96)), ("splitk_min", (32, 64, 128)),
-               ("f64_small_tile", (256, 0, 128, 512))]
+_KERNEL_KNOBS = [("fp64_block", (128, 64, 96)), ("splitk_min", (32, 64, 128))]
+_KERNEL_ORDER = 320  # the largest order whose FP64 calls run on the FP64 product kernels in any workspace
+_TILE_KNOBS = [("f64_small_tile", (256, 0, 128, 512))]
 _KNOB_IDS = {"mixed_defer": gp.GPC_TUNE_MIXED_DEFER, "mixed_free_sms": gp.GPC_TUNE_MIXED_FREE_SMS,
              "mixed_adj_free_sms": gp.GPC_TUNE_MIXED_ADJ_FREE_SMS, "fp64_block": gp.GPC_TUNE_BLOCK,
              "splitk_min": gp.GPC_TUNE_SPLITK_MIN, "f64_small_tile": gp.GPC_TUNE_F64_SMALL_TILE}
@@ -237,9 +254,42 @@ def tune_mixed(n: int = 16384, force: bool = False) -> dict:
 
 
 def tune_fp64(n: int = 4096, force: bool = False) -> dict:
-    """Tune the FP64 schedule (block size, split-K minimum K per split) on
-    chol + adjoint at n_bucket(n); applies the result."""
-    return _tune_schedule("fp64", "fp64", _FP64_KNOBS, n, force)
+    """Tune the FP64 schedule (block size and split-K minimum of the FP64 product
+    kernels, output tile of the FP64 products) on chol + adjoint; applies the result."""
+    nb = n_bucket(n)
+    key = f"{_device_key()}/fp64_schedule/{nb}"
+    db = _load()
+    if key in db and not force:
+        _apply(db[key]["best"])
+        return db[key]
+    knobs = _KERNEL_KNOBS + _TILE_KNOBS
+    saved = {name: gp.get_tuning(_KNOB_IDS[name]) for name, _ in knobs}
+    kernels = _kernels_pass(_KERNEL_ORDER)
+    K, Lbar = _chol_adjoint_stand_in(nb)
+    L, Kbar, ws = torch.empty_like(K), torch.empty_like(K), gp.workspace(nb, "fp64")
+
+    def own():
+        gp.chol(K, out=L, ws=ws, check=False)
+        gp.chol_adjoint(L, Lbar, out=Kbar, ws=ws)
+
+    def timed(run, reps):
+        def measure(cfg):
+            _apply(cfg)
+            return _time(run, reps)
+        return measure
+
+    try:
+        res = coordinate_search(_KERNEL_KNOBS, timed(kernels, 10), start={k: saved[k] for k, _ in _KERNEL_KNOBS})
+        _apply(res["best"])
+        tile = coordinate_search(_TILE_KNOBS, timed(own, 3), start={k: saved[k] for k, _ in _TILE_KNOBS})
+    finally:
+        _apply(saved)
+    best = dict(res["best"], **tile["best"])
+    _apply(best)
+    rec = {"best": best, "ms": dict(res["ms"], **tile["ms"]), "n": nb, "kernels_n": _KERNEL_ORDER, "when": time.time()}
+    db[key] = rec
+    _store(db)
+    return rec
 
 
 class _EventTimer:
@@ -351,10 +401,11 @@ def apply_cached() -> dict:
     for key, rec in db.items():
         if not key.startswith(dev + "/"):
             continue
-        if "/fp64_block/" in key:
+        # records under other names ("fp64_block", "fp64") timed calls that no longer read their knobs
+        if "/fp64_kernels_block/" in key:
             gp.set_tuning(gp.GPC_TUNE_BLOCK, rec["best"])
             applied["fp64_block"] = rec["best"]
-        elif "/mixed/" in key or "/fp64/" in key:
+        elif "/mixed/" in key or "/fp64_schedule/" in key:
             _apply(rec["best"])
             applied.update(rec["best"])
     return applied
