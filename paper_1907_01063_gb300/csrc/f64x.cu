@@ -93,7 +93,7 @@ __device__ __forceinline__ bool code_bad(int code) {
 struct FxParams {
   int M, N, chunks, qpc, kstages;  // qpc: stages per chunk; kstages: stages in all (0: chunks * qpc)
   int a_row0, b_row0, a_k0, b_k0;
-  int lower, lower_off;            // entries with col + lower_off <= row
+  int lower;                       // entries with col <= row
   int kskip, ksh_m, ksh_n;         // known-zero K ranges (Gemm::kskip), shifted by the panel's offsets
   int splits, tiles_m, tiles_n, per_batch, num_work;
   int sub;                         // 4: four CTAs per tile, each with 8 columns of every epilogue warp's 32 (else 1)
@@ -530,7 +530,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int i = 0; i < 32; ++i) {
           const int cb = __shfl_sync(0xffffffffu, code_b, i);
           const int col = colh + i;
-          if (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row) && !k.none) {
+          if (row < p.M && col < p.N && !(p.lower && col > row) && !k.none) {
             if (code_bad(code_a) || code_bad(cb)) bad = true;
             else if (code_a != kCodeZero && cb != kCodeZero && !(s[i] >= p.theta)) bad = true;
           }
@@ -553,7 +553,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         const bool add = p.accumulate && !p.partial;
         const bool interior =
-            row0 + 32 <= p.M && colh + 32 <= p.N && (!p.lower || colh + 31 + p.lower_off <= row0);
+            row0 + 32 <= p.M && colh + 32 <= p.N && (!p.lower || colh + 31 <= row0);
         const bool live = !p.flags || row0 >= p.M || colh >= p.N ||
                           p.flags[(size_t)k.b * p.flag_stride + (size_t)(4 * k.tm + q) * p.flag_ld + 2 * k.tn + half];
         const int ea = row0 + lane < p.M ? row_exp(p.ra, p.ra_codes, k.b * p.ra_stride + (row0 + lane) * p.ra_mul) -
@@ -574,7 +574,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
             for (int it = 0; it < 8; ++it) {
               const int row = row0 + 4 * it + rl;
-              const bool in = interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row));
+              const bool in = interior || (row < p.M && col < p.N && !(p.lower && col > row));
               v[it] = in ? base[(long long)row * ld + col] : 0.0;
             }
           };
@@ -657,7 +657,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int it = 0; it < 8; ++it) {
               const int row = row0 + 4 * it + rl, at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
               const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
-              if (interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row))) {
+              if (interior || (row < p.M && col < p.N && !(p.lower && col > row))) {
                 double *dst = base + (long long)row * ld + col;
                 double x = triple_to_f64(tb[at], tb[at + 256], tb[at + 512], sh);
                 if (off >> it & 1u) x = *dst + x;
@@ -678,7 +678,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
             for (int it = 0; it < 8; ++it) {
               const int row = row0 + 4 * it + rl, col = colh + cg * FX_EPI_COLS + cl;
-              const bool in = interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row));
+              const bool in = interior || (row < p.M && col < p.N && !(p.lower && col > row));
               v[cg][it] = in ? base[(long long)row * ld + col] : 0.0;
             }
 #pragma unroll
@@ -775,7 +775,7 @@ f64x_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           for (int it = 0; it < 8; ++it) {
             const int row = row0 + 4 * it + rl, at = (4 * it + rl) * FX_EPI_COLS + (cl ^ it);
             const int sh = eb + __shfl_sync(0xffffffffu, ea, 4 * it + rl);
-            if (interior || (row < p.M && col < p.N && !(p.lower && col + p.lower_off > row))) {
+            if (interior || (row < p.M && col < p.N && !(p.lower && col > row))) {
               double *dst = base + (long long)row * ld + col;
               double v = triple_to_f64(tb[at], tb[at + 256], tb[at + 512], sh);
               if (late >> (8 * cg + it) & 1u) v = *dst + v;

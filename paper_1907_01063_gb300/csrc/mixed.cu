@@ -42,7 +42,7 @@ constexpr size_t kPartialCap = size_t(40) << 20;
   } while (0)
 
 struct MixWs {
-  double *inv, *m, *t, *panel, *scratch;  // FP64 pieces (scratch doubles as the split-K partials)
+  double *inv, *m, *t, *scratch;          // FP64 pieces (scratch doubles as the split-K partials)
   void *sc, *sdc, *lt;                    // slices: panel rows, block-column columns, L^T
   void *grp, *tmp;                        // factorisation: two group buffers, per-step temporaries
   void *sx, *si;                          // adjoint, eight slices: panel rows, diagonal-block inverses
@@ -175,6 +175,8 @@ int nchunks(int n) { return std::max(1, (n + MB - 1) / MB); }
 size_t sbytes(int rows, int kchunks, bool f64) {
   return f64 ? f64x_slice_bytes(rows, kchunks) : slice_bytes(rows, kchunks);
 }
+// Panel rows of the adjoint; the mixed path's solved half panel has a buffer of its own.
+size_t sc_bytes(int n, bool f64) { return (f64 ? 1 : 2) * sbytes(n, 1, f64); }
 size_t exps_bytes(int n) { return align_up((size_t)n * sizeof(int), 256); }
 
 MixWs carve(void *ws, int n, bool adjoint, bool f64) {
@@ -183,9 +185,8 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
   w.inv = (double *)p; p += (size_t)nchunks(n) * b2();  // every diagonal-block inverse
   w.m = (double *)p; p += b2();
   w.t = (double *)p; p += b2();
-  w.panel = (double *)p; p += align_up((size_t)n * MB * sizeof(double), 256);
   w.scratch = (double *)p; p += scratch_bytes();
-  w.sc = p; p += 2 * sbytes(n, 1, f64);  // two buffers: a panel's rows, and its solved half
+  w.sc = p; p += sc_bytes(n, f64);
   if (adjoint) {
     w.sdc = p; p += sbytes(MB, nchunks(n), f64);
     w.lt = p; p += sbytes(n, nchunks(n), f64);
@@ -211,8 +212,7 @@ MixWs carve(void *ws, int n, bool adjoint, bool f64) {
 
 size_t mixed_workspace_bytes(int n, bool f64) {
   n = std::max(n, 1);
-  size_t common = ((size_t)nchunks(n) + 2) * b2() + align_up((size_t)n * MB * sizeof(double), 256) + scratch_bytes() +
-                  2 * sbytes(n, 1, f64) + 1024;
+  size_t common = ((size_t)nchunks(n) + 2) * b2() + scratch_bytes() + sc_bytes(n, f64) + 1024;
   size_t adj = sbytes(MB, nchunks(n), f64) + sbytes(n, nchunks(n), f64);
   const size_t fwd = 2 * sbytes(n, defer_depth(f64), f64) + sbytes(n, 1, f64);
   if (f64) {
