@@ -60,6 +60,10 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
 
 // Number of SMs of the current device (cached per device).
 int sm_count();
+// Lets a kernel whose shared memory varies from call to call take all that the
+// device has, once per device.  (The limit is process-wide: set to each call's own
+// size, a smaller call of another thread could lower it before the launch.)
+cudaError_t allow_all_smem(const void *fn, bool (&done)[64]);
 
 // ---------------------------------------------------------------- double-float conversions
 // On this part the FP64 pipe (which also runs the FP32 <-> FP64 conversion

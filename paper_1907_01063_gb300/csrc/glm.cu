@@ -453,8 +453,8 @@ cudaError_t glm_launch(GlmParams &p, long long n, int k, double *lp, double *dal
   p.part_s = (double *)(w + align_up((size_t)max_ctas(k) * (size_t)std::max(k, 1) * sizeof(double), 256));
   const size_t smem = narrow ? narrow_smem_bytes(p.R, k, p.family == kFamilyOrdinal) : smem_bytes(k);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(narrow ? glm_narrow_kernel : glm_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static bool done[2][64] = {};
+    cudaError_t e = allow_all_smem(narrow ? (const void *)glm_narrow_kernel : (const void *)glm_kernel, done[narrow]);
     if (e != cudaSuccess) return e;
   }
   const double bytes = 8.0 * ((double)n * k + 2.0 * n + k);

@@ -216,7 +216,8 @@ cudaError_t glm_categorical(long long n, int k, int C, const double *X, long lon
   p.part_s = (double *)(w + align_up((size_t)cat_max_ctas(k, C) * (size_t)std::max(kc, 1) * sizeof(double), 256));
   const size_t smem = cat_smem_bytes(k, C);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(glm_cat_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static bool done[64] = {};
+    cudaError_t e = allow_all_smem((const void *)glm_cat_kernel, done);
     if (e != cudaSuccess) return e;
   }
   GPC_LAUNCH(GPC_TRACE_GLM, 4.0 * (double)n * kc, 8.0 * ((double)n * k + 2.0 * n + 2.0 * kc), s,

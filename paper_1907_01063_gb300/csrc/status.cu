@@ -81,6 +81,20 @@ int launch_priority() { return t_launch_priority; }
 PriorityScope::PriorityScope(int p) : saved(t_launch_priority) { t_launch_priority = p; }
 PriorityScope::~PriorityScope() { t_launch_priority = saved; }
 
+cudaError_t allow_all_smem(const void *fn, bool (&done)[64]) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (done[dev]) return cudaSuccess;
+  cudaFuncAttributes a;
+  if ((e = cudaFuncGetAttributes(&a, fn)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+  if (e == cudaSuccess) done[dev] = true;
+  return e;
+}
+
 int greatest_priority() {
   static int cached[SymbolCache::kMaxDevices];
   static bool have[SymbolCache::kMaxDevices];
