@@ -22,6 +22,9 @@
  *    (ws, ws_bytes) sized by gpc_workspace_size().  Workspace contents are
  *    undefined on return; two calls in flight at the same time need two
  *    workspaces.
+ *  - Calls may come from several host threads at once, each on its own stream
+ *    with its own workspace and outputs (gpc_set_tuning, the trace calls and
+ *    gpc_trsv_noalloc as their comments say).
  *  - Every call is asynchronous on `stream` (a cudaStream_t; NULL = the
  *    legacy default stream) and returns a host status code once its kernels
  *    are enqueued.  Conditions found on the device (a failing pivot, NaN
@@ -53,7 +56,7 @@ typedef struct CUstream_st *gpc_stream_t;
 #define GPC_ERR_NO_CONVERGENCE 6 /* iterative refinement did not reach its tolerance */
 
 /* Arithmetic of the O(n^3) products. */
-#define GPC_FP64 0   /* every step in FP64 (DMMA tensor-core and FP64 ALU) */
+#define GPC_FP64 0   /* every step at FP64 accuracy (larger products on BF16 slices, see gpc_workspace_size) */
 #define GPC_MIXED 1  /* trailing/adjoint products as error-free split BF16 slices on tcgen05 */
 
 /*
@@ -108,7 +111,8 @@ int gpc_workspace_min_size(int n, int precision, size_t *bytes);
 /*
  * Tuning knobs (host-side, process-wide; not thread-safe against concurrent
  * calls).  key: GPC_TUNE_BLOCK = block size b of the blocked factorisation and
- * adjoint (16..128, multiple of 16; default 128), GPC_TUNE_SLICES = number of
+ * adjoint on the FP64 product kernels (16..128, multiple of 16; default 128; calls
+ * on slices always work on 128), GPC_TUNE_SLICES = number of
  * BF16 slices of the mixed path (read-only: the split kernels group their
  * products for 5 slices, so only 5 is accepted), GPC_TUNE_SPLITK_MIN = minimum K per
  * split of the split-K products.  Changing GPC_TUNE_BLOCK changes the
@@ -296,8 +300,9 @@ int gpc_tri_solve_adjoint_ws(int n, int m, const double *Linv, int ldi, const do
  * General matrix product C = A B (Section 3.1, primitive function) at FP64
  * accuracy.  A: m x k (lda >= k), B: k x n (ldb >= n), C: m x n (ldc >= n),
  * all row-major device arrays; C must not overlap A or B.  ws/ws_bytes: NULL/0,
- * or at least 40 MiB (gpc_gemm_workspace_size() gives a size for any product,
- * gpc_gemm_scratch_size() the one of a given product, 0 where none is used).
+ * or at least 40 MiB (gpc_gemm_workspace_size() gives a size for any product, in
+ * which a large one takes several passes; gpc_gemm_scratch_size() the one in which a
+ * given product takes as few as 1 GB allows, 0 where none is used).
  * With a workspace a large product runs on BF16 slices of its operands on the
  * tensor cores, to at least the accuracy of the FP64 chain (output blocks for
  * which that cannot be shown are computed in FP64), and a product whose output

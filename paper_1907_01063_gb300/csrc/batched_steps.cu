@@ -18,10 +18,10 @@
 // read it for the gradient and puts the factor there.  Members are taken in order
 // of size, largest first, in passes of as many as the workspace holds.
 //
-// 512 GPs of orders 64 .. 1024: 200 ms one CTA per GP, 43 ms here: 18 ms products
+// 512 GPs of orders 64 .. 1024: 200 ms one CTA per GP, 42 ms here: 18 ms products
 // (195 launches; few 128-deep chunks per output tile, so their epilogues' instructions
-// bound them), 9 ms splits (3 TB/s), 5 ms covariance and 7 ms diagonal blocks (FP64
-// units), 2 ms gradient.  96 of orders 32 .. 512: 12.6 -> 3.8 ms.  Accuracy: the
+// bound them), 8 ms splits (3 TB/s), 5 ms covariance and 7 ms diagonal blocks (FP64
+// units), 2 ms gradient.  96 of orders 32 .. 512: 12.6 -> 3.7 ms.  Accuracy: the
 // likelihood's error against 64 bits is that of the kernel it replaces (5.9e-13).
 #include "common.cuh"
 
