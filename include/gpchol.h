@@ -465,7 +465,9 @@ int gpc_se_hyper_grad_workspace_size(int n, size_t *bytes);
  *   hyp[3i..]  (alpha, rho, sigma) of GP i
  *   value[i], grad3[3i..3i+2], info[2i..2i+1]  outputs per GP (info as for
  *              gpc_chol; a GP whose factorisation fails gets NaN outputs)
- * nmax: host int, at most 4096; workspace from gpc_batched_workspace_size
+ * nmax: host int, at most 4096, best the largest order itself: the way is chosen
+ * from it, and block steps past every member's order cost their launches.
+ * Workspace from gpc_batched_workspace_size
  * for the same precision.  The persistent launch needs, per SM, room for Kbar, the
  * kernel values, the diagonal-block inverses and three vectors of order nmax; the
  * mixed path adds BF16 slice buffers of about 10 nmax^2 bytes.  The lockstep way
